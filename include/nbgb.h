@@ -184,7 +184,9 @@ const double *nb_image_device_ptr(const nb_sim *sim);
  * *evaluated_terms = the steps whose term was evaluated (NB_MIXED and
  * NB_F32 skip Gaussian terms whose F_latt^2 / (Na Nb Nc)^2 = exp(-2 sum
  * N^2 f^2 / 0.63) lies below exp(-88) < FLT_MIN, i.e. terms that vanish in
- * FP32; NB_F64 evaluates every step and reports 0 here).  Blocks until the
+ * FP32; NB_F64 reports 0 here: it accounts for every step, and leaves out
+ * only Gaussian terms that together are below 2^-56 of their pixel's sum, an
+ * eighth of one rounding).  Blocks until the
  * launch is done.  Errors: NB_EINVAL for NULL outputs. */
 int nb_get_stats(nb_sim *sim, long long *evaluated_terms,
                  long long *pixel_steps);
@@ -218,7 +220,9 @@ int nb_set_fcell_device(nb_sim *sim, const float *F, size_t n_elems);
  *                        against the Gaussian cut (every step for the
  *                        thread-per-pixel and FP64 kernels)
  *   NB_WORK_TERMS        steps whose term was evaluated (as nb_get_stats;
- *                        every step for NB_F64)
+ *                        every step for NB_F64, those included whose
+ *                        terms were shown to be below a rounding of the
+ *                        pixel's sum)
  * The warp kernel counts pairs, intervals and blocks only in launches made
  * with the option NB_OPT_COUNT_WORK set (a separate instantiation, so that
  * the counting costs the other launches nothing); otherwise those three

@@ -113,6 +113,7 @@ struct nb_sim {
   double daxes[6][9];  // d(lab axes)/d(tx, ty, tz, a, b, c)
   DevBuf d_dax, d_part, d_grad, d_F4, d_C4, d_F64t;
   bool F4_valid = false, C4_valid = false, F64_valid = false;
+  bool fmax_valid = false;  // the largest |F|, behind the counters
   int has_div = 0;
   double u0 = 0;
   bool tables_dirty = true;
@@ -702,6 +703,7 @@ int nb_set_crystal(nb_sim *s, const double axes[9], const double *umats,
     s->F4_valid = false;
     s->C4_valid = false;
     s->F64_valid = false;
+    s->fmax_valid = false;
   } else {
     if (interp == NB_INTERP_NEAREST || interp == NB_INTERP_TRICUBIC)
       s->interp = interp;
@@ -729,6 +731,7 @@ int nb_set_fcell_device(nb_sim *s, const float *F, size_t n_elems) {
   s->F4_valid = false;
   s->C4_valid = false;
   s->F64_valid = false;
+  s->fmax_valid = false;
   return NB_OK;
 }
 
@@ -935,6 +938,35 @@ static void ensure_cell_polynomials(nb_sim *s) {
     s->C4_valid = true;
 }
 
+// The bound that lets the FP64 warp kernel screen out negligible steps of a
+// Gaussian shape: the largest |F| (behind the counters in d_stats) and the
+// shot's constant.  Left unset, so that every step is evaluated, where a
+// weight is negative (the sum so far would not bound the sum) or default_F
+// is not finite.
+static cudaError_t screen_setup(nb_sim *s, SpotArgs &a) {
+  if (a.shape != NB_SHAPE_GAUSS || !std::isfinite(s->defF))
+    return cudaSuccess;
+  double W = 0.0;
+  for (double w : s->w) {
+    if (w < 0.0) return cudaSuccess;
+    W += w;
+  }
+  const double nn = s->N[0] * s->N[1] * s->N[2];
+  const double kb = 2.0 * std::log2(nn) + std::log2(W) + 56.0 +
+                    std::log2((double)a.os * a.os * a.T * a.PM);
+  if (!std::isfinite(kb)) return cudaSuccess;
+  float *fmax = (float *)((unsigned long long *)s->d_stats.p + 5);
+  if (!s->fmax_valid) {
+    cudaError_t e = nbgb::build_fmax(
+        a.F, (long long)a.hn[0] * a.hn[1] * a.hn[2], fmax, s->stream);
+    if (e != cudaSuccess) return e;
+    s->fmax_valid = true;
+  }
+  a.fmax = fmax;
+  a.screen_kb = (float)kb;
+  return cudaSuccess;
+}
+
 static int launch(nb_sim *s, const long long *dev_list, long long n_list) {
   if (!s->have_crystal || !s->have_beam || !s->have_det || !s->have_F)
     return fail(s, NB_ESTATE, "crystal, beam and detector must be set first");
@@ -963,10 +995,11 @@ static int launch(nb_sim *s, const long long *dev_list, long long n_list) {
     a.sinc_qG = 0.f;
   }
   // counters: [0] evaluated terms, [1..3] the warp kernel's pairs,
-  // intervals and source blocks
-  cudaError_t e = s->d_stats.ensure(4 * sizeof(unsigned long long));
+  // intervals and source blocks, [4] the next pixel of the FP64 warp
+  // kernel; behind them the largest |F|
+  cudaError_t e = s->d_stats.ensure(6 * sizeof(unsigned long long));
   if (e != cudaSuccess) return fail(s, NB_ENOMEM, "statistics counters");
-  e = cudaMemsetAsync(s->d_stats.p, 0, 4 * sizeof(unsigned long long),
+  e = cudaMemsetAsync(s->d_stats.p, 0, 5 * sizeof(unsigned long long),
                       s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "statistics reset");
   a.stats = (unsigned long long *)s->d_stats.p;
@@ -986,7 +1019,12 @@ static int launch(nb_sim *s, const long long *dev_list, long long n_list) {
   s->last_warp = warp_variant && s->precision != NB_F64;
   s->last_counted = s->count_work;
   if (s->precision == NB_F64) {
-    e = nbgb::launch_spots_f64(a, s->stream);
+    if ((e = screen_setup(s, a)) != cudaSuccess)
+      return cuda_fail(s, e, "structure-factor bound");
+    e = nbgb::f64_warp_supported(a)
+            ? nbgb::launch_spots_f64_warp(a, a.stats + 4, s->sm_count,
+                                          s->stream)
+            : nbgb::launch_spots_f64(a, s->stream);
   } else if (warp_variant) {
     ensure_cell_polynomials(s);
     a.C4 = s->C4_valid ? (const float4 *)s->d_C4.p : nullptr;

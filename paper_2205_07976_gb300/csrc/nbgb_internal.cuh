@@ -169,6 +169,11 @@ struct SpotArgs {
   // intervals solved, [2] source blocks tested; null to skip counting (the
   // kernel is then instantiated without the counters)
   unsigned long long *wstats;
+  // NB_F64, Gaussian shapes: screening of negligible steps
+  // (spots_f64_warp_kernel): the largest |F| of the table, and
+  // log2((Na Nb Nc)^2 U PM sum|w| 2^56), U = os^2 T
+  const float *fmax;
+  float screen_kb;
   // NB_CHECK builds: the word a failed bounds check writes (null: none)
   unsigned long long *check;
 };
@@ -356,6 +361,11 @@ void rotated_axes_table(const double *lab, const double *umats, int n_mosaic,
                         const double *spindle, std::vector<double> &ax);
 
 cudaError_t launch_spots_f64(const SpotArgs &a, cudaStream_t st);
+bool f64_warp_supported(const SpotArgs &a);
+cudaError_t launch_spots_f64_warp(const SpotArgs &a, unsigned long long *work,
+                                  int sm_count, cudaStream_t st);
+cudaError_t build_fmax(const float *F, long long n, float *fmax,
+                       cudaStream_t st);
 cudaError_t build_f64_table(const float *F, long long n, double *F64t,
                             cudaStream_t st);
 cudaError_t build_sliding_table(const float *F, const int hn[3], float4 *F4,
