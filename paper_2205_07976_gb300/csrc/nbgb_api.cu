@@ -1321,14 +1321,90 @@ int nb_add_background(nb_sim *s) {
     }
     double ep[3], bp[3];
     pol_basis(dk, s->evec, ep, bp);
-    for (int c = 0; c < 3; ++c) grp.push_back(dk[c]);
-    for (int c = 0; c < 3; ++c) grp.push_back(ep[c]);
-    for (int c = 0; c < 3; ++c) grp.push_back(bp[c]);
+    for (const double *v : {dk, (const double *)ep, (const double *)bp})
+      for (int c = 0; c < 4; ++c) grp.push_back(c < 3 ? v[c] : 0.0);
     rng.push_back(first);
     rng.push_back((int)order.size() - first);
+    rng.push_back(-1);
+    rng.push_back(0);
   }
-  const int G = (int)rng.size() / 2;
+  const int G = (int)rng.size() / 4;
   const bool f64 = s->precision == NB_F64;
+  // the nodes of each group without negative weights, in the layout of
+  // bg_group_sum; two runs are joined by their means and variance sums
+  struct Node {
+    double ubar = 0, W = 0, V = 0;
+    int n = 0;
+    void join(const Node &o) {  // o after this
+      const double w = W + o.W, d = o.ubar - ubar;
+      if (w > 0.0) {
+        V += o.V + d * d * (W * o.W / w);
+        ubar += d * (o.W / w);
+      } else {
+        ubar = (ubar * n + o.ubar * o.n) / (n + o.n);
+      }
+      W = w;
+      n += o.n;
+    }
+  };
+  std::vector<double> nodes;
+  for (int g = 0; g < G; ++g) {
+    const int first = rng[4 * g], cnt = rng[4 * g + 1];
+    bool ok = true;
+    std::vector<Node> leaf(cnt);
+    for (int i = 0; i < cnt; ++i) {
+      const int k = order[first + i];
+      leaf[i].ubar = 1.0 / s->lam[k];
+      leaf[i].W = s->w[k];
+      leaf[i].n = 1;
+      ok = ok && s->w[k] >= 0.0;
+    }
+    const double span = leaf[cnt - 1].ubar - leaf[0].ubar;
+    grp[12 * g + 3] = span > 0.0 ? (cnt - 1) / span : 0.0;
+    if (!ok) continue;
+    rng[4 * g + 2] = (int)nodes.size() / 4;
+    std::vector<Node> t(4 * (size_t)cnt);
+    t[cnt - 1] = leaf[cnt - 1];
+    for (int i = cnt - 2; i >= 0; --i) {  // suffixes
+      t[i] = leaf[i];
+      t[i].join(t[i + 1]);
+    }
+    for (int i = 0; i < cnt; ++i) {  // prefixes
+      t[cnt + i] = i ? t[cnt + i - 1] : leaf[0];
+      if (i) t[cnt + i].join(leaf[i]);
+    }
+    for (int len = 1; len <= cnt; len *= 2)  // aligned runs
+      for (int i = 0; i + len <= cnt; i += len) {
+        Node &o = t[2 * cnt + 2 * i + len - 1];
+        if (len == 1) {
+          o = leaf[i];
+        } else {
+          o = t[2 * cnt + 2 * i + len / 2 - 1];
+          o.join(t[2 * cnt + 2 * i + len + len / 2 - 1]);
+        }
+      }
+    for (const Node &o : t) {
+      const double lo = f64 ? 0.0 : o.ubar - (double)(float)o.ubar;
+      const double v[4] = {o.ubar, lo, o.W, o.V};
+      nodes.insert(nodes.end(), v, v + 4);
+    }
+  }
+  nbgb::BgArgs b;
+  std::memset(&b, 0, sizeof b);
+  b.n_knots = n;
+  b.n_groups = G;
+  b.geo.S = S;
+  if (nbgb::background_smem_bytes(b, f64) > 200 * 1024)
+    return fail(s, NB_EINVAL,
+                "background tables exceed 200 KB of shared memory");
+  // with many sources and knots the nodes may not fit as well: every source
+  // is then visited
+  b.n_nodes = (int)nodes.size() / 4;
+  if (nbgb::background_smem_bytes(b, f64) > 200 * 1024) {
+    b.n_nodes = 0;
+    nodes.clear();
+    for (int g = 0; g < G; ++g) rng[4 * g + 2] = -1;
+  }
   // one double blob: groups, then (F64) knots and sources; one float blob
   std::vector<double> b64(grp);
   std::vector<float> b32;
@@ -1341,6 +1417,7 @@ int nb_add_background(nb_sim *s) {
       b64.push_back(1.0 / s->lam[k]);
       b64.push_back(s->w[k]);
     }
+    b64.insert(b64.end(), nodes.begin(), nodes.end());
   } else {
     for (int j = 0; j < n; ++j) {
       double slope = j + 1 < n ? (s->bg_F[j + 1] - s->bg_F[j]) /
@@ -1354,6 +1431,7 @@ int nb_add_background(nb_sim *s) {
       b32.push_back((float)(1.0 / s->lam[k]));
       b32.push_back((float)s->w[k]);
     }
+    for (double v : nodes) b32.push_back((float)v);
   }
   cudaError_t e;
   if ((e = s->d_bg64.ensure(b64.size() * 8)) != cudaSuccess ||
@@ -1368,8 +1446,6 @@ int nb_add_background(nb_sim *s) {
                     cudaMemcpyHostToDevice, s->stream);
   cudaMemcpyAsync(s->d_bgrng.p, rng.data(), rng.size() * sizeof(int),
                   cudaMemcpyHostToDevice, s->stream);
-  nbgb::BgArgs b;
-  std::memset(&b, 0, sizeof b);
   SpotArgs &a = b.geo;
   a.check = (unsigned long long *)s->d_check.p;  // NB_CHECK builds only
   a.panels = (const DevPanel *)s->d_panels.p;
@@ -1384,21 +1460,18 @@ int nb_add_background(nb_sim *s) {
   a.S = S;
   a.kahn64 = s->kahn;
   a.image = (double *)s->d_image.p;
-  b.n_knots = n;
-  b.n_groups = G;
   const double *d64 = (const double *)s->d_bg64.p;
   b.grp64 = d64;
-  b.knots64 = d64 + 9 * G;
-  b.src64 = d64 + 9 * G + 2 * n;
+  b.knots64 = d64 + 12 * G;
+  b.src64 = b.knots64 + 2 * n;
+  b.nodes64 = b.src64 + 2 * S;
   b.knots32 = (const float *)s->d_bg32.p;
   b.src32 = b.knots32 + 3 * n;
+  b.nodes32 = b.src32 + 2 * S;
   b.grp_range = (const int *)s->d_bgrng.p;
   b.prefactor = nbgb::kElectronRadius * nbgb::kElectronRadius * s->fluence *
                 s->bg_nmol / ((double)s->os * s->os);
-  if (nbgb::background_smem_bytes(b, f64) > 200 * 1024)
-    return fail(s, NB_EINVAL,
-                "background tables exceed 200 KB of shared memory");
-  e = nbgb::launch_background(b, f64, s->stream);
+  e = nbgb::launch_background(b, f64, s->sm_count, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "background launch");
   // the pageable copies above are staged before the launch returns
   return read_check(s);

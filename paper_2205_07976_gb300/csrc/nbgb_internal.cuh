@@ -95,6 +95,7 @@ struct DevPanel {
   // the same vectors as double-float pairs (hi, lo) for the FP32 kernels'
   // geometry (panel_ff fills them)
   float ffo[3][2], fff[3][2], ffs[3][2], ffn[3][2], ffpx[2];
+  float fpx[3][2], spx[3][2];  // px fdir, px sdir
   long long pix0;  // global index of pixel (0, 0)
   int nfast, nslow;
   int tile0;       // first tile of this panel in the tiled launch
@@ -210,6 +211,8 @@ inline void panel_ff(DevPanel &d) {
     split_ff_host(d.fdir[c], d.fff[c]);
     split_ff_host(d.sdir[c], d.ffs[c]);
     split_ff_host(d.ndir[c], d.ffn[c]);
+    split_ff_host(d.px * d.fdir[c], d.fpx[c]);
+    split_ff_host(d.px * d.sdir[c], d.spx[c]);
   }
   split_ff_host(d.px, d.ffpx);
 }
@@ -399,14 +402,21 @@ struct BgArgs {
   int n_knots, n_groups;
   const double *knots64;  // [n][2] stol, F
   const float *knots32;   // [n][3] stol, F, slope to the next knot
-  const double *grp64;    // [G][9] direction, E', B'
-  const int *grp_range;   // [G][2] first source, count
+  const double *grp64;    // [G][12] direction, sources per 1/lambda, E', B'
+  const int *grp_range;   // [G][4] first source, count, first node or -1
+  // nodes [n_nodes][4]: mean 1/lambda (and its rest in FP32), sum of weights
+  // and variance sum of the suffixes, prefixes and aligned runs of each group
+  // (bg_group_sum), 4 times its sources
+  int n_nodes;
+  const double *nodes64;
+  const float *nodes32;
   const double *src64;    // [S][2] 1/lambda, w (grouped order)
   const float *src32;     // [S][2]
   double prefactor;       // r_e^2 fluence n_mol / os^2
 };
 constexpr int kMaxKnots = 4096;
 size_t background_smem_bytes(const BgArgs &b, bool f64);
-cudaError_t launch_background(const BgArgs &b, bool f64, cudaStream_t st);
+cudaError_t launch_background(const BgArgs &b, bool f64, int sm_count,
+                              cudaStream_t st);
 
 }  // namespace nbgb
