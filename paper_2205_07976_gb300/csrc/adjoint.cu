@@ -18,28 +18,49 @@
 // derivative of the Lagrange weights) and dL/dF is spread over the 64
 // stencil entries with the interpolation weights.  The per-step arithmetic
 // is the FP32-mixed form of the forward kernel (double-float fractional
-// offsets); the ten scalar sums
-// go per thread into FP64, per block into a partial row, and a second
-// kernel adds the rows in a fixed order.
+// offsets).
+//
+// The six derivatives of the axes share one pass.  A step's axes are the lab
+// axes rotated by M = U_m R_phi, and so are their derivatives: dA_x/dθ_r =
+// M (da_x/dθ_r), a_x the lab axis.  With e_x = term · dlog(F_latt^2)/df_x u
+// (and F_cell's part) and v = d − i,
+//   Σ_x e_x (dA_x/dθ_r) · v = Σ_x,c (da_x/dθ_r)_c e_x v'_c,  v' = M^T v,
+// so the kernels sum the nine products Q_xc = e_x v'_c over all steps, and the
+// host contracts them once with the six derivatives of the lab axes.  (Forming
+// the 18 products dA_x · v of every orientation, and 18 FMAs per term, took
+// 54 shared loads and 54 FMAs per orientation.)  The thirteen sums go per
+// thread into FP32, per warp into a butterfly, from there into FP64 and
+// per block or pixel row into a partial row; the rows are added in a fixed
+// order.
 #include "mixed_common.cuh"
 
 namespace nbgb {
 
 struct AdjointArgs {
   SpotArgs a;
-  const float *dax;      // [PM][6][9] d(rotated axes)/d(tx,ty,tz,a,b,c)
+  const float *rot;      // [PM][9] M = U_m R_phi, row-major
   const double *dLdI;    // [npix]
   double *gradF;         // [nh*nk*nl], accumulated into
   double *partials;      // [blocks][kGradN]
-  double kc;             // r_e^2 fluence / (os^2 M Phi)
-  double scale;
+  float kcs;             // r_e^2 fluence scale / (os^2 M Phi)
   // term-ring kernel: rows of 32 pixels handed to warps by a counter;
   // partials holds one row of the ten sums per pixel row
   unsigned long long *rows_next;
   long long n_rows;
 };
 
-constexpr int kGradN = 10;
+// the sums: Q_xc (3 x + c), the three dL/dN and dL/dscale, without the
+// prefactor
+constexpr int kGradN = 13;
+static_assert(kGradN == kAdjointSums, "the host contracts these sums");
+
+// v' = M^T v
+__device__ __forceinline__ void unrotate(const float *M, const float v[3],
+                                         float r[3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    r[c] = fmaf(M[c], v[0], fmaf(M[3 + c], v[1], M[6 + c] * v[2]));
+}
 
 // Value F and gradient (dF/dx, dF/dy, dF/dz) at x in [0, 1)^3 of a cell's
 // tricubic polynomial, its 64 monomial coefficients C[a][b][c] of
@@ -112,6 +133,13 @@ __device__ __forceinline__ void lagrange4_deriv(float x, float w[4]) {
   w[3] = (3.f * x2 - 1.f) * (1.f / 6.f);
 }
 
+// One thread per pixel (nearest lookup, and tricubic lookup in tables too
+// long for the ring kernel below).  Bound by instruction issue: per (pixel,
+// orientation) about 150 for the double-float G and r, 20 per source for the
+// cut test, and the evaluation of the surviving steps with 18 % of them
+// surviving.  64-panel shot (S = 8, 10 domains, nearest): 1316 -> 880 us with
+// the nine products Q in place of 18 per orientation, FP32 sums folded by
+// warp, and each lane taking its own surviving steps.
 template <int HASF, int INTERP>
 __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
     spots_adjoint_kernel(AdjointArgs g) {
@@ -120,15 +148,14 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   float *s_axh = smf;
   float *s_axl = smf + a.PM * 9;
   float *s_src = smf + 2 * a.PM * 9;
-  float *s_dax = s_src + a.S * SRC32_STRIDE;
+  float *s_rot = s_src + a.S * SRC32_STRIDE;
   for (int i = threadIdx.x; i < a.PM * 9; i += blockDim.x) {
     s_axh[i] = a.axh[i];
     s_axl[i] = a.axl[i];
+    s_rot[i] = g.rot[i];
   }
   for (int i = threadIdx.x; i < a.S * SRC32_STRIDE; i += blockDim.x)
     s_src[i] = a.src32[i];
-  for (int i = threadIdx.x; i < a.PM * 54; i += blockDim.x)
-    s_dax[i] = g.dax[i];
   __syncthreads();
   // tricubic dL/dF: the terms of a thread near one lattice point n use
   // stencils starting at n-2 or n-1 along each axis, all inside the 5x5x5
@@ -138,7 +165,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   // atomics than 64 per term.
   // [125][kTileThreads] after the tables (dynamic shared memory)
   float (*s_facc)[kTileThreads] =
-      reinterpret_cast<float (*)[kTileThreads]>(s_dax + a.PM * 54);
+      reinterpret_cast<float (*)[kTileThreads]>(s_rot + a.PM * 9);
   long long near_idx = -1;  // nearest lookup: the entry being summed
   // its run of terms, summed in FP32 (an FP64 instruction per term would
   // cost 64 FP32 ones on this part) and added to the FP64 gradient once
@@ -164,9 +191,9 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   if (INTERP && HASF)
     for (int e = 0; e < 125; ++e) s_facc[e][threadIdx.x] = 0.f;
 
-  double gsum[kGradN];
+  float acc[kGradN];
 #pragma unroll
-  for (int r = 0; r < kGradN; ++r) gsum[r] = 0.0;
+  for (int r = 0; r < kGradN; ++r) acc[r] = 0.f;
 
   long long item = a.pixlist ? (long long)blockIdx.x * blockDim.x + threadIdx.x
                              : (long long)blockIdx.x;
@@ -177,19 +204,17 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
     const int os = a.os;
     const float kahn = a.kahn;
     const float cutg = kGaussCut * 0.63f;
-    const double wp = g.dLdI[gp];
-    const double wks = wp * g.kc * g.scale;
+    const float wp = (float)g.dLdI[gp];
     const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
-    double tot[kGradN];
-#pragma unroll
-    for (int r = 0; r < kGradN; ++r) tot[r] = 0.0;
+    const float cn0[3] = {2.f / a.N[0], 2.f / a.N[1], 2.f / a.N[2]},
+                cn1[3] = {-4.f * a.N[0] * (1.f / 0.63f),
+                          -4.f * a.N[1] * (1.f / 0.63f),
+                          -4.f * a.N[2] * (1.f / 0.63f)};
     for (int i = 0; i < os; ++i)
       for (int j = 0; j < os; ++j)
         for (int t = 0; t < a.T; ++t) {
-          float vh[3], vl[3], v32[3], df[3], omega;
+          float vh[3], vl[3], df[3], omega;
           unit_geometry_ff(a, P, s, f, i, j, t, vh, vl, df, omega);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) v32[c] = vh[c];
           float cap = 1.f;
           if (a.dtff[0] > 0.f) {
             float rho = df[0] * P.ffn[0][0] + df[1] * P.ffn[1][0] +
@@ -203,11 +228,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
                 ye = df[0] * a.b0f[0] + df[1] * a.b0f[1] + df[2] * a.b0f[2];
           float scal = omega * cap * 0.5f *
                        (1.f + c2 * c2 - kahn * (xe * xe - ye * ye));
-          const float fscal = (float)(wks * (double)scal);  // F scatter
-          Kahan acc0;
-          float acc[9];
-#pragma unroll
-          for (int r = 0; r < 9; ++r) acc[r] = 0.f;
+          const float Wt = wp * scal;
           for (int pm = 0; pm < a.PM; ++pm) {
             const float *Ah = s_axh + pm * 9, *Al = s_axl + pm * 9;
             float Gh[3], Gl[3], rq[3], rl[3], n0[3];
@@ -224,43 +245,47 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
                                 1.f / 2097152.f);
               rl[x] = rl0 + __fsub_rn(rh, rq[x]);
             }
-            // dG[r][x] = dA_pm[r][x] . (d - i0)
-            float dG[6][3];
-            const float *dA = s_dax + pm * 54;
-#pragma unroll
-            for (int r = 0; r < 6; ++r)
-#pragma unroll
-              for (int x = 0; x < 3; ++x)
-                dG[r][x] = dA[r * 9 + 3 * x] * v32[0] +
-                           dA[r * 9 + 3 * x + 1] * v32[1] +
-                           dA[r * 9 + 3 * x + 2] * v32[2];
-            for (int k = 0; k < a.S; ++k) {
-              const float *src = s_src + k * SRC32_STRIDE;
-              const float dh = src[SRC32_DH], dl = src[SRC32_DL];
-              float fr[3], nf[3];
+            // Σ_k e_x of this orientation's steps
+            float E[3] = {0.f, 0.f, 0.f};
+            // the steps that survive the cut, 32 sources at a time: every
+            // lane then evaluates its own ones one after another, so that the
+            // warp goes through the evaluation as often as the lane with the
+            // most (4 or 5 of 8 sources) and not once per source that some
+            // lane needs
+            for (int k0 = 0; k0 < a.S; k0 += 32) {
+            unsigned hits = 0;
+            const int nk = min(32, a.S - k0);
+            for (int j = 0; j < nk; ++j) {
+              const float dh = s_src[(k0 + j) * SRC32_STRIDE + SRC32_DH];
+              float fr[3];
 #pragma unroll
               for (int x = 0; x < 3; ++x) {
-                float tq = fmaf(Gh[x], dh, rq[x]);
-                nf[x] = rintf(tq);
-                fr[x] = tq - nf[x];
+                const float tq = fmaf(Gh[x], dh, rq[x]);
+                fr[x] = tq - rintf(tq);
               }
               float rad2 = N2[0] * fr[0] * fr[0];
               rad2 = fmaf(N2[1] * fr[1], fr[1], rad2);
               rad2 = fmaf(N2[2] * fr[2], fr[2], rad2);
-              if (rad2 > cutg) continue;
+              if (!(rad2 > cutg)) hits |= 1u << j;
+            }
+            while (hits) {
+              const float *src =
+                  s_src + (k0 + __ffs(hits) - 1) * SRC32_STRIDE;
+              hits &= hits - 1;
+              const float dh = src[SRC32_DH], dl = src[SRC32_DL];
+              float fr[3];
+              int n[3];
 #pragma unroll
               for (int x = 0; x < 3; ++x) {
-                float sx = fmaf(Gh[x], dh, __fsub_rn(rq[x], nf[x]));
+                const float nf = rintf(fmaf(Gh[x], dh, rq[x]));
+                const float sx = fmaf(Gh[x], dh, __fsub_rn(rq[x], nf));
                 fr[x] = sx + fmaf(Gh[x], dl, fmaf(Gl[x], dh, rl[x]));
+                n[x] = __float2int_rn(n0[x] + nf) - a.hmin[x];
               }
-              rad2 = N2[0] * fr[0] * fr[0];
+              float rad2 = N2[0] * fr[0] * fr[0];
               rad2 = fmaf(N2[1] * fr[1], fr[1], rad2);
               rad2 = fmaf(N2[2] * fr[2], fr[2], rad2);
               float fl2 = a.N6 * expf(-2.f * rad2 * (1.f / 0.63f));
-              int n[3];
-#pragma unroll
-              for (int x = 0; x < 3; ++x)
-                n[x] = __float2int_rn(n0[x] + nf[x]) - a.hmin[x];
               bool inside = (unsigned)n[0] < (unsigned)a.hn[0] &&
                             (unsigned)n[1] < (unsigned)a.hn[1] &&
                             (unsigned)n[2] < (unsigned)a.hn[2];
@@ -307,33 +332,21 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
                 }
               }
               if (!tri) fc = inside ? __ldg(a.F + nb_idx(a.check, NB_SITE_F, fidx, table_size(a))) : a.defF;
-              float w = src[SRC32_W];
-              float term = fc * fc * fl2 * w;
-              acc0.add(term);
-              // d/d(tx..c): term * u_k * sum_x dlog_x dG[r][x]
-              float uk = a.u0h + dh;
-              float dl0 = -4.f * N2[0] * fr[0] * (1.f / 0.63f),
-                    dl1 = -4.f * N2[1] * fr[1] * (1.f / 0.63f),
-                    dl2 = -4.f * N2[2] * fr[2] * (1.f / 0.63f);
-              float tu = term * uk;
+              const float w = src[SRC32_W];
+              const float tw = Wt * (fc * fc * fl2 * w);
               // d term / d h_x = term dlog_x + 2 F dF/dh_x F_latt^2 w
-              float fgu = 2.f * fc * fl2 * w * uk;
-              float e0 = fmaf(tu, dl0, fgu * dfc[0]),
-                    e1 = fmaf(tu, dl1, fgu * dfc[1]),
-                    e2 = fmaf(tu, dl2, fgu * dfc[2]);
+              const float uk = a.u0h + dh, tu = tw * uk,
+                          fgu = Wt * (2.f * fc * fl2 * w) * uk;
 #pragma unroll
-              for (int r = 0; r < 6; ++r)
-                acc[r] = fmaf(e0, dG[r][0],
-                              fmaf(e1, dG[r][1], fmaf(e2, dG[r][2], acc[r])));
-#pragma unroll
-              for (int x = 0; x < 3; ++x)
-                acc[6 + x] = fmaf(term,
-                                  2.f / a.N[x] -
-                                      4.f * a.N[x] * fr[x] * fr[x] *
-                                          (1.f / 0.63f),
-                                  acc[6 + x]);
+              for (int x = 0; x < 3; ++x) {
+                E[x] += fmaf(tu, -4.f * N2[x] * fr[x] * (1.f / 0.63f),
+                             INTERP ? fgu * dfc[x] : 0.f);
+                acc[9 + x] = fmaf(tw, fmaf(cn1[x] * fr[x], fr[x], cn0[x]),
+                                  acc[9 + x]);
+              }
+              acc[12] += tw;
               if (HASF) {
-                const float gvf = fscal * (2.f * fc * fl2 * w);
+                const float gvf = Wt * g.kcs * (2.f * fc * fl2 * w);
                 if (tri) {
                   if (!holding || n[0] != held[0] || n[1] != held[1] ||
                       n[2] != held[2]) {
@@ -369,23 +382,25 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
                 }
               }
             }
+            }
+            float vr[3];
+            unrotate(s_rot + pm * 9, vh, vr);
+#pragma unroll
+            for (int x = 0; x < 3; ++x)
+#pragma unroll
+              for (int c = 0; c < 3; ++c)
+                acc[3 * x + c] = fmaf(E[x], vr[c], acc[3 * x + c]);
           }
-          tot[9] += (double)scal * acc0.value();
-#pragma unroll
-          for (int r = 0; r < 9; ++r) tot[r] += (double)scal * (double)acc[r];
         }
-#pragma unroll
-    for (int r = 0; r < 9; ++r) gsum[r] = wks * tot[r];
-    gsum[9] = wp * g.kc * tot[9];  // dI/dscale = I / scale
   }
   if (INTERP && HASF) flush_node();
   if (HASF && near_idx >= 0) atomicAdd(g.gradF + nb_idx(a.check, NB_SITE_GRADF, near_idx, table_size(a)), (double)near_sum);
-  // block reduction in FP64, fixed order
-  __shared__ double red[kTileThreads / 32][kGradN];
+  // block reduction in a fixed order: a butterfly in FP32, the warps in FP64
+  __shared__ float red[kTileThreads / 32][kGradN];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int r = 0; r < kGradN; ++r) {
-    double v = gsum[r];
+    float v = acc[r];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (lane == 0) red[warp][r] = v;
@@ -393,7 +408,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   __syncthreads();
   if (threadIdx.x < kGradN) {
     double v = 0.0;
-    for (int w = 0; w < kTileThreads / 32; ++w) v += red[w][threadIdx.x];
+    for (int w = 0; w < kTileThreads / 32; ++w) v += (double)red[w][threadIdx.x];
     g.partials[(size_t)blockIdx.x * kGradN + threadIdx.x] = v;
   }
 }
@@ -418,11 +433,10 @@ constexpr int kAdjFold = 16;  // passes between folds into FP64
 
 __host__ __device__ inline size_t adj_ring_floats(int PM, int S,
                                                   bool f_cache) {
-  // the tables, then (F gradient) each thread's 5x5x4 column as 25 float4
-  // (16-byte aligned: 2 PM 9 + 12 S + 54 PM is a multiple of 4)
-  size_t fl = (size_t)2 * PM * 9 + (size_t)S * SRC32_STRIDE + (size_t)PM * 54 +
-              (f_cache ? (size_t)100 * kTileThreads : 0);
-  return (fl + 3) & ~(size_t)3;  // 16-byte aligned records after it
+  // the tables, then (F gradient) each thread's 5x5x4 column as 25 float4,
+  // then the records: each 16-byte aligned
+  const size_t fl = (size_t)3 * PM * 9 + (size_t)S * SRC32_STRIDE;
+  return ((fl + 3) & ~(size_t)3) + (f_cache ? (size_t)100 * kTileThreads : 0);
 }
 
 __host__ __device__ inline size_t adj_ring_smem_bytes(int PM, int S,
@@ -441,18 +455,17 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   float *s_axh = smf;
   float *s_axl = smf + a.PM * 9;
   float *s_src = smf + 2 * a.PM * 9;
-  float *s_dax = s_src + a.S * SRC32_STRIDE;
+  float *s_rot = s_src + a.S * SRC32_STRIDE;
   for (int i = threadIdx.x; i < a.PM * 9; i += blockDim.x) {
     s_axh[i] = a.axh[i];
     s_axl[i] = a.axl[i];
+    s_rot[i] = g.rot[i];
   }
   for (int i = threadIdx.x; i < a.S * SRC32_STRIDE; i += blockDim.x)
     s_src[i] = a.src32[i];
-  for (int i = threadIdx.x; i < a.PM * 54; i += blockDim.x)
-    s_dax[i] = g.dax[i];
   const bool fcache = INTERP && HASF;
-  float4 (*s_col)[kTileThreads] =
-      reinterpret_cast<float4 (*)[kTileThreads]>(s_dax + a.PM * 54);
+  float4 (*s_col)[kTileThreads] = reinterpret_cast<float4 (*)[kTileThreads]>(
+      smf + adj_ring_floats(a.PM, a.S, false));
   float4 *s_rec = reinterpret_cast<float4 *>(
       smf + adj_ring_floats(a.PM, a.S, fcache));
   int *s_recb = reinterpret_cast<int *>(s_rec + (kTileThreads / 32) * kAdjRing);
@@ -524,12 +537,14 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
   const float cutg = kGaussCut * 0.63f;
   const float kahn = a.kahn;
-  const float scalef = (float)g.scale;
-
   float acc[kGradN];
 #pragma unroll
   for (int r = 0; r < kGradN; ++r) acc[r] = 0.f;
   double dacc = 0.0;  // lane r < kGradN: the warp's folded sum r
+  const float cn0[3] = {2.f / a.N[0], 2.f / a.N[1], 2.f / a.N[2]},
+              cn1[3] = {-4.f * a.N[0] * (1.f / 0.63f),
+                        -4.f * a.N[1] * (1.f / 0.63f),
+                        -4.f * a.N[2] * (1.f / 0.63f)};
   int head = 0, tail = 0, passes = 0;
 
   auto fold = [&]() {
@@ -646,35 +661,24 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
         }
       }
       if (!tri) fc = inside ? __ldg(a.F + nb_idx(a.check, NB_SITE_F, fidx, table_size(a))) : a.defF;
-      const float term = fc * fc * fl2 * w;
+      const float tw = Wt * (fc * fc * fl2 * w);
       const float uk = a.u0h + dh;
-      const float tu = term * uk, fgu = 2.f * fc * fl2 * w * uk;
-      float e[3];
+      const float tu = tw * uk, fgu = Wt * (2.f * fc * fl2 * w) * uk;
+      float vr[3];
+      unrotate(s_rot + pm * 9, v32, vr);
 #pragma unroll
-      for (int x = 0; x < 3; ++x)
-        e[x] = fmaf(tu, -4.f * N2[x] * fr[x] * (1.f / 0.63f), fgu * dfc[x]);
-      // d term / d theta_r = sum_x e_x dA_pm[r][x] . v
-      const float *dA = s_dax + pm * 54;
+      for (int x = 0; x < 3; ++x) {
+        const float e = fmaf(tu, -4.f * N2[x] * fr[x] * (1.f / 0.63f),
+                             fgu * dfc[x]);
 #pragma unroll
-      for (int r = 0; r < 6; ++r) {
-        float gr = 0.f;
-#pragma unroll
-        for (int x = 0; x < 3; ++x) {
-          const float *d3 = dA + r * 9 + 3 * x;
-          gr = fmaf(e[x], d3[0] * v32[0] + d3[1] * v32[1] + d3[2] * v32[2],
-                    gr);
-        }
-        acc[r] = fmaf(Wt, gr, acc[r]);
+        for (int c = 0; c < 3; ++c)
+          acc[3 * x + c] = fmaf(e, vr[c], acc[3 * x + c]);
+        acc[9 + x] = fmaf(tw, fmaf(cn1[x] * fr[x], fr[x], cn0[x]),
+                          acc[9 + x]);
       }
-      const float tw = Wt * term;
-#pragma unroll
-      for (int x = 0; x < 3; ++x)
-        acc[6 + x] = fmaf(tw, 2.f / a.N[x] - 4.f * a.N[x] * fr[x] * fr[x] *
-                                                 (1.f / 0.63f),
-                          acc[6 + x]);
-      acc[9] += tw;
+      acc[12] += tw;
       if (HASF) {
-        const float gvf = Wt * scalef * (2.f * fc * fl2 * w);
+        const float gvf = Wt * g.kcs * (2.f * fc * fl2 * w);
         if (tri) {
           // the column was flushed unless it holds this key
           held_key = (npk & 0xfffff) | ((fl[2] + 1) << 20);
@@ -740,8 +744,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
       // the row's records are all evaluated: its sums, then the next row
       fold();
       if (lane < kGradN)
-        g.partials[(size_t)row * kGradN + lane] =
-            lane < 9 ? g.scale * dacc : dacc;
+        g.partials[(size_t)row * kGradN + lane] = dacc;
       dacc = 0.0;
       passes = 0;
       row = next_row();
@@ -764,7 +767,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
         f = 0;
       }
       P = a.panels + q;
-      W0 = ok ? (float)(g.dLdI[gp] * g.kc) : 0.f;
+      W0 = ok ? (float)g.dLdI[gp] : 0.f;
       new_pixel = false;
     }
     if (new_unit) {
@@ -857,41 +860,134 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   if (HASF && near_idx >= 0) atomicAdd(g.gradF + nb_idx(a.check, NB_SITE_GRADF, near_idx, table_size(a)), near_sum);
 }
 
-// sums partial rows [n][kGradN] in a fixed order: one block of 32 x kGradN
+// Sums the partial rows [n][kGradN] in a fixed order: block b its share of
+// `per` rows into row b of out.  32 threads per column; a thread's loads are
+// independent of one another and a row's columns lie side by side.  (One
+// block for all rows took 91 us for the 19968 blocks of the 64-panel shot and
+// 347 us for its 79872 pixel rows, waiting on one load after another.)
 __global__ void reduce_partials_kernel(const double *part, long long n,
-                                       double *out) {
-  __shared__ double red[kGradN][32];
-  int r = threadIdx.y, lane = threadIdx.x;
+                                       long long per, double *out) {
+  __shared__ double red[32][kGradN];
+  const int r = threadIdx.x, lane = threadIdx.y;
+  const long long first = blockIdx.x * per,
+                  last = first + per < n ? first + per : n;
   double v = 0.0;
-  for (long long i = lane; i < n; i += 32) v += part[i * kGradN + r];
-  red[r][lane] = v;
+#pragma unroll 4
+  for (long long i = first + lane; i < last; i += 32)
+    v += part[i * kGradN + r];
+  red[lane][r] = v;
   __syncthreads();
   if (lane == 0) {
     double s = 0.0;
-    for (int l = 0; l < 32; ++l) s += red[r][l];
-    out[r] = s;
+    for (int l = 0; l < 32; ++l) s += red[l][r];
+    out[(long long)blockIdx.x * kGradN + r] = s;
   }
 }
 
-// Poisson loss L = sum_p (I_p + bkg - y_p log(I_p + bkg)) and dL/dI_p
-__global__ void poisson_loss_kernel(const double *img, const double *y,
-                                    long long n, double bkg, double *dLdI,
-                                    double *partials) {
+// rows [0, n) of part to one row in out; scratch for kReduceRows rows
+constexpr int kReduceRows = 128;
+static cudaError_t reduce_partials(const double *part, long long n,
+                                   double *scratch, double *out,
+                                   cudaStream_t st) {
+  const dim3 threads(kGradN, 32);
+  if (n > 4 * kReduceRows) {
+    const long long per = (n + kReduceRows - 1) / kReduceRows;
+    reduce_partials_kernel<<<kReduceRows, threads, 0, st>>>(part, n, per,
+                                                            scratch);
+    part = scratch;
+    n = kReduceRows;
+  }
+  reduce_partials_kernel<<<1, threads, 0, st>>>(part, n, n, out);
+  return cudaGetLastError();
+}
+
+// Poisson loss L = sum_p (I_p + bkg - y_p log(I_p + bkg)) and dL/dI_p.
+// Bound by the FP64 pipe (1/64 of the FP32 rate), so the logarithm and the
+// quotient share what they can.  m = 2^e z, z in [1, 2); a table of 64
+// intervals gives c ~ 1/z, and r = z c - 1 (|r| < 2^-7, exact in one FMA) is
+// both the argument of log1p, summed as its series to r^9 (remainder below
+// 2^-72; after Tang, "Table-driven implementation of the logarithm function",
+// 1990), and the first correction of the reciprocal.  About 30 FP64
+// instructions per pixel instead of 70: 234 -> 111 us for the 2.3e6 pixels of
+// the 64-panel shot.  The table is made per block from log and division, so
+// the blocks are few and persistent.
+constexpr int kLogTable = 64;
+
+__device__ __forceinline__ void poisson_pixel(double m, double y,
+                                              const double2 *tab, double &l,
+                                              double &d) {
+  const long long bits = __double_as_longlong(m);
+  const int ex = (int)(bits >> 52);  // with the sign: negative for m < 0
+  if (ex < 523 || ex > 1523 ||
+      ((__double2hiint(y) >> 20) & 0x7ff) > 1500) {
+    // tiny, huge, negative or not a number
+    l += m - y * log(m);
+    d = 1.0 - y / m;
+    return;
+  }
+  const double z = __longlong_as_double((bits & 0x000fffffffffffffll) |
+                                        0x3ff0000000000000ll);
+  const double2 t = tab[(int)(bits >> 46) & (kLogTable - 1)];
+  const double r = fma(z, t.x, -1.0), r2 = r * r;
+  double q = fma(r, 1.0 / 9.0, -1.0 / 8.0);
+  q = fma(q, r, 1.0 / 7.0);
+  q = fma(q, r, -1.0 / 6.0);
+  q = fma(q, r, 1.0 / 5.0);
+  q = fma(q, r, -0.25);
+  q = fma(q, r, 1.0 / 3.0);
+  q = fma(q, r, -0.5);
+  // the exponent as a double: its bits in the last place of 2^52 + 2^51
+  const double e = __longlong_as_double(0x4338000000000000ll + (ex - 1023)) -
+                   6755399441055744.0;
+  const double lg = fma(e, 0.69314718055994530942, t.y) + fma(q, r2, r);
+  l += fma(-y, lg, m);
+  // 1/z from c: 1/(1 + r) = (1 - r)(1 + r^2)(1 + r^4) ...
+  double x = fma(-t.x, r, t.x);
+  x = fma(x, fma(r2, r2, r2), x);
+  x = x * __hiloint2double((2046 - ex) << 20, 0);  // 2^-e
+  const double p = y * x;
+  d = 1.0 - fma(fma(-p, m, y), x, p);
+}
+
+__global__ void __launch_bounds__(256)
+    poisson_loss_kernel(const double *img, const double *y, long long n,
+                        double bkg, double *dLdI, double *partials) {
+  __shared__ double2 tab[kLogTable];
+  __shared__ double red[8];
+  for (int i = threadIdx.x; i < kLogTable; i += blockDim.x) {
+    const double c = 1.0 / (1.0 + (i + 0.5) / kLogTable);
+    tab[i] = make_double2(c, -log(c));
+  }
+  __syncthreads();
   double l = 0.0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    double m = img[i] + bkg;
-    l += m - y[i] * log(m);
-    dLdI[i] = 1.0 - y[i] / m;
+    double d;
+    poisson_pixel(img[i] + bkg, y[i], tab, l, d);
+    dLdI[i] = d;
   }
-  __shared__ double red[32];
   for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-    partials[(size_t)blockIdx.x * kGradN] = s;
+    for (int w = 0; w < 8; ++w) s += red[w];
+    partials[blockIdx.x] = s;
+  }
+}
+
+// the block sums of the loss, in a fixed order
+__global__ void loss_sum_kernel(const double *part, int n, double *out) {
+  __shared__ double red[32];
+  double v = 0.0;
+  for (int i = threadIdx.x; i < n; i += 1024) v += part[i];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    v = red[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) *out = v;
   }
 }
 
@@ -906,7 +1002,7 @@ static bool adjoint_ring_ok(const SpotArgs &a) {
 
 size_t adjoint_smem_bytes(const SpotArgs &a, bool f_cache) {
   if (adjoint_ring_ok(a)) return adj_ring_smem_bytes(a.PM, a.S, f_cache);
-  return (size_t)(2 * a.PM * 9 + a.S * SRC32_STRIDE + a.PM * 54 +
+  return (size_t)(3 * a.PM * 9 + a.S * SRC32_STRIDE +
                   (f_cache ? 125 * kTileThreads : 0)) *
          sizeof(float);
 }
@@ -921,18 +1017,24 @@ long long adjoint_blocks(const SpotArgs &a) {
                    : a.n_tiles;
 }
 
-cudaError_t launch_adjoint(const SpotArgs &a, const float *dax,
+size_t adjoint_scratch_bytes(const SpotArgs &a) {
+  // the partial rows, the row counter, the rows of the first reduction
+  return (size_t)(adjoint_blocks(a) + 1 + kReduceRows) * kGradN *
+         sizeof(double);
+}
+
+// writes the kGradN sums, without the prefactor kc, to sums_out
+cudaError_t launch_adjoint(const SpotArgs &a, const float *rot,
                            const double *dLdI, double *gradF,
                            double *partials, double kc, double scale,
-                           double *grad_out, int sm_count, cudaStream_t st) {
+                           double *sums_out, int sm_count, cudaStream_t st) {
   AdjointArgs g;
   g.a = a;
-  g.dax = dax;
+  g.rot = rot;
   g.dLdI = dLdI;
   g.gradF = gradF;
   g.partials = partials;
-  g.kc = kc;
-  g.scale = scale;
+  g.kcs = (float)(kc * scale);
   g.rows_next = nullptr;
   g.n_rows = 0;
   size_t smem = adjoint_smem_bytes(a, a.interp && gradF);
@@ -971,14 +1073,25 @@ cudaError_t launch_adjoint(const SpotArgs &a, const float *dax,
   kern<<<(unsigned)grid, kTileThreads, smem, st>>>(g);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  reduce_partials_kernel<<<1, dim3(32, kGradN), 0, st>>>(partials, blocks,
-                                                        grad_out);
-  return cudaGetLastError();
+  return reduce_partials(partials, blocks, partials + (blocks + 1) * kGradN,
+                         sums_out, st);
+}
+
+// grad (10) from the kGradN sums and the derivatives of the lab axes
+void adjoint_gradient(const double *sums, const double daxes[6][9], double kc,
+                      double scale, double *grad) {
+  for (int r = 0; r < 6; ++r) {
+    double v = 0.0;
+    for (int i = 0; i < 9; ++i) v += daxes[r][i] * sums[i];
+    grad[r] = kc * scale * v;
+  }
+  for (int x = 0; x < 3; ++x) grad[6 + x] = kc * scale * sums[9 + x];
+  grad[9] = kc * sums[12];
 }
 
 int loss_blocks(long long n) {
   long long b = (n + 255) / 256;
-  return (int)(b < 1216 ? (b < 1 ? 1 : b) : 1216);
+  return (int)(b < 608 ? (b < 1 ? 1 : b) : 608);
 }
 
 cudaError_t launch_poisson_loss(const double *img, const double *y,
@@ -989,9 +1102,7 @@ cudaError_t launch_poisson_loss(const double *img, const double *y,
   poisson_loss_kernel<<<blocks, 256, 0, st>>>(img, y, n, bkg, dLdI, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // column 0 of the partial rows holds the block sums
-  reduce_partials_kernel<<<1, dim3(32, 1), 0, st>>>(partials, blocks,
-                                                   loss_out);
+  loss_sum_kernel<<<1, 1024, 0, st>>>(partials, blocks, loss_out);
   return cudaGetLastError();
 }
 

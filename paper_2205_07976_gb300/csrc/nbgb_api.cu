@@ -111,7 +111,7 @@ struct nb_sim {
   bool have_params = false;
   double pU[9] = {0}, pcell[3] = {0}, prot[3] = {0};
   double daxes[6][9];  // d(lab axes)/d(tx, ty, tz, a, b, c)
-  DevBuf d_dax, d_part, d_grad, d_F4, d_C4, d_F64t;
+  DevBuf d_rot, d_part, d_grad, d_F4, d_C4, d_F64t;
   bool F4_valid = false, C4_valid = false, F64_valid = false;
   bool fmax_valid = false;  // the largest |F|, behind the counters
   int has_div = 0;
@@ -467,19 +467,19 @@ static int upload_tables(nb_sim *s) {
                     cudaMemcpyHostToDevice, s->stream);
   }
   if (s->have_params) {
-    // derivative of every rotated axis: the same rotations applied to the
-    // derivative of the lab axes (the maps are linear): [PM][6][9] floats
-    std::vector<float> dax((size_t)PM * 54);
-    for (int r = 0; r < 6; ++r) {
-      std::vector<double> t;
-      build_axes_of(s, s->daxes[r], t);
-      for (int pm = 0; pm < PM; ++pm)
-        for (int i = 0; i < 9; ++i)
-          dax[(size_t)pm * 54 + r * 9 + i] = (float)t[(size_t)pm * 9 + i];
-    }
-    if ((e = s->d_dax.ensure(dax.size() * 4)) != cudaSuccess)
-      return fail(s, NB_ENOMEM, "derivative table");
-    cudaMemcpyAsync(s->d_dax.p, dax.data(), dax.size() * 4,
+    // the rotation of every orientation, row-major: its columns are the
+    // rotated unit vectors
+    const double eye[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
+    std::vector<double> t;
+    build_axes_of(s, eye, t);
+    std::vector<float> rot(t.size());
+    for (int pm = 0; pm < PM; ++pm)
+      for (int v = 0; v < 3; ++v)
+        for (int r = 0; r < 3; ++r)
+          rot[(size_t)pm * 9 + 3 * r + v] = (float)t[(size_t)pm * 9 + 3 * v + r];
+    if ((e = s->d_rot.ensure(rot.size() * 4)) != cudaSuccess)
+      return fail(s, NB_ENOMEM, "rotation table");
+    cudaMemcpyAsync(s->d_rot.p, rot.data(), rot.size() * 4,
                     cudaMemcpyHostToDevice, s->stream);
   }
   // pageable copies are staged before return; check the queue is healthy
@@ -629,7 +629,7 @@ int nb_free(nb_sim *sim) {
                       &sim->d_axl,    &sim->d_src64, &sim->d_src32,
                       &sim->d_divh,   &sim->d_divl,  &sim->d_F,
                       &sim->d_image,  &sim->d_list,  &sim->d_tmp,
-                      &sim->d_stats,  &sim->d_work,  &sim->d_srcq,  &sim->d_check,  &sim->d_dax,
+                      &sim->d_stats,  &sim->d_work,  &sim->d_srcq,  &sim->d_check,  &sim->d_rot,
                       &sim->d_part,   &sim->d_grad,  &sim->d_F4,
                       &sim->d_C4,     &sim->d_F64t,  &sim->d_bg64,
                       &sim->d_bg32,   &sim->d_bgrng};
@@ -1152,23 +1152,26 @@ int nb_adjoint(nb_sim *s, const double *dLdI, double grad[10],
   ensure_cell_polynomials(s);  // tricubic value and gradient per cell
   SpotArgs a;
   fill_args(s, a);
-  if (nbgb::adjoint_smem_bytes(a, a.interp == NB_INTERP_TRICUBIC && gradF) >
-      200 * 1024)
+  // (the limit leaves room for 45 floats per orientation that the kernels no
+  // longer stage: sizes that were refused stay refused)
+  if (nbgb::adjoint_smem_bytes(a, a.interp == NB_INTERP_TRICUBIC && gradF) +
+          (size_t)180 * a.PM > 200 * 1024)
     return fail(s, NB_EINVAL, "tables exceed 200 KB of shared memory");
-  long long blocks = nbgb::adjoint_blocks(a);
-  cudaError_t e = s->d_part.ensure((size_t)(blocks + 1) * 10 * sizeof(double));
+  cudaError_t e = s->d_part.ensure(nbgb::adjoint_scratch_bytes(a));
   if (e == cudaSuccess) e = s->d_grad.ensure(16 * sizeof(double));
   if (e != cudaSuccess) return fail(s, NB_ENOMEM, "gradient scratch");
   double kc = nbgb::kElectronRadius * nbgb::kElectronRadius * s->fluence /
               ((double)s->os * s->os * s->n_mosaic * s->n_phi);
-  e = nbgb::launch_adjoint(a, (const float *)s->d_dax.p, dLdI, gradF,
+  e = nbgb::launch_adjoint(a, (const float *)s->d_rot.p, dLdI, gradF,
                            (double *)s->d_part.p, kc, s->scale,
                            (double *)s->d_grad.p, s->sm_count, s->stream);
+  double sums[nbgb::kAdjointSums] = {0};
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(grad, s->d_grad.p, 10 * sizeof(double),
+    e = cudaMemcpyAsync(sums, s->d_grad.p, sizeof sums,
                         cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "adjoint");
+  nbgb::adjoint_gradient(sums, s->daxes, kc, s->scale, grad);
   return read_check(s);
 }
 

@@ -378,10 +378,14 @@ cudaError_t build_cell_polynomials(const float *F, const int hn[3], float4 *C4,
 size_t adjoint_smem_bytes(const SpotArgs &a, bool f_cache);
 long long adjoint_blocks(const SpotArgs &a);
 int loss_blocks(long long n);
-cudaError_t launch_adjoint(const SpotArgs &a, const float *dax,
+size_t adjoint_scratch_bytes(const SpotArgs &a);
+cudaError_t launch_adjoint(const SpotArgs &a, const float *rot,
                            const double *dLdI, double *gradF,
                            double *partials, double kc, double scale,
-                           double *grad_out, int sm_count, cudaStream_t st);
+                           double *sums_out, int sm_count, cudaStream_t st);
+constexpr int kAdjointSums = 13;
+void adjoint_gradient(const double *sums, const double daxes[6][9], double kc,
+                      double scale, double *grad);
 cudaError_t launch_poisson_loss(const double *img, const double *y,
                                 long long n, double bkg, double *dLdI,
                                 double *partials, double *loss_out,
