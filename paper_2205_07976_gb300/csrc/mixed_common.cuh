@@ -87,9 +87,11 @@ __device__ __forceinline__ void ff_mul(float ah, float al, float bh, float bl,
 // Geometry of sub-pixel unit (i, j, layer t) of pixel (s, f) of panel P in
 // double-float FP32 arithmetic (FP64 issues at 1/64 of the FP32 rate on
 // this part): v = d - i0 as (vh, vl), d rounded to FP32, and the solid
-// angle omega = px^2 (n . P) / |P|^3 in FP32.  The reciprocal length is
+// angle omega = px^2 (n . P) / |P|^3 in FP32 (OMEGA_FF: formed in
+// double-float and rounded once).  The reciprocal length is
 // the FP32 rsqrt estimate refined by one Newton step carried in
 // double-float, so d is good to ~1e-13.
+template <bool OMEGA_FF = false>
 __device__ __forceinline__ void unit_geometry_ff(const SpotArgs &a,
                                                  const DevPanel &P, int s,
                                                  int f, int i, int j, int t,
@@ -141,6 +143,20 @@ __device__ __forceinline__ void unit_geometry_ff(const SpotArgs &a,
     ff_mul(ph[c], pl[c], rih, ril, dh, dl);
     df[c] = dh;
     ff_add(dh, dl, -a.i0ff[c][0], -a.i0ff[c][1], vh[c], vl[c]);
+  }
+  if (OMEGA_FF) {
+    float nh, nl, qh2, ql2;
+    ff_mul(P.ffn[0][0], P.ffn[0][1], ph[0], pl[0], nh, nl);
+    ff_mul(P.ffn[1][0], P.ffn[1][1], ph[1], pl[1], th, tl);
+    ff_add(nh, nl, th, tl, nh, nl);
+    ff_mul(P.ffn[2][0], P.ffn[2][1], ph[2], pl[2], th, tl);
+    ff_add(nh, nl, th, tl, nh, nl);
+    ff_mul(P.ffpx[0], P.ffpx[1], rih, ril, qh2, ql2);  // px / |P|
+    ff_mul(qh2, ql2, qh2, ql2, qh2, ql2);
+    ff_mul(nh, nl, rih, ril, nh, nl);
+    ff_mul(nh, nl, qh2, ql2, nh, nl);
+    omega = nh;
+    return;
   }
   const float nd = P.ffn[0][0] * ph[0] + P.ffn[1][0] * ph[1] +
                    P.ffn[2][0] * ph[2];

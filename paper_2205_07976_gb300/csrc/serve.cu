@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kTileThreads, 4)
 // run one warp per pixel (tricubic lookup, >= 8 subpixel x mosaic items):
 // each work item stages its request's tables once, then each warp sums its
 // pixels with the same device function as the stand-alone kernel.
-template <int INTERP>
+template <int INTERP, bool FF>
 __global__ void __launch_bounds__(kSplitThreads, 5)
     serve_warp_kernel(SpotArgs base, const SlotParams *slots,
                       const WorkList *wl, unsigned *counter, double *pool) {
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
         const long long p = w.first + warp + (long long)(i0 + bi) * kSplitWarps;
         const int s = sp.s0 + (int)(p / sp.nf);
         const int f = sp.f0 + (int)(p % sp.nf);
-        split_unit<0>(base, P, s, f, lane - bi * U, unit + lane * kUnitFloats);
+        split_unit<0, FF>(base, P, s, f, lane - bi * U, unit + lane * kUnitFloats);
       }
       __syncwarp();
       for (int bi = 0; bi < nb; ++bi) {
@@ -327,8 +327,9 @@ static int build_graph(nb_server *s, int b) {
       s->base, (const SlotParams *)s->d_slots.p, dw, ctr,
       (double *)s->d_pool.p);
   if (s->interp == NB_INTERP_TRICUBIC) {
-    nbgb::serve_warp_kernel<1><<<s->blocks_w, nbgb::kSplitThreads, s->smem_w,
-                                 st>>>(
+    auto warp_kern = nbgb::split_ff(s->base) ? nbgb::serve_warp_kernel<1, true>
+                                             : nbgb::serve_warp_kernel<1, false>;
+    warp_kern<<<s->blocks_w, nbgb::kSplitThreads, s->smem_w, st>>>(
         s->base, (const SlotParams *)s->d_slots.p, dww, ctr + 1,
         (double *)s->d_pool.p);
   }
@@ -539,13 +540,14 @@ int nb_server_create(nb_server **out, int device, void *cuda_stream,
     s->blocks = s->sm_count * (per_sm > 0 ? per_sm : 1);
     if (interp == NB_INTERP_TRICUBIC) {
       s->smem_w = nbgb::serve_warp_smem_bytes();
-      cudaFuncSetAttribute(nbgb::serve_warp_kernel<1>,
+      auto warp_kern = nbgb::split_ff(a) ? nbgb::serve_warp_kernel<1, true>
+                                         : nbgb::serve_warp_kernel<1, false>;
+      cudaFuncSetAttribute(warp_kern,
                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)s->smem_w);
       int per_sm_w = 0;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &per_sm_w, nbgb::serve_warp_kernel<1>, nbgb::kSplitThreads,
-          s->smem_w);
+          &per_sm_w, warp_kern, nbgb::kSplitThreads, s->smem_w);
       s->blocks_w = s->sm_count * (per_sm_w > 0 ? per_sm_w : 1);
     }
     for (int i = max_slots - 1; i >= 0; --i) s->free_slots.push_back(i);

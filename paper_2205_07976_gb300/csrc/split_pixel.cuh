@@ -13,6 +13,10 @@ constexpr int kSplitWarps = 4;
 constexpr int kSplitThreads = kSplitWarps * 32;
 constexpr int kMaxUnits = 32;
 constexpr int kUnitFloats = 10;  // vh[3], vl[3], scal, df[3]
+constexpr int kFfUnits = 2;      // double-float geometry up to so many units
+inline bool split_ff(const SpotArgs &a) {
+  return a.os * a.os * a.T <= kFfUnits;
+}
 constexpr int kSrcBlock = 8;     // sources per pruning block
 // Per-warp ring of source intervals.  An entry is one (item, source range)
 // pair that can hold surviving terms, with a copy of its item's state, so
@@ -408,7 +412,8 @@ __device__ __forceinline__ int guess_index(float x, float dmin, float inv,
 // Geometry of sub-pixel unit u (subpixel i, j, sensor layer t) of pixel
 // (s, f) of panel P into ud[kUnitFloats]: v = d - i0 as double-float,
 // omega cap (times the polarization for one beam direction), and d in FP32.
-template <int HASDIV>
+// FF: double-float geometry, for shots of up to kFfUnits units (split_ff).
+template <int HASDIV, bool FF>
 __device__ __forceinline__ void split_unit(const SpotArgs &a,
                                            const DevPanel &P, int s, int f,
                                            int u, float *ud) {
@@ -416,11 +421,19 @@ __device__ __forceinline__ void split_unit(const SpotArgs &a,
   const float kahn = a.kahn;
   int t = u % a.T, ij = u / a.T, i = ij / os, j = ij % os;
   float vh[3], vl[3], df[3], omega;
-  // FP64 here (one rsqrt, products): in these kernels the FP32 pipe is the
-  // busy one and the FP64 work of a batch of units overlaps with it; the
-  // double-float form (unit_geometry_ff, which the thread-per-pixel kernel
-  // uses) measured slower here
-  {
+  // Up to kFfUnits units per pixel: double-float (unit_geometry_ff, as the
+  // thread-per-pixel kernel).  A pass over the units of one or a few pixels
+  // has few lanes at work, and ~110 FP64-pipe instructions at 16 cycles each
+  // then cost more than such a pixel's whole sum (128^2 pixels, 1 unit, 99
+  // steps: 83 -> 40 us with batches of pixels, below).  With more units: FP64
+  // (one rsqrt, products), which overlaps with the FP32 work of their many
+  // steps (1500^2 pixels, 4 units, 99 steps: double-float 2.58, FP64 2.40 ms;
+  // large shot, 8 units: 220.4 and 216.5 ms at the time).  The choice depends
+  // on the shot alone, so a pixel's value does not depend on the launch, and
+  // it is a template parameter: both in one kernel cost the large shot 0.4 %.
+  if (FF) {
+    unit_geometry_ff<true>(a, P, s, f, i, j, t, vh, vl, df, omega);
+  } else {
     const double px = P.px, inv_os = 1.0 / os;
     double cf = (f + (i + 0.5) * inv_os) * px,
            cs = (s + (j + 0.5) * inv_os) * px, cn = t * a.dt;

@@ -35,7 +35,7 @@
 namespace nbgb {
 
 // COUNT: also count the pairs, intervals and block tests (a.wstats)
-template <int INTERP, int HASDIV, int COUNT>
+template <int INTERP, int HASDIV, int COUNT, bool FF>
 __global__ void __launch_bounds__(kSplitThreads, 5)
     spots_split_kernel(SpotArgs a, unsigned long long *work) {
   extern __shared__ float sms[];
@@ -46,11 +46,17 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
   SplitCounts cnt;  // work of this warp
   // a warp takes B pixels at a time and sets up all their sub-pixel units
   // in one pass, so the FP64 geometry fills up to 32 lanes
-  // (one pixel at a time when a warp gets few pixels: pixels differ in
-  // cost, and grabbing several near the end of a launch leaves a tail)
+  // (one pixel at a time when a warp gets few pixels of many steps: pixels
+  // differ in cost, and grabbing several near the end of a launch leaves a
+  // tail; with few steps the geometry of single pixels would cost more: 512^2
+  // pixels of 1 unit and 99 steps 1.09 -> 0.22 ms, 8 units and 4800 steps
+  // 1.45 -> 1.20 ms, but 4 units and 20000 steps 2.81 -> 3.51 ms)
   const int U = a.os * a.os * a.T;
   const long long per_warp = n_work / ((long long)gridDim.x * kSplitWarps);
-  const int B = per_warp >= 256 ? kMaxUnits / U : 1;
+  const long long most =
+      per_warp >= 256 ? kMaxUnits
+      : (long long)U * a.PM * a.S <= 8192 ? per_warp / 16 : 1;
+  const int B = (int)max(1ll, min((long long)(kMaxUnits / U), most));
   float *unit = b.unit_base + warp * kMaxUnits * kUnitFloats;
   while (true) {
     long long first = 0;
@@ -65,7 +71,7 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
       const long long local = gp - P.pix0;
       const int s = (int)(local / P.nfast);
       const int f = (int)(local - (long long)s * P.nfast);
-      split_unit<HASDIV>(a, P, s, f, lane - bi * U, unit + lane * kUnitFloats);
+      split_unit<HASDIV, FF>(a, P, s, f, lane - bi * U, unit + lane * kUnitFloats);
     }
     __syncwarp();
     double mine = 0.0;  // lane bi keeps the sum of pixel bi
@@ -91,6 +97,19 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
   }
 }
 
+template <bool FF>
+static void (*pick_split(const SpotArgs &a))(SpotArgs, unsigned long long *) {
+  if (a.wstats)
+    return a.interp ? (a.has_div ? spots_split_kernel<1, 1, 1, FF>
+                                 : spots_split_kernel<1, 0, 1, FF>)
+                    : (a.has_div ? spots_split_kernel<0, 1, 1, FF>
+                                 : spots_split_kernel<0, 0, 1, FF>);
+  return a.interp ? (a.has_div ? spots_split_kernel<1, 1, 0, FF>
+                               : spots_split_kernel<1, 0, 0, FF>)
+                  : (a.has_div ? spots_split_kernel<0, 1, 0, FF>
+                               : spots_split_kernel<0, 0, 0, FF>);
+}
+
 size_t split_smem_bytes(const SpotArgs &a) {
   return split_smem_layout(a.PM, a.S);
 }
@@ -103,17 +122,7 @@ bool split_supported(const SpotArgs &a) {
 cudaError_t launch_spots_split(const SpotArgs &a, unsigned long long *work,
                                int sm_count, cudaStream_t st) {
   size_t smem = split_smem_bytes(a);
-  void (*kern)(SpotArgs, unsigned long long *);
-  if (a.wstats)
-    kern = a.interp ? (a.has_div ? spots_split_kernel<1, 1, 1>
-                                 : spots_split_kernel<1, 0, 1>)
-                    : (a.has_div ? spots_split_kernel<0, 1, 1>
-                                 : spots_split_kernel<0, 0, 1>);
-  else
-    kern = a.interp ? (a.has_div ? spots_split_kernel<1, 1, 0>
-                                 : spots_split_kernel<1, 0, 0>)
-                    : (a.has_div ? spots_split_kernel<0, 1, 0>
-                                 : spots_split_kernel<0, 0, 0>);
+  auto kern = split_ff(a) ? pick_split<true>(a) : pick_split<false>(a);
   cudaError_t e = cudaFuncSetAttribute(
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
