@@ -4,20 +4,23 @@
 //
 // Loop nest per pixel: subpixel x sensor layer -> source -> phi x mosaic.
 // Everything is FP64 and this file is compiled without FMA contraction.
-// The Miller indices, the fractional offsets and the sinc are evaluated in
-// the order the definition is written, so h and the sinc's phases are
-// bitwise those of any other uncontracted FP64 evaluation (the sinc at
-// N = 200 multiplies h's rounding by pi N).  The rest, which is not
-// sensitive to the last bits, is arranged for the FP64 pipe, which on this
-// part issues at 1/64 of the FP32 rate and so sets the kernel's time:
-//   * the sinc's denominators sin(pi f), |pi f| <= pi/2, come from a
-//     truncated Taylor series (sin_half_period) instead of the general
-//     sine with its range reduction; their argument is unchanged;
+// The Miller indices and the fractional offsets are evaluated in the order the
+// definition is written, so they are bitwise those of any other uncontracted
+// FP64 evaluation (the sinc at N = 200 multiplies h's rounding by pi N).  The
+// rest, which is not sensitive to the last bits, is arranged for the FP64
+// pipe, which on this part issues at 1/64 of the FP32 rate and so sets the
+// kernel's time:
+//   * the nearest lattice point comes from an addition that rounds up at the
+//     units' place; its integer is then the low word of the sum (a ceil and
+//     three conversions less);
+//   * the sinc's sines are sin(pi x) for |x| <= 1/2 from one polynomial
+//     (sinpi_half); the numerator's argument N f is reduced exactly by one
+//     FMA, and its sign drops out;
 //   * the Gaussian exponent (summed in explicit FMAs) and the Lagrange
 //     weights multiply by 1/0.63 and 1/6 instead of dividing, and the sinc
-//     divides once per step, not once per axis (an IEEE division is a
-//     sequence of about ten FP64 instructions; the result moves by an ulp
-//     or two);
+//     divides once per step, by a reciprocal from the hardware estimate and
+//     one cubic correction (an IEEE division is a sequence of about ten FP64
+//     instructions; the result moves by an ulp or two);
 //   * the tricubic sum is nested per axis in explicit FMAs, sum_i w_i
 //     sum_j w_j sum_k w_k F_ijk: 84 FP64 operations instead of 256 for the
 //     flat triple product sum (the rounding differs at the 1e-15 level);
@@ -26,6 +29,9 @@
 //     from the nearest lattice point instead of a floor;
 //   * the step's weight, capture, polarization and solid angle are one
 //     factor per source.
+// 307 x 211 pixels of the precision sweep at N = 200: 42.3 -> 33.3 ms with the
+// lattice point, sines and reciprocal above (about 170 -> 110 FP64-pipe
+// instructions per sinc step, the pipe 85 % busy).
 // Only loop invariants are hoisted (pixel position, solid angle, capture
 // fraction per subpixel/layer; scattering vector, polarization and that
 // factor per source).  The rotated axes and the source table are staged in
@@ -38,59 +44,93 @@ __device__ __forceinline__ double dot3d(const double *a, const double *b) {
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
-// sin(x) for |x| <= pi/2 from its Taylor series through x^21/21!: the
-// remainder is below (pi/2)^23/23! < 2e-18, the coefficients are the
-// reciprocal factorials rounded once (every factorial up to 21! is exact
-// in FP64), and x + x^3 p with p by Horner in x^2 keeps the error to a few
-// ulp; 12 FP64 operations, no range reduction (the sinc's denominators
-// have |pi f| <= pi/2)
-__device__ __forceinline__ double sin_half_period(double x) {
-  const double x2 = x * x;
-  double p = 1.0 / 51090942171709440000.0;  // 1/21!
-  p = fma(p, x2, -1.0 / 121645100408832000.0);
-  p = fma(p, x2, 1.0 / 355687428096000.0);
-  p = fma(p, x2, -1.0 / 1307674368000.0);
-  p = fma(p, x2, 1.0 / 6227020800.0);
-  p = fma(p, x2, -1.0 / 39916800.0);
-  p = fma(p, x2, 1.0 / 362880.0);
-  p = fma(p, x2, -1.0 / 5040.0);
-  p = fma(p, x2, 1.0 / 120.0);
-  p = fma(p, x2, -1.0 / 6.0);
-  return fma(x * x2, p, x);
+// sin(pi x) for |x| <= 1/2: x p(x^2), p the degree-8 minimax polynomial of
+// sin(pi x)/x in x^2 on [0, 1/4] (Remez exchange in 60 digits; relative error
+// 2.6e-19, 4.0e-17 with the coefficients rounded to FP64): 10 FP64
+// operations and an ulp or two of rounding
+__device__ __forceinline__ double sinpi_half(double x) {
+  const double t = x * x;
+  double p = fma(7.6947273844559142e-07, t, -2.1903185429548639e-05);
+  p = fma(p, t, 0.00046629968877916672);
+  p = fma(p, t, -0.0073704304787646294);
+  p = fma(p, t, 0.082145886569893037);
+  p = fma(p, t, -0.5992645293187383);
+  p = fma(p, t, 2.550164039877294);
+  p = fma(p, t, -5.1677127800499694);
+  p = fma(p, t, 3.1415926535897931);
+  return x * p;
 }
 
+// 1.5 * 2^52: adding it rounds to an integer, which the low word then holds
+constexpr double kRoundBias = 6755399441055744.0;
+
+// The lattice point n nearest to h (ties down: ceil(h - 1/2)) and the offset
+// f = h - n (exact)
+__device__ __forceinline__ void nearest_f64(const double h[3], long long n[3],
+                                            double f[3]) {
+  // |h| < 2^30 on all axes (integer compares of the high words; a double
+  // compare is one more FP64-pipe instruction)
+  const int big = max(max(__double2hiint(h[0]) & 0x7fffffff,
+                          __double2hiint(h[1]) & 0x7fffffff),
+                      __double2hiint(h[2]) & 0x7fffffff);
+  if (big < 0x41d00000) {
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const double s = __dadd_ru(h[x] - 0.5, kRoundBias);
+      n[x] = __double2loint(s);
+      f[x] = h[x] - (s - kRoundBias);
+    }
+  } else {
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const double c = ceil(h[x] - 0.5);
+      n[x] = (long long)c;
+      f[x] = h[x] - c;
+    }
+  }
+}
+
+// F_latt (up to its sign) at the fractional offset f
 template <int SHAPE>
 __device__ __forceinline__ double flatt_f64(const SpotArgs &a,
-                                            const double h[3], double n[3]) {
-  // sinc: the three numerators and the three denominators multiplied
-  // separately and divided once (a division is a sequence of about ten
-  // FP64 instructions); an axis with |f| below 1e-100 (f = 0 in practice:
-  // h is a sum of products of order-one values) contributes its limit N,
-  // so the product of denominators cannot underflow
+                                            const double f[3]) {
+  // sinc: sin(pi N h)/sin(pi h) = +-sin(pi N f)/sin(pi f); the three
+  // numerators and the three denominators are multiplied separately and
+  // divided once; an axis with |f| below 1e-100 (f = 0 in practice: h is a
+  // sum of products of order-one values) contributes its limit N, so the
+  // product of denominators cannot underflow
   double num = 1.0, den = 1.0, rad2 = 0.0;
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
-    n[x] = ceil(h[x] - 0.5);  // nearest integer, ties down
-    double fr = h[x] - n[x];
     if (SHAPE == 0) {
-      // sin(pi N h)/sin(pi h) = +-sin(pi N f)/sin(pi f); the sign drops out
-      // |f| < 1e-100 as an integer compare of the magnitudes' bit patterns
-      // (ordered like the values for non-negative doubles; a double
-      // compare is one more FP64-pipe instruction)
-      if ((__double_as_longlong(fr) & 0x7fffffffffffffffll) <
-          __double_as_longlong(1e-100)) {
-        num *= a.N64[x];
+      const double N = a.N64[x];
+      double sn;
+      if (N < 1e12) {
+        // r = N f - round(N f), exact
+        const double m = fma(N, f[x], kRoundBias) - kRoundBias;
+        sn = sinpi_half(fma(N, f[x], -m));
       } else {
-        num *= sin(M_PI * a.N64[x] * fr);
-        den *= sin_half_period(M_PI * fr);
+        sn = sin(M_PI * N * f[x]);
       }
+      // |f| < 1e-100 from the high word of its bit pattern
+      const bool zero =
+          (__double2hiint(f[x]) & 0x7fffffff) < __double2hiint(1e-100);
+      sn = zero ? N : sn;
+      const double sd = zero ? 1.0 : sinpi_half(f[x]);
+      num = x ? num * sn : sn;
+      den = x ? den * sd : sd;
     } else {
       // sum N^2 f^2 / 0.63 in explicit FMAs (N^2 / 0.63 is loop-invariant)
-      rad2 = fma(a.N64[x] * a.N64[x] * (1.0 / 0.63) * fr, fr, rad2);
+      rad2 = fma(a.N64[x] * a.N64[x] * (1.0 / 0.63) * f[x], f[x], rad2);
     }
   }
   if (SHAPE == 1) return a.N64[0] * a.N64[1] * a.N64[2] * exp(-rad2);
-  return num / den;
+  // 1 / den: the hardware's estimate (20 bits) and one step of third order
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(den));
+  const double e = fma(-den, r, 1.0);
+  r = fma(r, fma(e, e, e), r);
+  return num * r;
 }
 
 __device__ __forceinline__ bool in_table(const SpotArgs &a, long long i,
@@ -126,28 +166,27 @@ __device__ __forceinline__ double tricubic_sum(const SpotArgs &a,
   return sum;
 }
 
-// F_cell at h, whose nearest lattice point is n (ties down, flatt_f64):
-// the cell's first node is floor(h) = n - 1 where h < n, else n, so no
-// floor and no second float-to-integer conversion per axis are needed
+// F_cell at the offset f from lattice point n (ties down, nearest_f64): the
+// cell's first node is floor(h) = n - 1 where f < 0, else n, so no floor and
+// no second float-to-integer conversion per axis are needed
 template <int INTERP>
 __device__ __forceinline__ double fcell_f64(const SpotArgs &a,
-                                            const double h[3],
-                                            const double n[3]) {
+                                            const double f[3],
+                                            const long long n[3]) {
   long long nn[3];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) nn[c] = (long long)n[c] - a.hmin[c];
+  for (int c = 0; c < 3; ++c) nn[c] = n[c] - a.hmin[c];
   if (INTERP == 1) {
     long long fl[3];
     double x[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      // h - n is exact (h and n lie within 1/2), and so is h - floor(h)
-      // for h < n: (h - n) + 1 holds no bit below h's last one
-      const double fr = h[c] - n[c];
-      // f < 0 from the sign bit (an integer test; f = h - n is never -0)
-      const bool below = __double_as_longlong(fr) < 0;
+      // f = h - n is exact (h and n lie within 1/2), and so is h - floor(h)
+      // for f < 0: f + 1 holds no bit below h's last one
+      // f < 0 from the sign bit (an integer test; f is never -0)
+      const bool below = __double_as_longlong(f[c]) < 0;
       fl[c] = nn[c] - (below ? 1 : 0);
-      x[c] = below ? fr + 1.0 : fr;
+      x[c] = below ? f[c] + 1.0 : f[c];
     }
     if (in_table(a, fl[0] - 1, fl[1] - 1, fl[2] - 1) &&
         in_table(a, fl[0] + 2, fl[1] + 2, fl[2] + 2)) {
@@ -199,9 +238,11 @@ cudaError_t build_f64_table(const float *F, long long n, double *F64t,
   return cudaGetLastError();
 }
 
+// 2^lsplit neighbouring lanes share a pixel (f64_split): 2^lk of them take
+// every 2^lk-th source, each with the orientations of its residue
 template <int SHAPE, int INTERP>
 __global__ void __launch_bounds__(kTileThreads, 4)
-    spots_f64_kernel(SpotArgs a) {
+    spots_f64_kernel(SpotArgs a, int lsplit, int lk) {
   extern __shared__ double sm[];
   double *s_ax = sm;
   double *s_src = sm + a.PM * 9;
@@ -210,20 +251,26 @@ __global__ void __launch_bounds__(kTileThreads, 4)
     s_src[i] = a.src64[i];
   __syncthreads();
 
-  long long item = a.pixlist ? (long long)blockIdx.x * blockDim.x + threadIdx.x
-                             : (long long)blockIdx.x;
-  long long gp;
-  int q, s, f;
-  if (!map_pixel(a, item, threadIdx.x, gp, q, s, f)) return;
+  const long long slot =
+      ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> lsplit;
+  const int part = threadIdx.x & ((1 << lsplit) - 1);
+  const int k0 = part & ((1 << lk) - 1), dk = 1 << lk, m0 = part >> lk,
+            dm = 1 << (lsplit - lk);
+  long long gp = 0;
+  int q = 0, s = 0, fp = 0;
+  const bool ok =
+      a.pixlist ? map_pixel(a, slot, 0, gp, q, s, fp)
+                : map_pixel(a, slot / kTileThreads,
+                            (int)(slot % kTileThreads), gp, q, s, fp);
   const DevPanel &P = a.panels[q];
   const double px = P.px;
   const int os = a.os;
   double acc = 0.0;
-  for (int i = 0; i < os; ++i) {
+  for (int i = 0; i < (ok ? os : 0); ++i) {
     for (int j = 0; j < os; ++j) {
       for (int t = 0; t < a.T; ++t) {
-        double cf = (f + (i + 0.5) / os) * px, cs = (s + (j + 0.5) / os) * px,
-               cn = t * a.dt;
+        double cf = (fp + (i + 0.5) / os) * px,
+               cs = (s + (j + 0.5) / os) * px, cn = t * a.dt;
         double pos[3], d[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
@@ -238,7 +285,7 @@ __global__ void __launch_bounds__(kTileThreads, 4)
           double L = a.atten * dot3d(d, P.ndir);
           cap = exp(-t * a.dt / L) - exp(-(t + 1) * a.dt / L);
         }
-        for (int k = 0; k < a.S; ++k) {
+        for (int k = k0; k < a.S; k += dk) {
           const double *src = s_src + k * SRC64_STRIDE;
           const double lam = src[SRC64_LAM];
           const double *dir = src + SRC64_DIR;
@@ -251,28 +298,50 @@ __global__ void __launch_bounds__(kTileThreads, 4)
           double pol = 0.5 * (1.0 + c2 * c2 - a.kahn64 * (x * x - y * y));
           // the step's factors that do not depend on phi x mosaic
           const double wcpo = src[SRC64_W] * cap * pol * omega;
-          for (int pm = 0; pm < a.PM; ++pm) {
+          for (int pm = m0; pm < a.PM; pm += dm) {
             const double *A = s_ax + pm * 9;
             double h[3] = {dot3d(A, Sv), dot3d(A + 3, Sv), dot3d(A + 6, Sv)};
-            double n[3];
-            double fl = flatt_f64<SHAPE>(a, h, n);
-            double fc = fcell_f64<INTERP>(a, h, n);
-            const double a_ = fc * fl;
-            acc += a_ * a_ * wcpo;
+            long long n[3];
+            double f[3];
+            nearest_f64(h, n, f);
+            const double a_ =
+                fcell_f64<INTERP>(a, f, n) * flatt_f64<SHAPE>(a, f);
+            acc = fma(a_ * a_, wcpo, acc);
           }
         }
       }
     }
   }
-  a.image[nb_idx(a.check, NB_SITE_IMAGE, gp, a.npix)] += a.prefactor * acc;
+  for (int o = 1; o < (1 << lsplit); o <<= 1)
+    acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (ok && part == 0)
+    a.image[nb_idx(a.check, NB_SITE_IMAGE, gp, a.npix)] += a.prefactor * acc;
+}
+
+// How many lanes share a pixel (log2).  The FP64 unit is a scheduler's own, so
+// a launch takes as long as the scheduler with the most warps: 307 x 211
+// pixels one per lane are 3.6 warps for each of the 608 schedulers, so 4 for
+// most.  Parts of at least 128 steps keep the repeated geometry (~130 FP64
+// instructions against 110 per sinc step) below 1 %, and a rule on the shot
+// alone keeps a pixel's value the same in every launch.  That shot (sinc, 2000
+// steps): 33.3 -> 30.2 ms.
+static int f64_split(const SpotArgs &a) {
+  int l = 0;
+  while (l < 5 && ((long long)a.S * a.PM) >> (l + 1) >= 128) ++l;
+  return l;
 }
 
 cudaError_t launch_spots_f64(const SpotArgs &a, cudaStream_t st) {
   size_t smem = (size_t)(a.PM * 9 + a.S * SRC64_STRIDE) * sizeof(double);
-  long long blocks = a.pixlist ? (a.n_list + kTileThreads - 1) / kTileThreads
-                               : a.n_tiles;
+  const int lsplit = f64_split(a);
+  int lk = 0;  // as many sources side by side as there are
+  while (lk < lsplit && 2 << lk <= a.S) ++lk;
+  const long long pixels =
+      a.pixlist ? a.n_list : (long long)a.n_tiles * kTileThreads;
+  const long long blocks =
+      ((pixels << lsplit) + kTileThreads - 1) / kTileThreads;
   if (blocks <= 0) return cudaSuccess;
-  void (*kern)(SpotArgs) = nullptr;
+  void (*kern)(SpotArgs, int, int) = nullptr;
   int key = a.shape * 2 + a.interp;
   switch (key) {
     case 0: kern = spots_f64_kernel<0, 0>; break;
@@ -283,7 +352,7 @@ cudaError_t launch_spots_f64(const SpotArgs &a, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)blocks, kTileThreads, smem, st>>>(a);
+  kern<<<(unsigned)blocks, kTileThreads, smem, st>>>(a, lsplit, lk);
   return cudaGetLastError();
 }
 
@@ -513,10 +582,12 @@ __global__ void __launch_bounds__(kF64Threads, 4)
                   const double *A = s_ax + (c >> 8) * 9;
                   const double h[3] = {dot3d(A, Sv), dot3d(A + 3, Sv),
                                        dot3d(A + 6, Sv)};
-                  double n[3];
-                  const double fl = flatt_f64<1>(a, h, n);
-                  const double a_ = fcell_f64<INTERP>(a, h, n) * fl;
-                  acc += a_ * a_ * s1.y;
+                  long long n[3];
+                  double f[3];
+                  nearest_f64(h, n, f);
+                  const double a_ =
+                      fcell_f64<INTERP>(a, f, n) * flatt_f64<1>(a, f);
+                  acc = fma(a_ * a_, s1.y, acc);
                 }
                 head += cnt;
                 __syncwarp();
