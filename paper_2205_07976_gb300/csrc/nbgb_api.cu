@@ -97,8 +97,17 @@ struct nb_sim {
   int os = 1, T = 1;
   double thick = 0, atten = 0;
   // device
-  DevBuf d_panels, d_ax64, d_axh, d_axl, d_src64, d_src32, d_divh, d_divl,
-      d_F, d_image, d_list, d_tmp, d_stats, d_work, d_srcq, d_check;
+  DevBuf d_panels, d_tab, d_divh, d_divl, d_F, d_image, d_list, d_tmp,
+      d_stats, d_check;
+  // the shot's tables: staged one after another in h_tab and uploaded to
+  // d_tab in one copy (six small copies took 15 us of a 57 us call); byte
+  // offsets of each
+  std::vector<unsigned char> h_tab;
+  size_t o_ax64 = 0, o_axh = 0, o_axl = 0, o_src64 = 0, o_src32 = 0,
+         o_srcq = 0, o_rot = 0;
+  const void *tab(size_t off) const {
+    return (const unsigned char *)d_tab.p + off;
+  }
   float sinc_qG = 0.f;  // grid of G for the sinc fast path (0: off)
   float sinc_dq[2] = {0.f, 0.f};  // range of the sources' delta on its grid
   int variant = NB_VARIANT_AUTO;
@@ -111,7 +120,7 @@ struct nb_sim {
   bool have_params = false;
   double pU[9] = {0}, pcell[3] = {0}, prot[3] = {0};
   double daxes[6][9];  // d(lab axes)/d(tx, ty, tz, a, b, c)
-  DevBuf d_rot, d_part, d_grad, d_F4, d_C4, d_F64t;
+  DevBuf d_part, d_grad, d_F4, d_C4, d_F64t;
   bool F4_valid = false, C4_valid = false, F64_valid = false;
   bool fmax_valid = false;  // the largest |F|, behind the counters
   int has_div = 0;
@@ -433,30 +442,39 @@ static int upload_tables(nb_sim *s) {
         }
       }
   }
-  cudaError_t e;
-  if ((e = s->d_ax64.ensure(ax.size() * 8)) != cudaSuccess ||
-      (e = s->d_axh.ensure(axh.size() * 4)) != cudaSuccess ||
-      (e = s->d_axl.ensure(axl.size() * 4)) != cudaSuccess ||
-      (e = s->d_src64.ensure(src64.size() * 8)) != cudaSuccess ||
-      (e = s->d_src32.ensure(src32.size() * 4)) != cudaSuccess)
+  std::vector<float> rot;
+  if (s->have_params) {
+    // the rotation of every orientation, row-major: its columns are the
+    // rotated unit vectors
+    const double eye[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
+    std::vector<double> t;
+    build_axes_of(s, eye, t);
+    rot.resize(t.size());
+    for (int pm = 0; pm < PM; ++pm)
+      for (int v = 0; v < 3; ++v)
+        for (int r = 0; r < 3; ++r)
+          rot[(size_t)pm * 9 + 3 * r + v] = (float)t[(size_t)pm * 9 + 3 * v + r];
+  }
+  s->h_tab.clear();
+  auto put = [&](const void *p, size_t bytes) {
+    const size_t off = (s->h_tab.size() + 255) & ~(size_t)255;
+    s->h_tab.resize(off + bytes);
+    if (bytes) std::memcpy(s->h_tab.data() + off, p, bytes);
+    return off;
+  };
+  s->o_ax64 = put(ax.data(), ax.size() * 8);
+  s->o_axh = put(axh.data(), axh.size() * 4);
+  s->o_axl = put(axl.data(), axl.size() * 4);
+  s->o_src64 = put(src64.data(), src64.size() * 8);
+  s->o_src32 = put(src32.data(), src32.size() * 4);
+  s->o_srcq = put(srcq.data(), srcq.size() * 4);
+  s->o_rot = put(rot.data(), rot.size() * 4);
+  cudaError_t e = s->d_tab.ensure(s->h_tab.size());
+  if (e != cudaSuccess)
     return fail(s, NB_ENOMEM, std::string("device tables: ") +
                                   cudaGetErrorString(e));
-  cudaMemcpyAsync(s->d_ax64.p, ax.data(), ax.size() * 8,
+  cudaMemcpyAsync(s->d_tab.p, s->h_tab.data(), s->h_tab.size(),
                   cudaMemcpyHostToDevice, s->stream);
-  cudaMemcpyAsync(s->d_axh.p, axh.data(), axh.size() * 4,
-                  cudaMemcpyHostToDevice, s->stream);
-  cudaMemcpyAsync(s->d_axl.p, axl.data(), axl.size() * 4,
-                  cudaMemcpyHostToDevice, s->stream);
-  cudaMemcpyAsync(s->d_src64.p, src64.data(), src64.size() * 8,
-                  cudaMemcpyHostToDevice, s->stream);
-  cudaMemcpyAsync(s->d_src32.p, src32.data(), src32.size() * 4,
-                  cudaMemcpyHostToDevice, s->stream);
-  if (!srcq.empty()) {
-    if ((e = s->d_srcq.ensure(srcq.size() * 4)) != cudaSuccess)
-      return fail(s, NB_ENOMEM, "source grid table");
-    cudaMemcpyAsync(s->d_srcq.p, srcq.data(), srcq.size() * 4,
-                    cudaMemcpyHostToDevice, s->stream);
-  }
   if (s->has_div) {
     if ((e = s->d_divh.ensure(divh.size() * 4)) != cudaSuccess ||
         (e = s->d_divl.ensure(divl.size() * 4)) != cudaSuccess)
@@ -464,22 +482,6 @@ static int upload_tables(nb_sim *s) {
     cudaMemcpyAsync(s->d_divh.p, divh.data(), divh.size() * 4,
                     cudaMemcpyHostToDevice, s->stream);
     cudaMemcpyAsync(s->d_divl.p, divl.data(), divl.size() * 4,
-                    cudaMemcpyHostToDevice, s->stream);
-  }
-  if (s->have_params) {
-    // the rotation of every orientation, row-major: its columns are the
-    // rotated unit vectors
-    const double eye[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
-    std::vector<double> t;
-    build_axes_of(s, eye, t);
-    std::vector<float> rot(t.size());
-    for (int pm = 0; pm < PM; ++pm)
-      for (int v = 0; v < 3; ++v)
-        for (int r = 0; r < 3; ++r)
-          rot[(size_t)pm * 9 + 3 * r + v] = (float)t[(size_t)pm * 9 + 3 * v + r];
-    if ((e = s->d_rot.ensure(rot.size() * 4)) != cudaSuccess)
-      return fail(s, NB_ENOMEM, "rotation table");
-    cudaMemcpyAsync(s->d_rot.p, rot.data(), rot.size() * 4,
                     cudaMemcpyHostToDevice, s->stream);
   }
   // pageable copies are staged before return; check the queue is healthy
@@ -501,9 +503,9 @@ static void fill_args(const nb_sim *s, SpotArgs &a) {
   a.thickness = s->thick;
   a.atten = s->atten;
   a.PM = s->n_phi * s->n_mosaic;
-  a.ax64 = (const double *)s->d_ax64.p;
-  a.axh = (const float *)s->d_axh.p;
-  a.axl = (const float *)s->d_axl.p;
+  a.ax64 = (const double *)s->tab(s->o_ax64);
+  a.axh = (const float *)s->tab(s->o_axh);
+  a.axl = (const float *)s->tab(s->o_axl);
   for (int i = 0; i < 3; ++i) {
     a.N64[i] = s->N[i];
     a.N[i] = (float)s->N[i];
@@ -522,8 +524,8 @@ static void fill_args(const nb_sim *s, SpotArgs &a) {
   a.defF = (float)s->defF;
   a.defF64 = s->defF;
   a.S = s->n_src;
-  a.src64 = (const double *)s->d_src64.p;
-  a.src32 = (const float *)s->d_src32.p;
+  a.src64 = (const double *)s->tab(s->o_src64);
+  a.src32 = (const float *)s->tab(s->o_src32);
   a.u0 = s->u0;
   split_ff(s->u0, a.u0h, a.u0l);
   pol_basis(s->dirs.data(), s->evec, a.e0, a.b0);
@@ -532,7 +534,7 @@ static void fill_args(const nb_sim *s, SpotArgs &a) {
   a.has_div = s->has_div;
   a.divh = (const float *)s->d_divh.p;
   a.divl = (const float *)s->d_divl.p;
-  a.srcq = s->sinc_qG > 0.f ? (const float *)s->d_srcq.p : nullptr;
+  a.srcq = s->sinc_qG > 0.f ? (const float *)s->tab(s->o_srcq) : nullptr;
   a.sinc_qG = a.srcq ? s->sinc_qG : 0.f;
   a.sinc_dq[0] = s->sinc_dq[0];
   a.sinc_dq[1] = s->sinc_dq[1];
@@ -625,14 +627,12 @@ int nb_free(nb_sim *sim) {
   {
     DeviceGuard g(sim->device);
     cudaStreamSynchronize(sim->stream);
-    DevBuf *bufs[] = {&sim->d_panels, &sim->d_ax64, &sim->d_axh,
-                      &sim->d_axl,    &sim->d_src64, &sim->d_src32,
-                      &sim->d_divh,   &sim->d_divl,  &sim->d_F,
-                      &sim->d_image,  &sim->d_list,  &sim->d_tmp,
-                      &sim->d_stats,  &sim->d_work,  &sim->d_srcq,  &sim->d_check,  &sim->d_rot,
-                      &sim->d_part,   &sim->d_grad,  &sim->d_F4,
-                      &sim->d_C4,     &sim->d_F64t,  &sim->d_bg64,
-                      &sim->d_bg32,   &sim->d_bgrng};
+    DevBuf *bufs[] = {&sim->d_panels, &sim->d_tab,   &sim->d_divh,
+                      &sim->d_divl,   &sim->d_F,     &sim->d_image,
+                      &sim->d_list,   &sim->d_tmp,   &sim->d_stats,
+                      &sim->d_check,  &sim->d_part,  &sim->d_grad,
+                      &sim->d_F4,     &sim->d_C4,    &sim->d_F64t,
+                      &sim->d_bg64,   &sim->d_bg32,  &sim->d_bgrng};
     for (DevBuf *b : bufs) b->release();
   }
   delete sim;
@@ -995,8 +995,8 @@ static int launch(nb_sim *s, const long long *dev_list, long long n_list) {
     a.sinc_qG = 0.f;
   }
   // counters: [0] evaluated terms, [1..3] the warp kernel's pairs,
-  // intervals and source blocks, [4] the next pixel of the FP64 warp
-  // kernel; behind them the largest |F|
+  // intervals and source blocks, [4] the next pixel of the warp kernels;
+  // behind them the largest |F|
   cudaError_t e = s->d_stats.ensure(6 * sizeof(unsigned long long));
   if (e != cudaSuccess) return fail(s, NB_ENOMEM, "statistics counters");
   e = cudaMemsetAsync(s->d_stats.p, 0, 5 * sizeof(unsigned long long),
@@ -1028,13 +1028,7 @@ static int launch(nb_sim *s, const long long *dev_list, long long n_list) {
   } else if (warp_variant) {
     ensure_cell_polynomials(s);
     a.C4 = s->C4_valid ? (const float4 *)s->d_C4.p : nullptr;
-    e = s->d_work.ensure(sizeof(unsigned long long));
-    if (e != cudaSuccess) return fail(s, NB_ENOMEM, "work counter");
-    e = cudaMemsetAsync(s->d_work.p, 0, sizeof(unsigned long long),
-                        s->stream);
-    if (e == cudaSuccess)
-      e = nbgb::launch_spots_split(a, (unsigned long long *)s->d_work.p,
-                                   s->sm_count, s->stream);
+    e = nbgb::launch_spots_split(a, a.stats + 4, s->sm_count, s->stream);
   } else {
     e = nbgb::launch_spots_mixed(a, s->precision, s->stream);
   }
@@ -1162,7 +1156,7 @@ int nb_adjoint(nb_sim *s, const double *dLdI, double grad[10],
   if (e != cudaSuccess) return fail(s, NB_ENOMEM, "gradient scratch");
   double kc = nbgb::kElectronRadius * nbgb::kElectronRadius * s->fluence /
               ((double)s->os * s->os * s->n_mosaic * s->n_phi);
-  e = nbgb::launch_adjoint(a, (const float *)s->d_rot.p, dLdI, gradF,
+  e = nbgb::launch_adjoint(a, (const float *)s->tab(s->o_rot), dLdI, gradF,
                            (double *)s->d_part.p, kc, s->scale,
                            (double *)s->d_grad.p, s->sm_count, s->stream);
   double sums[nbgb::kAdjointSums] = {0};
