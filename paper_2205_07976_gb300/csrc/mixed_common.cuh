@@ -41,6 +41,28 @@ __device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
   return upk2(d);
 }
 
+// The same on register pairs, for loops whose operands are pairs made once (a
+// float2 of twice the same value is otherwise put together at every use)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 splat2(float v) {
+  return pk2(make_float2(v, v));
+}
+__device__ __forceinline__ f32x2 ffma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 fadd2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 fmul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 __device__ __forceinline__ double dot3d_m(const double *a, const double *b) {
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }

@@ -9,12 +9,11 @@
 //   submit  -> FIFO queue (inputs copied, tables built on the host)
 //   step    -> admit while a slot and room in the image pool exist (first
 //              fit; a blocked head request stops bypassing after 8 steps);
-//              cut the active requests into work items (128 pixels for the
-//              thread kernel, 64 for the warp kernel) up to a pixel-step
-//              budget: half shared equally by the running requests, the
+//              cut the active requests into work items of 128 pixels up to a
+//              pixel-step budget: half shared equally by the running requests, the
 //              rest to the oldest first; replay one of two CUDA graphs
 //              (work list upload from its own pinned buffer, counter reset,
-//              the two persistent kernels); then wait for the step queued
+//              the persistent kernels); then wait for the step queued
 //              by the previous call, so the GPU runs one step while the host
 //              prepares the next; requests whose last item ran in a
 //              finished step are complete
@@ -46,7 +45,10 @@ namespace nbgb {
 constexpr int kServeMaxPM = 64;
 constexpr int kServeMaxSrc = 128;
 constexpr int kServeItemPixels = kTileThreads;  // one pixel per thread
-constexpr int kServeWarpItemPixels = 64;  // warp kernel: 16 pixels per warp
+// the warp kernels: 32 pixels per warp (of 48 requests with up to 4e6 pixels:
+// 64 pixels 28.0 ms, 128 26.9, 256 27.2; as parallel branches of the graph
+// instead of one kernel after another, 28.9, 27.6 and 29.5)
+constexpr int kServeWarpItemPixels = 128;
 constexpr int kServeMaxItems = 16384;
 
 struct SlotParams {
@@ -119,8 +121,9 @@ __global__ void __launch_bounds__(kTileThreads, 4)
 // run one warp per pixel (tricubic lookup, >= 8 subpixel x mosaic items):
 // each work item stages its request's tables once, then each warp sums its
 // pixels with the same device function as the stand-alone kernel.
-template <int INTERP, bool FF>
-__global__ void __launch_bounds__(kSplitThreads, 5)
+template <int INTERP, bool FF, int FORM>
+__global__ void __launch_bounds__(kSplitThreads, FORM == kLines ? kLineBlocks
+                                                                : 5)
     serve_warp_kernel(SpotArgs base, const SlotParams *slots,
                       const WorkList *wl, unsigned *counter, double *pool) {
   extern __shared__ float sms[];
@@ -163,7 +166,7 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
       __syncwarp();
       for (int bi = 0; bi < nb; ++bi) {
         const long long p = w.first + warp + (long long)(i0 + bi) * kSplitWarps;
-        const double v = split_sum<INTERP, 0>(
+        const double v = split_sum<INTERP, 0, FORM>(
             base, b, unit + bi * U * kUnitFloats, cnt);
         if (lane == 0) pool[sp.img_off + p] = sp.prefactor * v;
       }
@@ -171,6 +174,22 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
     }
     __syncthreads();  // the tables may be restaged for the next item
   }
+}
+
+// the warp kernels of a server's requests that are summed pair by pair, and
+// line by line (split_form)
+using ServeKernel = void (*)(SpotArgs, const SlotParams *, const WorkList *,
+                             unsigned *, double *);
+template <bool FF>
+static ServeKernel pick_serve_warp(const SpotArgs &a, bool lines) {
+  if (lines) return serve_warp_kernel<1, FF, kLines>;
+  return split_form(a, 1, 1) == kPairsEarly
+             ? serve_warp_kernel<1, FF, kPairsEarly>
+             : serve_warp_kernel<1, FF, kPairs>;
+}
+static ServeKernel serve_warp(const SpotArgs &a, bool lines) {
+  return split_ff(a) ? pick_serve_warp<true>(a, lines)
+                     : pick_serve_warp<false>(a, lines);
 }
 
 size_t serve_warp_smem_bytes() {
@@ -202,6 +221,8 @@ struct Buf {
   }
 };
 
+constexpr int kKinds = 3;  // kinds of requests (Request::kind)
+
 struct Request {
   long long id;
   SlotParams params;  // host copy (img_off set at admission)
@@ -212,7 +233,9 @@ struct Request {
   long long pool_off = -1;
   int state = NB_REQ_QUEUED;
   int blocked_steps = 0;
-  bool warp = false;  // computed by the warp-per-pixel kernel
+  // 0: computed by the thread-per-pixel kernel, 1: by the warp-per-pixel
+  // kernel pair by pair, 2: line by line
+  int kind = 0;
 };
 
 }  // namespace
@@ -236,12 +259,12 @@ struct nb_server {
   int hmin[3], hn[3];
   double defF = 0;
   double fluence = 0, kahn = 0, evec[3] = {1, 0, 0}, dir[3] = {0, 0, 1};
-  Buf d_F, d_F4, d_C4, d_panel, d_slots, d_pool, d_work, d_work_w, d_counter;
-  // two host work-list buffers, each with its graph: the next step is
-  // built and queued while the previous one runs
-  WorkList *h_work[2] = {nullptr, nullptr};    // pinned: thread-kernel items
-  WorkList *h_work_w[2] = {nullptr, nullptr};  // pinned: warp-kernel items
-  int blocks_w = 0;
+  Buf d_F, d_F4, d_C4, d_panel, d_slots, d_pool, d_work, d_counter;
+  // two host buffers of work lists (pinned, one list per kind of request),
+  // each with its graph: the next step is built and queued while the previous
+  // one runs
+  WorkList *h_work[2] = {nullptr, nullptr};
+  int blocks_w[2] = {0, 0};  // of the warp kernels, pairs and lines
   size_t smem_w = 0;
   nbgb::SpotArgs base;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -306,32 +329,28 @@ static cudaStream_t stream_of(const nb_server *s, int b) {
 }
 
 // The graph of one step from host buffer b, on stream_of(b): its work
-// lists to its own device copies, its counters reset, the two persistent
+// lists to its own device copies, its counters reset, the persistent
 // kernels.
 static int build_graph(nb_server *s, int b) {
   cudaStream_t st = stream_of(s, b);
   cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return sfail(s, NB_ECUDA, "graph capture begin");
-  WorkList *dw = (WorkList *)s->d_work.p + b;
-  WorkList *dww = (WorkList *)s->d_work_w.p + b;
-  unsigned *ctr = (unsigned *)s->d_counter.p + 2 * b;
-  cudaMemcpyAsync(dw, s->h_work[b], sizeof(WorkList), cudaMemcpyHostToDevice,
-                  st);
-  cudaMemcpyAsync(dww, s->h_work_w[b], sizeof(WorkList),
+  WorkList *dw = (WorkList *)s->d_work.p + kKinds * b;
+  unsigned *ctr = (unsigned *)s->d_counter.p + kKinds * b;
+  cudaMemcpyAsync(dw, s->h_work[b], kKinds * sizeof(WorkList),
                   cudaMemcpyHostToDevice, st);
-  cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned), st);
-  void (*kern)(nbgb::SpotArgs, const SlotParams *, const WorkList *,
-               unsigned *, double *) =
-      s->interp ? nbgb::serve_kernel<1> : nbgb::serve_kernel<0>;
-  kern<<<s->blocks, nbgb::kTileThreads, 0, st>>>(
-      s->base, (const SlotParams *)s->d_slots.p, dw, ctr,
-      (double *)s->d_pool.p);
-  if (s->interp == NB_INTERP_TRICUBIC) {
-    auto warp_kern = nbgb::split_ff(s->base) ? nbgb::serve_warp_kernel<1, true>
-                                             : nbgb::serve_warp_kernel<1, false>;
-    warp_kern<<<s->blocks_w, nbgb::kSplitThreads, s->smem_w, st>>>(
-        s->base, (const SlotParams *)s->d_slots.p, dww, ctr + 1,
-        (double *)s->d_pool.p);
+  cudaMemsetAsync(ctr, 0, kKinds * sizeof(unsigned), st);
+  // the kernel with the longest items first: the last blocks of each leave
+  // SMs to the next one (in the order thread, pairs, lines the batch of 48
+  // requests above took 29.6 instead of 26.9 ms)
+  for (int k = s->interp == NB_INTERP_TRICUBIC ? kKinds - 1 : 0; k >= 0; --k) {
+    const nbgb::ServeKernel kern =
+        k ? nbgb::serve_warp(s->base, k == 2)
+          : s->interp ? nbgb::serve_kernel<1> : nbgb::serve_kernel<0>;
+    kern<<<k ? s->blocks_w[k - 1] : s->blocks,
+           k ? nbgb::kSplitThreads : nbgb::kTileThreads, k ? s->smem_w : 0,
+           st>>>(s->base, (const SlotParams *)s->d_slots.p, dw + k, ctr + k,
+                 (double *)s->d_pool.p);
   }
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(st, &g);
@@ -429,25 +448,18 @@ int nb_server_create(nb_server **out, int device, void *cuda_stream,
             cudaSuccess ||
         s->d_pool.alloc((size_t)s->pool_elems * sizeof(double)) !=
             cudaSuccess ||
-        s->d_work.alloc(2 * sizeof(WorkList)) != cudaSuccess ||
-        s->d_work_w.alloc(2 * sizeof(WorkList)) != cudaSuccess ||
-        s->d_counter.alloc(4 * sizeof(unsigned)) != cudaSuccess ||
-        cudaHostAlloc((void **)&s->h_work[0], sizeof(WorkList),
+        s->d_work.alloc(2 * kKinds * sizeof(WorkList)) != cudaSuccess ||
+        s->d_counter.alloc(2 * kKinds * sizeof(unsigned)) != cudaSuccess ||
+        cudaHostAlloc((void **)&s->h_work[0], kKinds * sizeof(WorkList),
                       cudaHostAllocDefault) != cudaSuccess ||
-        cudaHostAlloc((void **)&s->h_work_w[0], sizeof(WorkList),
-                      cudaHostAllocDefault) != cudaSuccess ||
-        cudaHostAlloc((void **)&s->h_work[1], sizeof(WorkList),
-                      cudaHostAllocDefault) != cudaSuccess ||
-        cudaHostAlloc((void **)&s->h_work_w[1], sizeof(WorkList),
+        cudaHostAlloc((void **)&s->h_work[1], kKinds * sizeof(WorkList),
                       cudaHostAllocDefault) != cudaSuccess) {
       cudaGetLastError();
       rc = sfail(s, NB_ENOMEM, "server buffers");
       break;
     }
-    for (int b = 0; b < 2; ++b) {
-      std::memset(s->h_work[b], 0, sizeof(WorkList));
-      std::memset(s->h_work_w[b], 0, sizeof(WorkList));
-    }
+    for (int b = 0; b < 2; ++b)
+      std::memset(s->h_work[b], 0, kKinds * sizeof(WorkList));
     cudaMemcpy(s->d_F.p, F, nF * 4, cudaMemcpyHostToDevice);
     nbgb::DevPanel P;
     std::memset(&P, 0, sizeof P);
@@ -540,15 +552,15 @@ int nb_server_create(nb_server **out, int device, void *cuda_stream,
     s->blocks = s->sm_count * (per_sm > 0 ? per_sm : 1);
     if (interp == NB_INTERP_TRICUBIC) {
       s->smem_w = nbgb::serve_warp_smem_bytes();
-      auto warp_kern = nbgb::split_ff(a) ? nbgb::serve_warp_kernel<1, true>
-                                         : nbgb::serve_warp_kernel<1, false>;
-      cudaFuncSetAttribute(warp_kern,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)s->smem_w);
-      int per_sm_w = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &per_sm_w, warp_kern, nbgb::kSplitThreads, s->smem_w);
-      s->blocks_w = s->sm_count * (per_sm_w > 0 ? per_sm_w : 1);
+      for (int k = 0; k < 2; ++k) {
+        const nbgb::ServeKernel kern = nbgb::serve_warp(a, k == 1);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)s->smem_w);
+        int per_sm_w = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm_w, kern, nbgb::kSplitThreads, s->smem_w);
+        s->blocks_w[k] = s->sm_count * (per_sm_w > 0 ? per_sm_w : 1);
+      }
     }
     for (int i = max_slots - 1; i >= 0; --i) s->free_slots.push_back(i);
     s->free_ranges[0] = s->pool_elems;
@@ -599,13 +611,11 @@ int nb_server_free(nb_server *s) {
     if (s->done_ev[b]) cudaEventDestroy(s->done_ev[b]);
     if (s->up_ev[b]) cudaEventDestroy(s->up_ev[b]);
     if (s->h_work[b]) cudaFreeHost(s->h_work[b]);
-    if (s->h_work_w[b]) cudaFreeHost(s->h_work_w[b]);
   }
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
   {
     Buf *bufs[] = {&s->d_F,    &s->d_F4,     &s->d_C4,     &s->d_panel,
-                   &s->d_slots, &s->d_pool, &s->d_work, &s->d_work_w,
-                   &s->d_counter};
+                   &s->d_slots, &s->d_pool, &s->d_work, &s->d_counter};
     for (Buf *b : bufs) {
       if (b->p) cudaFree(b->p);
       b->p = nullptr;
@@ -674,9 +684,11 @@ int nb_server_submit(nb_server *s, const double axes[9], const double *umats,
   r.steps_per_pixel =
       (long long)s->os * s->os * s->T * n_src * (long long)n_mosaic;
   // the same choice as nb_add_spots makes for this shot
-  r.warp = s->interp == NB_INTERP_TRICUBIC &&
-           (long long)s->os * s->os * s->T * n_mosaic >= 8 &&
-           s->os * s->os * s->T <= 32;
+  if (s->interp == NB_INTERP_TRICUBIC &&
+      (long long)s->os * s->os * s->T * n_mosaic >= 8 &&
+      s->os * s->os * s->T <= 32)
+    r.kind =
+        nbgb::split_form(s->base, n_mosaic, n_src) == nbgb::kLines ? 2 : 1;
   s->queue.push_back(r.id);
   *request_id = r.id;
   s->reqs.emplace(r.id, std::move(r));
@@ -768,8 +780,8 @@ int nb_server_step(nb_server *s, double timeout_s, int *n_active) {
         act.push_back(&kv.second);
         next0.push_back(kv.second.next);
       }
-    WorkList *wl = s->h_work[s->cur], *ww = s->h_work_w[s->cur];
-    int nt = 0, nw = 0;
+    WorkList *wl = s->h_work[s->cur];
+    int n_items[kKinds] = {0};
     long long used = 0;
     // half of the budget is shared equally by the active requests (at
     // least one work item each, so none starves and a new request is not
@@ -782,9 +794,9 @@ int nb_server_step(nb_server *s, double timeout_s, int *n_active) {
     for (int pass = 0; pass < 2 && used < s->budget; ++pass) {
       for (size_t j = 0; j < act.size() && used < s->budget; ++j) {
         Request &r = *act[j];
-        WorkList *L = r.warp ? ww : wl;
-        int &n = r.warp ? nw : nt;
-        const long long cap = r.warp ? nbgb::kServeWarpItemPixels
+        WorkList *L = wl + r.kind;
+        int &n = n_items[r.kind];
+        const long long cap = r.kind ? nbgb::kServeWarpItemPixels
                                      : nbgb::kServeItemPixels;
         long long mine = 0;  // pixel-steps given to r in this pass
         for (int k = 0; r.next < r.npix && used < s->budget &&
@@ -804,9 +816,12 @@ int nb_server_step(nb_server *s, double timeout_s, int *n_active) {
         }
       }
     }
-    wl->n = nt;
-    ww->n = nw;
-    if (nt + nw > 0) {
+    int items = 0;
+    for (int k = 0; k < kKinds; ++k) {
+      wl[k].n = n_items[k];
+      items += n_items[k];
+    }
+    if (items > 0) {
       const int b = s->cur;
       cudaStream_t st = stream_of(s, b);
       // this step's slot uploads are on st; those of the previous build

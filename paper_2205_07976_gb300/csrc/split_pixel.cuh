@@ -43,6 +43,16 @@ struct SplitEntry {
              // pm | unit << 16 | interval entry << 31
 };
 constexpr int kIntervalEntry = 1 << 31;
+// Lines: from so many sources and steps per pixel interval entries are summed
+// segment by segment (sum_tasks), in tasks of at most kTaskLen steps (even; 16
+// cost the large shot 6 % more).  Kernels of this form have 128 registers (4
+// blocks per SM): 96 (5) spill 540 bytes, 168 (3) hide less: 13.4, 11.6 and
+// 11.8 ms on 1024^2 pixels of the large shot when it was chosen.
+constexpr int kLineSources = 32;
+constexpr int kLineSteps = 1200;
+constexpr int kTaskLen = 32;
+constexpr int kLineBlocks = 4;
+constexpr int SRC32_PAIR = 4;
 static_assert(sizeof(SplitEntry) % 16 == 0, "entries stay 16-byte aligned");
 static_assert(SRC32_DL == 0 && SRC32_W == 1 && SRC32_DH == 2 &&
                   SRC32_STRIDE % 4 == 0 && kUnitFloats % 2 == 0,
@@ -275,6 +285,7 @@ struct SplitBlock {
   int PM, S, nblk, sstep;
   float u0h, u0l, cwide, dmin, dmax, dmarg, inv_step;
   float cmarg[3];
+  float umid, dhalf, nmarg[3];  // split_item's early test
   bool iv_ok, even;
 };
 
@@ -328,6 +339,20 @@ __device__ __forceinline__ void split_stage(SplitBlock &b, float *sms,
   for (int i = threadIdx.x; i < S * SRC32_STRIDE; i += blockDim.x)
     s_src[i] = src32[i];
   __syncthreads();
+  // with one beam direction a row's other columns hold the source and the
+  // next one side by side (sum_tasks): (delta_hi x2, delta_lo x2), w x2; the
+  // last source is followed by itself with weight 0
+  if (!a.has_div)
+    for (int k = threadIdx.x; k < S; k += blockDim.x) {
+      float *q = s_src + k * SRC32_STRIDE;
+      const float *q1 = k + 1 < S ? q + SRC32_STRIDE : q;
+      q[SRC32_PAIR] = q[SRC32_DH];
+      q[SRC32_PAIR + 1] = q1[SRC32_DH];
+      q[SRC32_PAIR + 2] = q[SRC32_DL];
+      q[SRC32_PAIR + 3] = q1[SRC32_DL];
+      q[SRC32_PAIR + 4] = q[SRC32_W];
+      q[SRC32_PAIR + 5] = k + 1 < S ? q1[SRC32_W] : 0.f;
+    }
   // delta_hi range of every block of kSrcBlock sources (the pruning test)
   for (int bb = threadIdx.x; bb < nblk; bb += blockDim.x) {
     float mn = 3.0e38f, mx = -3.0e38f;
@@ -376,6 +401,25 @@ __device__ __forceinline__ void split_stage(SplitBlock &b, float *sms,
   int sstep = 1;
   while (sstep * 2 <= S) sstep *= 2;
   b.sstep = sstep;
+  // the early test: 1/lambda = umid +- dhalf; cmarg plus the error of h in
+  // plain FP32 (a few roundings of sum |A_i v_i| / lambda, |v| <= 2)
+  {
+    float am = 0.f;
+    for (int r = threadIdx.x; r < PM * 3; r += blockDim.x)
+      am = fmaxf(am, fabsf(s_ax2[3 * r].x) + fabsf(s_ax2[3 * r + 1].x) +
+                         fabsf(s_ax2[3 * r + 2].x));
+    // positive floats order like their bits
+    am = __uint_as_float(
+        __reduce_max_sync(0xffffffffu, __float_as_uint(am)));
+    __shared__ float s_am[kSplitWarps];
+    if ((threadIdx.x & 31) == 0) s_am[threadIdx.x >> 5] = am;
+    __syncthreads();
+    for (int w = 0; w < kSplitWarps; ++w) am = fmaxf(am, s_am[w]);
+    b.umid = u0h + 0.5f * (b.dmin + b.dmax);
+    b.dhalf = 0.5f * (b.dmax - b.dmin) * 1.00001f;
+    for (int x = 0; x < 3; ++x)
+      b.nmarg[x] = b.cmarg[x] + 2e-6f * am * (b.umid + b.dhalf) + 1e-5f;
+  }
   // nearly even delta spacing (an equispaced spectrum): the position of a
   // bound in the table is then guessed from the spacing and corrected by a
   // step or two, instead of a binary search
@@ -492,11 +536,11 @@ struct PairQueue {
   int e0 = 0, en = 0, ch = 0, ct = 0;
 };
 
-// Appends one entry per lane with len > 0 (sources k1 .. k1 + len - 1 of the
-// item whose state the lane holds; r and d4 as SplitEntry describes), in
-// lane order.  Called by all lanes.
+// Appends one entry per lane with len > 0 pairs (or tasks), in lane order: the
+// state of the lane's item (r and d4 as SplitEntry describes) and the words
+// of SplitEntry::m.  Called by all lanes.
 __device__ __forceinline__ void push_entries(
-    SplitEntry *ring, PairQueue &pq, int len, int k1, int aux,
+    SplitEntry *ring, PairQueue &pq, int len, int mx, int my, int mw,
     const float Gh[3], const float r[3], const float Gl[3], const float rl[3],
     float4 d4) {
   const int lane = threadIdx.x & 31;
@@ -516,7 +560,7 @@ __device__ __forceinline__ void push_entries(
     E.b = make_float4(Gl[0], Gl[1], rl[0], rl[1]);
     E.c = make_float4(Gh[2], r[2], Gl[2], rl[2]);
     E.d = d4;
-    E.m = make_int4(k1, len, pq.ct + inc - len, aux);
+    E.m = make_int4(mx, my, pq.ct + inc - len, mw);
   }
   pq.en += __popc(hm);
   pq.ct += tot;
@@ -530,7 +574,8 @@ __device__ __forceinline__ void push_entries(
 template <int INTERP, int HASDIV>
 __device__ __forceinline__ unsigned sum_pairs(
     const SpotArgs &a, const SplitBlock &b, const SplitEntry *ring,
-    PairQueue &pq, const float *unit, float4 *cache, int *tags, Kahan &acc) {
+    PairQueue &pq, const float *unit, float4 *cache, int *tags, Kahan &acc,
+    unsigned &npairs) {
   const int lane = threadIdx.x & 31;
   const int np = min(32, pq.ct - pq.ch);
   // entries e0 .. e0 + 31 can overlap the window [ch, ch + 32)
@@ -627,6 +672,7 @@ __device__ __forceinline__ unsigned sum_pairs(
     const float yy = df[0] * bv[0] + df[1] * bv[1] + df[2] * bv[2];
     w *= 0.5f * (1.f + c2 * c2 - a.kahn * (xx * xx - yy * yy));
   }
+  npairs += valid;
   const unsigned hm = __ballot_sync(0xffffffffu, hit);
   if (hm != 0u) {
     CellRef cr;
@@ -644,208 +690,699 @@ __device__ __forceinline__ unsigned sum_pairs(
   return __popc(hm);
 }
 
+// ------------------------------------------------- lines through a cell
+//
+// The steps of an interval entry lie on a line: with t = delta - delta_0 their
+// offset from the lattice point is f = f0 + G t.  So
+//   sum N^2 f^2 = Rmin + A (t - t*)^2,  A = sum N^2 G^2,
+// and, as long as no offset changes its sign, F_cell is one cell's tricubic
+// polynomial on a line: a polynomial of degree 9 in t.  A lane that takes such
+// a segment makes its ten coefficients once (cell_line: ~180 FMAs, packed where
+// two powers of x go side by side) and then spends ~25 instructions on a step,
+// one of them a shared load, where the pair queue spends ~250 per 32 steps on
+// finding entry, source and cell and on 63 FMAs and 16 shared loads per step.
+
+// Coefficients q of F(x0 + g tau), a cell's polynomial (SpotArgs::C4 at cp) on
+// a line: shifted and scaled per power of z, then Horner in y and x with
+// polynomials in tau as coefficients.
+__device__ __forceinline__ void cell_line(const float4 *cp, const float x0[3],
+                                          const float g[3], float q[10]) {
+  const f32x2 z0 = splat2(x0[2]), y0 = splat2(x0[1]), gy = splat2(g[1]),
+              g1 = splat2(g[2]), g2 = splat2(g[2] * g[2]),
+              g3 = splat2(g[2] * g[2] * g[2]);
+  const ulonglong2 *c2 = reinterpret_cast<const ulonglong2 *>(cp);
+  f32x2 Q[2][7];
+#pragma unroll
+  for (int P = 0; P < 2; ++P) {
+    f32x2 V[7];
+#pragma unroll
+    for (int ib = 3; ib >= 0; --ib) {
+      const ulonglong2 A = __ldg(c2 + (P * 4 + ib) * 2),
+                       B = __ldg(c2 + (P * 4 + ib) * 2 + 1);
+      // c3 z^3 + .. + c0 about z0: repeated synthetic division
+      const f32x2 c3 = A.x;
+      f32x2 d[4];
+      d[2] = ffma2(c3, z0, A.y);
+      d[1] = ffma2(d[2], z0, B.x);
+      d[0] = ffma2(d[1], z0, B.y);
+      d[2] = ffma2(c3, z0, d[2]);
+      d[1] = fmul2(ffma2(d[2], z0, d[1]), g1);
+      d[2] = fmul2(ffma2(c3, z0, d[2]), g2);
+      d[3] = fmul2(c3, g3);
+      if (ib == 3) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) V[i] = d[i];
+      } else {
+        // V (y0 + gy tau) + d; V has L coefficients
+        const int L = 6 - ib;
+        V[L] = fmul2(V[L - 1], gy);
+#pragma unroll
+        for (int i = 5; i > 0; --i)
+          if (i < L)
+            V[i] = ffma2(V[i], y0,
+                         i < 4 ? ffma2(V[i - 1], gy, d[i])
+                               : fmul2(V[i - 1], gy));
+        V[0] = ffma2(V[0], y0, d[0]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 7; ++i) Q[P][i] = V[i];
+  }
+  // Q[P] = the pair of x^(2P) and x^(2P+1): Horner in x
+#pragma unroll
+  for (int i = 0; i < 7; ++i) q[i] = upk2(Q[1][i]).y;
+#pragma unroll
+  for (int ia = 2; ia >= 0; --ia) {
+    const int L = 9 - ia;  // coefficients of q: 7, 8, 9
+    q[L] = q[L - 1] * g[0];
+#pragma unroll
+    for (int i = 8; i >= 0; --i)
+      if (i < L) {
+        const float2 c2i = i < 7 ? upk2(Q[ia == 2][i]) : make_float2(0.f, 0.f);
+        const float c = ia == 1 ? c2i.y : c2i.x;
+        q[i] = fmaf(q[i], x0[0],
+                    i == 0  ? c
+                    : i < 7 ? fmaf(q[i - 1], g[0], c)
+                            : q[i - 1] * g[0]);
+      }
+  }
+}
+
+// The segments of an interval entry [k1, k2) between the sources at which an
+// offset changes its sign (tricubic lookup), as the words of SplitEntry::m of
+// a line entry: k1 | k2 << 11, number of tasks | b3 << 8, (first task,) b1 | b2
+// << 11 with k1 <= b1 <= b2 <= b3 <= k2.  S <= 1024 and at most 3 + S /
+// kTaskLen tasks keep the fields.
+__device__ __forceinline__ int seg_tasks(int len) {
+  return (len + kTaskLen - 1) / kTaskLen;
+}
+template <int INTERP>
+__device__ __forceinline__ void line_segments(const SplitBlock &b, int k1,
+                                              int k2, const float Gh[3],
+                                              const float dx[3],
+                                              const float rl[3], int &mx,
+                                              int &my, int &mw) {
+  int c[3] = {k2, k2, k2};
+  if (INTERP == 1) {
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      // the first source beyond the zero of G delta + dx + rl
+      const float z = -__fdividef(dx[x] + rl[x], Gh[x]);
+      int lo = k1;
+      if (b.even) {
+        lo = count_below(b.dh, b.S, guess_index(z, b.dmin, b.inv_step, b.S),
+                         z);
+      } else {
+        int hi = k2;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (b.dh[mid] < z)
+            lo = mid + 1;
+          else
+            hi = mid;
+        }
+      }
+      c[x] = min(max(lo, k1), k2);
+    }
+  }
+  const int lo01 = min(c[0], c[1]), hi01 = max(c[0], c[1]);
+  const int b1 = min(lo01, c[2]), b3 = max(hi01, c[2]),
+            b2 = max(lo01, min(hi01, c[2]));
+  const int n = seg_tasks(b1 - k1) + seg_tasks(b2 - b1) + seg_tasks(b3 - b2) +
+                seg_tasks(k2 - b3);
+  mx = k1 | (k2 << 11);
+  my = n | (b3 << 8);
+  mw = b1 | (b2 << 11);
+}
+
+// Sums the next min(32, ct - ch) tasks of a queue of line entries, one per
+// lane, into the lane's Kahan sum.  Called by all lanes; returns the lane's
+// number of steps under the cut and adds its steps to npairs.
+template <int INTERP>
+__device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
+                                              const SplitBlock &b,
+                                              const SplitEntry *ring,
+                                              PairQueue &pq, Kahan &acc,
+                                              unsigned &npairs) {
+  constexpr float kLog2 = 2.f / 0.63f * 1.44269504f;  // exponent per R
+  const float ecut = -kGaussCut * 0.63f * kLog2;
+  const int lane = threadIdx.x & 31;
+  const int np = min(32, pq.ct - pq.ch);
+  // the entry of each task, as in sum_pairs
+  int4 mm = make_int4(0, 0, 0x7fffffff, 0);
+  if (pq.e0 + lane < pq.en) mm = ring[(pq.e0 + lane) & (kEntries - 1)].m;
+  const int mt = mm.y & 255;
+  const bool ov = pq.e0 + lane < pq.en && mm.z < pq.ch + np &&
+                  mm.z + mt > pq.ch;
+  const unsigned M = __reduce_or_sync(
+      0xffffffffu, ov ? 1u << max(mm.z - pq.ch, 0) : 0u);
+  const int j = __popc(M & (0xffffffffu >> (31 - lane))) - 1;
+  const int ex = __shfl_sync(0xffffffffu, mm.x, j),
+            ey = __shfl_sync(0xffffffffu, mm.y, j),
+            pos = __shfl_sync(0xffffffffu, mm.z, j),
+            ew = __shfl_sync(0xffffffffu, mm.w, j);
+  const unsigned done =
+      __ballot_sync(0xffffffffu, ov && mm.z + mt <= pq.ch + np);
+  // the task's sources [p, e)
+  int p = 0, e = 0;
+  if (lane < np) {
+    const int bd[5] = {ex & 2047, ew & 2047, (ew >> 11) & 2047, ey >> 8,
+                       ex >> 11};
+    int rem = pq.ch + lane - pos;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int nt = seg_tasks(bd[q + 1] - bd[q]);
+      if (rem >= 0 && rem < nt) {
+        p = bd[q] + rem * kTaskLen;
+        e = min(p + kTaskLen, bd[q + 1]);
+      }
+      rem -= nt;
+    }
+  }
+  const int n = e - p;
+  npairs += n;
+  const SplitEntry &E4 = ring[(pq.e0 + j) & (kEntries - 1)];
+  const float4 Ea = E4.a, Eb = E4.b, Ec = E4.c, Ed = E4.d;
+  const float Gh[3] = {Ea.x, Ea.y, Ec.x}, dx[3] = {Ea.z, Ea.w, Ec.y};
+  const float Gl[3] = {Eb.x, Eb.y, Ec.z}, rl[3] = {Eb.z, Eb.w, Ec.w};
+  const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
+  // the middle source is the origin of the line
+  const int mid = (p + e) >> 1;
+  const float4 sm =
+      *reinterpret_cast<const float4 *>(b.src + mid * SRC32_STRIDE);
+  const float half = fmaxf(b.dh[max(e - 1, 0)] - sm.z, sm.z - b.dh[p]);
+  const float ih = half > 0.f ? __fdividef(1.f, half) : 0.f;
+  float f0[3], fl0[3], g[3];
+  float A = 0.f, Bq = 0.f;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    const float sx = fmaf(Gh[x], sm.z, dx[x]);
+    const float c = fmaf(Gh[x], sm.x, fmaf(Gl[x], sm.z, rl[x]));
+    f0[x] = __fadd_rn(sx, c);
+    fl0[x] = __fsub_rn(c, __fsub_rn(f0[x], sx));
+    g[x] = Gh[x] * half;
+    A = fmaf(N2[x] * g[x], g[x], A);
+    Bq = fmaf(N2[x] * g[x], f0[x], Bq);
+  }
+  // tau = (delta - delta_0) / half; R = Rmin + A (tau - ts)^2
+  const float ts = A > 0.f ? -__fdividef(Bq, A) : 0.f;
+  float R = 0.f;
+  const float th = ts * half;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    const float fs = fmaf(Gh[x], th, f0[x]) + fmaf(Gl[x], th, fl0[x]);
+    R = fmaf(N2[x] * fs, fs, R);
+  }
+  const float e0 = -kLog2 * R, cA = -kLog2 * A;
+  float q[10], Fn = 0.f;
+  bool line = true;  // the segment's cell lies in the table
+  int nt[3];
+  if (INTERP == 1) {
+    const int npk = __float_as_int(Ed.y);
+    nt[0] = (npk & 1023) - 1;
+    nt[1] = ((npk >> 10) & 1023) - 1;
+    nt[2] = ((npk >> 20) & 1023) - 1;
+    CellRef c;
+    cell_of_entry(a, n > 0, f0, __float_as_int(Ed.x), __float_as_int(Ed.z), c);
+    line = c.tri || n == 0;
+    if (c.tri)
+      cell_line(a.C4 + (size_t)nb_idx(a.check, NB_SITE_CELL, c.ci,
+                                      cell_count(a)) * kCellChunks,
+                c.x, g, q);
+  } else {
+    nt[0] = __float_as_int(Ed.x);
+    nt[1] = __float_as_int(Ed.y);
+    nt[2] = __float_as_int(Ed.z);
+    if (n) Fn = fcell_f32<0>(a, nt, f0);
+  }
+  unsigned hits = 0;
+  if (__all_sync(0xffffffffu, line)) {
+    const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
+    const float *src = b.src + p * SRC32_STRIDE + SRC32_PAIR;
+    const f32x2 ih2 = splat2(ih), rl2 = splat2(-sm.x * ih),
+                rh2 = splat2(-sm.z), ts2 = splat2(-ts), cA2 = splat2(cA),
+                e02 = splat2(e0);
+    f32x2 q2[10];
+    if (INTERP == 1) {
+#pragma unroll
+      for (int d = 0; d < 10; ++d) q2[d] = splat2(q[d]);
+    }
+    // (nearest lookup: the entry's one structure factor)
+    const float fac = INTERP == 1 ? a.N6 * Ed.w : Fn * Fn * (a.N6 * Ed.w);
+    for (int i0 = 0; i0 < nmax; i0 += 16) {
+      f32x2 sum2 = splat2(0.f);  // at most 8 terms per lane half
+      const int iend = min(i0 + 16, nmax);
+      for (int i = i0; i < iend; i += 2) {
+        if (i < n) {
+          const ulonglong2 sd = *reinterpret_cast<const ulonglong2 *>(
+              src + i * SRC32_STRIDE);
+          const f32x2 w =
+              *reinterpret_cast<const f32x2 *>(src + i * SRC32_STRIDE + 4);
+          const f32x2 tau =
+              ffma2(fadd2(sd.x, rh2), ih2, ffma2(sd.y, ih2, rl2));
+          const f32x2 tt = fadd2(tau, ts2);
+          const float2 xe = upk2(ffma2(fmul2(cA2, tt), tt, e02));
+          float2 Ex;
+          asm("ex2.approx.f32 %0, %1;" : "=f"(Ex.x) : "f"(xe.x));
+          asm("ex2.approx.f32 %0, %1;" : "=f"(Ex.y) : "f"(xe.y));
+          const bool h0 = xe.x >= ecut, h1 = xe.y >= ecut && i + 1 < n;
+          Ex.x = h0 ? Ex.x : 0.f;
+          Ex.y = h1 ? Ex.y : 0.f;
+          hits += h0;
+          hits += h1;
+          const f32x2 wE = fmul2(w, pk2(Ex));
+          if (INTERP == 1) {
+            f32x2 F = q2[9];
+#pragma unroll
+            for (int d = 8; d >= 0; --d) F = ffma2(F, tau, q2[d]);
+            sum2 = ffma2(fmul2(F, F), wE, sum2);
+          } else {
+            sum2 = fadd2(sum2, wE);
+          }
+        }
+      }
+      const float2 sum = upk2(sum2);
+      acc.add((sum.x + sum.y) * fac);
+    }
+  } else {
+    // some lane's cell reaches out of the table: step by step from the table
+    for (int i = 0; i < n; ++i) {
+      const float4 sw = *reinterpret_cast<const float4 *>(
+          b.src + (p + i) * SRC32_STRIDE);
+      float fr[3], rad2 = 0.f;
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        fr[x] = fmaf(Gh[x], sw.z, dx[x]) +
+                fmaf(Gh[x], sw.x, fmaf(Gl[x], sw.z, rl[x]));
+        rad2 = fmaf(N2[x] * fr[x], fr[x], rad2);
+      }
+      if (rad2 <= kGaussCut * 0.63f) {
+        const float F = fcell_f32<INTERP>(a, nt, fr);
+        acc.add(F * F * (a.N6 * __expf(-2.f * rad2 * (1.f / 0.63f))) *
+                (sw.y * Ed.w));
+        ++hits;
+      }
+    }
+  }
+  pq.e0 += __popc(done);
+  pq.ch += np;
+  __syncwarp();  // the ring slots read above may be refilled next
+  return hits;
+}
+
+// The lane's item (unit u, orientation pm) of a batch, 32 items further per
+// step without a division.
+struct ItemWalk {
+  int u, pm, du, dpm;
+  __device__ __forceinline__ ItemWalk(int lane, int PM) {
+    u = lane / PM;
+    pm = lane - u * PM;
+    du = 32 / PM;
+    dpm = 32 - du * PM;
+  }
+  __device__ __forceinline__ void next(int PM) {
+    u += du;
+    pm += dpm;
+    if (pm >= PM) {
+      pm -= PM;
+      ++u;
+    }
+  }
+};
+
+// One (unit, phi x mosaic) item of a lane: G and r = u0 G - n0 in
+// double-float, r's high part on a 2^-21 grid.
+struct SplitItem {
+  bool valid;
+  int aux;     // pm | unit << 16
+  float scal;  // omega cap pol of the unit
+  float Gh[3], Gl[3], rq[3], rl[3], n0[3];
+};
+
+// Forms the lane's item (u, pm).  EARLY: returns false, with the
+// items not formed, where no lane's sweep comes near a lattice point.
+template <bool EARLY>
+__device__ __forceinline__ bool split_item(const SplitBlock &b,
+                                           const float *unit, int u, int pm,
+                                           bool valid, SplitItem &t) {
+  const float u0h = b.u0h, u0l = b.u0l;
+  t.valid = valid;
+  t.aux = pm | (u << 16);
+  const float *ud = unit + u * kUnitFloats;
+  // vh[3], vl[3], scal as four float2 loads (unit rows are 8-byte aligned)
+  const float2 *u2 = reinterpret_cast<const float2 *>(ud);
+  const float2 p0 = u2[0], p1 = u2[1], p2 = u2[2], p3 = u2[3];
+  const float vh[3] = {p0.x, p0.y, p1.x}, vl[3] = {p1.y, p2.x, p2.y};
+  t.scal = p3.x;
+  if (EARLY && b.iv_ok) {
+    // h in plain FP32 at the sweep's middle, the distance to the nearest
+    // integer against half the sweep and the margin
+    bool near = t.valid;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const float2 *A3 = b.ax2 + pm * 9 + 3 * x;
+      const float g = fmaf(A3[0].x, vh[0], fmaf(A3[1].x, vh[1],
+                                                A3[2].x * vh[2]));
+      const float h = g * b.umid;
+      near = near && !(fabsf(h - rintf(h)) > fmaf(fabsf(g), b.dhalf,
+                                                  b.nmarg[x]));
+    }
+    if (!__any_sync(0xffffffffu, near)) return false;
+  }
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    ff_dot3_pairs(b.ax2 + pm * 9 + 3 * x, vh, vl, t.Gh[x], t.Gl[x]);
+    float qh, qe;
+    two_prod(t.Gh[x], u0h, qh, qe);
+    const float ql = fmaf(t.Gh[x], u0l, fmaf(t.Gl[x], u0h, qe));
+    t.n0[x] = rintf(qh);
+    float rh, rl0;
+    two_sum(__fsub_rn(qh, t.n0[x]), ql, rh, rl0);
+    // r_hi on a 2^-21 grid: r_hi - n is then exact for |n| < 7
+    t.rq[x] = __fmul_rn(rintf(__fmul_rn(rh, 2097152.f)), 1.f / 2097152.f);
+    t.rl[x] = rl0 + __fsub_rn(rh, t.rq[x]);
+  }
+  return true;
+}
+
+// The lattice points an item's sweep can come near: per axis the integers
+// ml + 0 .. nm - 1 within sqrt(cwide)/N_x of [h(dmin), h(dmax)], in odometer
+// order (dg); A = sum N^2 G^2 of the exponent along the sweep.
+struct LatticeRange {
+  int ncomb, ml[3], nm[3], dg[3];
+  float A;
+};
+__device__ __forceinline__ void lattice_range(const SplitBlock &b,
+                                              const float N2[3],
+                                              const SplitItem &t,
+                                              LatticeRange &L) {
+  L.ncomb = 0;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) L.ml[x] = L.nm[x] = L.dg[x] = 0;
+  if (b.iv_ok && t.valid) {
+    L.ncomb = 1;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const float lo = fmaf(t.Gh[x], b.dmin, t.rq[x]),
+                  hi = fmaf(t.Gh[x], b.dmax, t.rq[x]);
+      L.ml[x] = (int)ceilf(fminf(lo, hi) - b.cmarg[x]);
+      L.nm[x] = (int)floorf(fmaxf(lo, hi) + b.cmarg[x]) - L.ml[x] + 1;
+      if (L.nm[x] < 0) L.nm[x] = 0;
+      L.ncomb *= L.nm[x];
+    }
+  }
+  L.A = N2[0] * t.Gh[0] * t.Gh[0];
+  L.A = fmaf(N2[1] * t.Gh[1], t.Gh[1], L.A);
+  L.A = fmaf(N2[2] * t.Gh[2], t.Gh[2], L.A);
+}
+
+// The next lattice point of the lane's range (the c-th of all lanes): for
+// lattice point m the exponent sum along the sweep is A d^2 + 2 B d + C, below
+// cwide on one interval [k1, k2) of the sorted delta table.  dx = r_q - (m -
+// n0), nt = the table-relative m.
+__device__ __forceinline__ void lattice_interval(
+    const SpotArgs &a, const SplitBlock &b, const float N2[3],
+    const SplitItem &t, LatticeRange &L, int c, int &k1, int &k2, float dx[3],
+    int nt[3]) {
+  const int S = b.S;
+  const float *s_dh = b.dh;
+  k1 = k2 = 0;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    dx[x] = 0.f;
+    nt[x] = 0;
+  }
+  if (c >= L.ncomb) return;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    // lattice point n0 + mx; its table index nt
+    const int mx = L.ml[x] + L.dg[x];
+    dx[x] = t.rq[x] - (float)mx;  // exact: r_q on a 2^-21 grid
+    nt[x] = (int)t.n0[x] + mx - a.hmin[x];
+  }
+  if (++L.dg[0] == L.nm[0]) {
+    L.dg[0] = 0;
+    if (++L.dg[1] == L.nm[1]) {
+      L.dg[1] = 0;
+      ++L.dg[2];
+    }
+  }
+  float B = N2[0] * t.Gh[0] * dx[0];
+  B = fmaf(N2[1] * t.Gh[1], dx[1], B);
+  B = fmaf(N2[2] * t.Gh[2], dx[2], B);
+  float C0 = N2[0] * dx[0] * dx[0];
+  C0 = fmaf(N2[1] * dx[1], dx[1], C0);
+  C0 = fmaf(N2[2] * dx[2], dx[2], C0);
+  if (L.A > 0.f) {
+    const float disc = fmaf(B, B, -L.A * (C0 - b.cwide));
+    if (disc >= 0.f) {
+      // the bounds carry a relative margin far above the error of the
+      // reciprocal
+      const float sq = sqrtf(disc), ia = __frcp_rn(L.A);
+      float lo = (-B - sq) * ia, hi = (-B + sq) * ia;
+      const float mg = 1e-4f * (fabsf(lo) + fabsf(hi)) + b.dmarg;
+      lo -= mg;
+      hi += mg;
+      // k1 = #{delta < lo}, k2 = #{delta <= hi} (sorted table)
+      if (b.even) {
+        k1 = count_below(s_dh, S, guess_index(lo, b.dmin, b.inv_step, S), lo);
+        k2 = count_at_most(s_dh, S, guess_index(hi, b.dmin, b.inv_step, S),
+                           hi);
+      } else {
+        for (int st = b.sstep; st > 0; st >>= 1) {
+          if (k1 + st <= S && s_dh[k1 + st - 1] < lo) k1 += st;
+          if (k2 + st <= S && s_dh[k2 + st - 1] <= hi) k2 += st;
+        }
+      }
+    }
+  } else if (C0 <= b.cwide) {
+    k2 = S;  // the sweep does not move: all or nothing
+  }
+}
+
+// SplitEntry::d of an interval entry at lattice point nt
+template <int INTERP>
+__device__ __forceinline__ float4 entry_data(const SpotArgs &a, bool any,
+                                             const int nt[3], float scal) {
+  if (INTERP == 1 && a.C4) {
+    // the lattice point's cell data once per entry; the index packed
+    // (clamped to [-1, hn]: any index outside the table looks up
+    // default_F, and cell tables exist only for hn < 1024)
+    int ci0 = 0, pk = 0, npk = 0;
+    if (any) {
+      entry_cell_data(a, nt, ci0, pk);
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+        npk |= (min(max(nt[x], -1), a.hn[x]) + 1) << (10 * x);
+    }
+    return make_float4(__int_as_float(ci0), __int_as_float(npk),
+                       __int_as_float(pk), scal);
+  }
+  return make_float4(__int_as_float(nt[0]), __int_as_float(nt[1]),
+                     __int_as_float(nt[2]), scal);
+}
+
+// Pruned scan: h_x = G_x delta + r_x is linear in delta, so a block of
+// sources whose delta range keeps some axis farther than sqrt(cut)/N_x from
+// every integer holds no surviving term.  Pushes block bb of every lane's
+// item that may hold one.
+__device__ __forceinline__ void push_block(const SplitBlock &b,
+                                           SplitEntry *ring, PairQueue &pq,
+                                           const SplitItem &t, int bb) {
+  bool pass = false;
+  if (t.valid) {
+    const float dmn = b.blk[2 * bb], dmx = b.blk[2 * bb + 1];
+    pass = true;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const float lo0 = fmaf(t.Gh[x], dmn, t.rq[x]),
+                  hi0 = fmaf(t.Gh[x], dmx, t.rq[x]);
+      const float lo = fminf(lo0, hi0) - b.cmarg[x],
+                  hi = fmaxf(lo0, hi0) + b.cmarg[x];
+      pass = pass && floorf(hi) >= ceilf(lo);
+    }
+  }
+  const int st0 = bb * kSrcBlock;
+  const int len = pass ? min(kSrcBlock, b.S - st0) : 0;
+  push_entries(ring, pq, len, st0, len, t.aux, t.Gh, t.rq, t.Gl, t.rl,
+               make_float4(t.n0[0], t.n0[1], t.n0[2], t.scal));
+}
+
+// How split_sum goes through the interval entries: pair by pair; the same
+// with split_item's early test; line by line, with that test (split_form)
+enum { kPairs = 0, kPairsEarly = 1, kLines = 2 };
+
+// The form for a shot of PM orientations and S sources.  Lines need enough
+// tasks per pixel to fill a pass, and enough steps per line to pay for its
+// coefficients (pairs with the early test -> lines, 700^2 pixels: 1 unit, S =
+// 100, M = 12 0.605 -> 0.541 ms; S = 60, M = 30 0.750 -> 0.621; S = 30, M = 50
+// 0.820 -> 0.816; S = 20, M = 50 0.696 -> 0.777; S = 60, M = 12, 1000^2 0.787 ->
+// 0.873; large shot, 1024^2: 18.2 -> 10.2).  The early test pays where lattice
+// points are rare: N = 25 (0.07 of h space lies within the cut) 1.22 -> 1.05
+// ms on 1500^2 pixels with S = 11, M = 9, but at N = 15 (0.34) it finds one in
+// most batches, 1.86 -> 2.11 ms on the 64-panel shot.
+__host__ __device__ inline int split_form(const SpotArgs &a, int PM, int S) {
+  if (a.has_div) return kPairs;
+  if ((a.interp == 0 || a.C4) && S >= kLineSources &&
+      (long long)a.os * a.os * a.T * PM * S >= kLineSteps)
+    return kLines;
+  // the share of h space within the cut of a lattice point, per axis
+  const float m = sqrtf(kGaussCut * 0.63f) * 2.f;
+  return m / a.N[0] * (m / a.N[1]) * (m / a.N[2]) < 0.2f ? kPairsEarly
+                                                          : kPairs;
+}
+
 // The sum, without the prefactor, of the pixel whose U sub-pixel units are
 // already in `unit` (split_unit), computed by the calling warp (all 32
 // lanes); every lane returns the same value.  Adds the terms it evaluated
 // to `cnt` and, with COUNT, the rest of the work it performed.
-template <int INTERP, int HASDIV, int COUNT = 0>
+template <int INTERP, int HASDIV, int FORM, int COUNT = 0>
 __device__ __forceinline__ double split_sum(const SpotArgs &a,
                                             const SplitBlock &b,
                                             const float *unit,
                                             SplitCounts &cnt) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int PM = b.PM, S = b.S, nblk = b.nblk, sstep = b.sstep;
-  const float2 *s_ax2 = b.ax2;
-  const float *s_blk = b.blk, *s_dh = b.dh;
   SplitEntry *ring = b.ent_base + warp * kEntries;
   float4 *cache = b.cell_cache + warp * kCellChunks * kCellSlots;
   int *tags = b.cell_tags + warp * kCellSlots;
-  const int U = a.os * a.os * a.T, items = U * PM;
+  const int items = a.os * a.os * a.T * b.PM;
   const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
-  const float cwide = b.cwide;
-  const float cmarg[3] = {b.cmarg[0], b.cmarg[1], b.cmarg[2]};
-  const bool iv_ok = b.iv_ok;
-  const float dmin = b.dmin, dmax = b.dmax, dmarg = b.dmarg;
-  const bool even = b.even;
-  const float inv_step = b.inv_step;
-  const float u0h = b.u0h, u0l = b.u0l;
 
   Kahan acc;
   PairQueue pq;
   unsigned nterms = 0, nivals = 0, nblocks = 0;
-  auto drain = [&]() {
-    while (pq.ct - pq.ch >= 32)
-      nterms += sum_pairs<INTERP, HASDIV>(a, b, ring, pq, unit, cache, tags,
-                                          acc);
-  };
-  // ---- items: lanes take (unit, phi x mosaic) items 32 at a time, form
-  // G and r, and push their source intervals; the pair queue is summed
-  // 32 pairs at a time as it fills
-  for (int base = 0; base < items; base += 32) {
-    const int it = base + lane;
-    const bool valid = it < items;
-    const int u = valid ? it / PM : 0, pm = valid ? it - u * PM : 0;
-    const float *ud = unit + u * kUnitFloats;
-    // vh[3], vl[3], scal as four float2 loads (unit rows are 8-byte aligned)
-    const float2 *u2 = reinterpret_cast<const float2 *>(ud);
-    const float2 p0 = u2[0], p1 = u2[1], p2 = u2[2], p3 = u2[3];
-    const float vh[3] = {p0.x, p0.y, p1.x}, vl[3] = {p1.y, p2.x, p2.y};
-    const float scal = p3.x;
-    float Gh[3], Gl[3], rq[3], rl[3], n0[3];
-#pragma unroll
-    for (int x = 0; x < 3; ++x) {
-      ff_dot3_pairs(s_ax2 + pm * 9 + 3 * x, vh, vl, Gh[x], Gl[x]);
-      float qh, qe;
-      two_prod(Gh[x], u0h, qh, qe);
-      const float ql = fmaf(Gh[x], u0l, fmaf(Gl[x], u0h, qe));
-      n0[x] = rintf(qh);
-      float rh, rl0;
-      two_sum(__fsub_rn(qh, n0[x]), ql, rh, rl0);
-      // r_hi on a 2^-21 grid: r_hi - n is then exact for |n| < 7
-      rq[x] = __fmul_rn(rintf(__fmul_rn(rh, 2097152.f)), 1.f / 2097152.f);
-      rl[x] = rl0 + __fsub_rn(rh, rq[x]);
-    }
-    if (HASDIV) {
-      // sources of different directions: every source of every item
-      push_entries(ring, pq, valid ? S : 0, 0, pm | (u << 16), Gh, rq, Gl, rl,
-                   make_float4(n0[0], n0[1], n0[2], scal));
-      drain();
-      continue;
-    }
-    // lattice points the item's sweep can come near: per axis the
-    // integers within sqrt(cwide)/N_x of [h(dmin), h(dmax)]
-    int ml[3] = {0, 0, 0}, nm[3] = {0, 0, 0}, ncomb = 0;
-    if (iv_ok && valid) {
-      ncomb = 1;
-#pragma unroll
-      for (int x = 0; x < 3; ++x) {
-        const float lo = fmaf(Gh[x], dmin, rq[x]), hi = fmaf(Gh[x], dmax, rq[x]);
-        ml[x] = (int)ceilf(fminf(lo, hi) - cmarg[x]);
-        nm[x] = (int)floorf(fmaxf(lo, hi) + cmarg[x]) - ml[x] + 1;
-        if (nm[x] < 0) nm[x] = 0;
-        ncomb *= nm[x];
+  unsigned nlines = 0, npairs = 0;  // the lane's own terms and pairs
+  SplitItem t;
+  LatticeRange L;
+  float dx[3];
+  int nt[3], k1, k2;
+  if (FORM == kLines) {
+    // One loop with a single place where the queue is summed and one where
+    // each kind of entry is pushed (with the summing inlined at every push
+    // the kernel waited for instructions a fifth of its time, large shot
+    // 1024^2 11.6 -> 10.2 ms): the queue, then the next lattice point or
+    // source block of the current batch of items, then the next batch.
+    enum { kItems, kLattice, kScan } state = kItems;
+    bool line_q = false;  // the queue holds tasks, not pairs
+    bool flush = false;   // sum the queue to its end first
+    int base = 0, c = 0, maxc = 0;
+    ItemWalk walk(lane, b.PM);
+    while (true) {
+      if (pq.ct - pq.ch >= 32 || (flush && pq.ct > pq.ch)) {
+        if (line_q)
+          nlines += sum_tasks<INTERP>(a, b, ring, pq, acc, npairs);
+        else
+          nterms += sum_pairs<INTERP, HASDIV>(a, b, ring, pq, unit, cache,
+                                              tags, acc, npairs);
+        continue;
       }
-    }
-    if (iv_ok && __all_sync(0xffffffffu, ncomb <= 8)) {
-      // exact intervals: for lattice point m the exponent sum along the
-      // sweep is A d^2 + 2 B d + C, below cwide on one interval of the
-      // sorted delta table
-      const int maxc = (int)__reduce_max_sync(0xffffffffu, (unsigned)ncomb);
-      if (COUNT) nivals += __reduce_add_sync(0xffffffffu, (unsigned)ncomb);
-      // the lattice points ml + (d0, d1, d2), d_x < nm_x, in odometer order;
-      // A of the quadratic depends on the item only
-      float A = N2[0] * Gh[0] * Gh[0];
-      A = fmaf(N2[1] * Gh[1], Gh[1], A);
-      A = fmaf(N2[2] * Gh[2], Gh[2], A);
-      int dg[3] = {0, 0, 0};
-      for (int c = 0; c < maxc; ++c) {
-        int k1 = 0, k2 = 0;
-        float dx[3] = {0.f, 0.f, 0.f};
-        int nt[3] = {0, 0, 0};
-        if (c < ncomb) {
-#pragma unroll
-          for (int x = 0; x < 3; ++x) {
-            // lattice point n0 + mx; its table index nt
-            const int mx = ml[x] + dg[x];
-            dx[x] = rq[x] - (float)mx;  // exact: r_q on a 2^-21 grid
-            nt[x] = (int)n0[x] + mx - a.hmin[x];
-          }
-          if (++dg[0] == nm[0]) {
-            dg[0] = 0;
-            if (++dg[1] == nm[1]) {
-              dg[1] = 0;
-              ++dg[2];
-            }
-          }
-          float B = N2[0] * Gh[0] * dx[0];
-          B = fmaf(N2[1] * Gh[1], dx[1], B);
-          B = fmaf(N2[2] * Gh[2], dx[2], B);
-          float C0 = N2[0] * dx[0] * dx[0];
-          C0 = fmaf(N2[1] * dx[1], dx[1], C0);
-          C0 = fmaf(N2[2] * dx[2], dx[2], C0);
-          if (A > 0.f) {
-            const float disc = fmaf(B, B, -A * (C0 - cwide));
-            if (disc >= 0.f) {
-              // the bounds carry a relative margin far above the error of
-              // the reciprocal
-              const float sq = sqrtf(disc), ia = __frcp_rn(A);
-              float lo = (-B - sq) * ia, hi = (-B + sq) * ia;
-              const float mg = 1e-4f * (fabsf(lo) + fabsf(hi)) + dmarg;
-              lo -= mg;
-              hi += mg;
-              // k1 = #{delta < lo}, k2 = #{delta <= hi} (sorted table)
-              if (even) {
-                k1 = count_below(s_dh, S, guess_index(lo, dmin, inv_step, S),
-                                 lo);
-                k2 = count_at_most(s_dh, S, guess_index(hi, dmin, inv_step, S),
-                                   hi);
-              } else {
-                for (int st = sstep; st > 0; st >>= 1) {
-                  if (k1 + st <= S && s_dh[k1 + st - 1] < lo) k1 += st;
-                  if (k2 + st <= S && s_dh[k2 + st - 1] <= hi) k2 += st;
-                }
-              }
-            }
-          } else if (C0 <= cwide) {
-            k2 = S;  // the sweep does not move: all or nothing
-          }
+      flush = false;
+      if (state != kItems && line_q != (state == kLattice)) {
+        // the other kind of entry: the queue first
+        if (pq.ct > pq.ch) {
+          flush = true;
+          continue;
         }
+        line_q = state == kLattice;
+      }
+      if (state == kLattice) {
+        if (c == maxc) {
+          state = kItems;
+          continue;
+        }
+        lattice_interval(a, b, N2, t, L, c++, k1, k2, dx, nt);
         // no lane has an entry for this lattice point: nothing to push
         if (!__any_sync(0xffffffffu, k2 > k1)) continue;
-        float4 d4;
-        if (INTERP == 1 && a.C4) {
-          // the lattice point's cell data once per entry; the index packed
-          // (clamped to [-1, hn]: any index outside the table looks up
-          // default_F, and cell tables exist only for hn < 1024)
-          int ci0 = 0, pk = 0, npk = 0;
-          if (k2 > k1) {
-            entry_cell_data(a, nt, ci0, pk);
-#pragma unroll
-            for (int x = 0; x < 3; ++x)
-              npk |= (min(max(nt[x], -1), a.hn[x]) + 1) << (10 * x);
-          }
-          d4 = make_float4(__int_as_float(ci0), __int_as_float(npk),
-                           __int_as_float(pk), scal);
-        } else {
-          d4 = make_float4(__int_as_float(nt[0]), __int_as_float(nt[1]),
-                           __int_as_float(nt[2]), scal);
-        }
-        push_entries(ring, pq, k2 > k1 ? k2 - k1 : 0, k1,
-                     pm | (u << 16) | kIntervalEntry, Gh, dx, Gl, rl, d4);
-        drain();
+        int mx = 0, my = 0, mw = 0;
+        if (k2 > k1)
+          line_segments<INTERP>(b, k1, k2, t.Gh, dx, t.rl, mx, my, mw);
+        push_entries(ring, pq, my & 255, mx, my, mw, t.Gh, dx, t.Gl, t.rl,
+                     entry_data<INTERP>(a, k2 > k1, nt, t.scal));
+        continue;
       }
-    } else {
-      // pruned scan: h_x = G_x delta + r_x is linear in delta, so a block
-      // of sources whose delta range [dmn, dmx] keeps some axis farther
-      // than sqrt(cut)/N_x from every integer holds no surviving term
-      if (COUNT) nblocks += __popc(__ballot_sync(0xffffffffu, valid)) * nblk;
-      for (int bb = 0; bb < nblk; ++bb) {
-        bool pass = false;
-        if (valid) {
-          const float dmn = s_blk[2 * bb], dmx = s_blk[2 * bb + 1];
-          pass = true;
-#pragma unroll
-          for (int x = 0; x < 3; ++x) {
-            const float lo0 = fmaf(Gh[x], dmn, rq[x]),
-                        hi0 = fmaf(Gh[x], dmx, rq[x]);
-            const float lo = fminf(lo0, hi0) - cmarg[x],
-                        hi = fmaxf(lo0, hi0) + cmarg[x];
-            pass = pass && floorf(hi) >= ceilf(lo);
-          }
+      if (state == kScan) {
+        if (c == b.nblk) {
+          state = kItems;
+          continue;
         }
-        const int st0 = bb * kSrcBlock;
-        push_entries(ring, pq, pass ? min(kSrcBlock, S - st0) : 0, st0,
-                     pm | (u << 16), Gh, rq, Gl, rl,
-                     make_float4(n0[0], n0[1], n0[2], scal));
-        drain();
+        push_block(b, ring, pq, t, c++);
+        continue;
+      }
+      if (base >= items) {
+        if (pq.ct == pq.ch) break;
+        flush = true;
+        continue;
+      }
+      const bool valid = base + lane < items;
+      const int u = valid ? walk.u : 0, pm = valid ? walk.pm : 0;
+      base += 32;
+      walk.next(b.PM);
+      if (!split_item<true>(b, unit, u, pm, valid, t)) continue;
+      lattice_range(b, N2, t, L);
+      c = 0;
+      if (b.iv_ok && __all_sync(0xffffffffu, L.ncomb <= 8)) {
+        state = kLattice;
+        maxc = (int)__reduce_max_sync(0xffffffffu, (unsigned)L.ncomb);
+        if (COUNT) nivals += __reduce_add_sync(0xffffffffu, (unsigned)L.ncomb);
+      } else {
+        state = kScan;
+        if (COUNT)
+          nblocks += __popc(__ballot_sync(0xffffffffu, t.valid)) * b.nblk;
       }
     }
+  } else {
+    auto drain = [&]() {
+      while (pq.ct - pq.ch >= 32)
+        nterms += sum_pairs<INTERP, HASDIV>(a, b, ring, pq, unit, cache, tags,
+                                            acc, npairs);
+    };
+    // items: lanes take (unit, phi x mosaic) items 32 at a time, form G and r,
+    // and push their source intervals; the pair queue is summed 32 pairs at a
+    // time as it fills
+    ItemWalk walk(lane, b.PM);
+    for (int base = 0; base < items; base += 32, walk.next(b.PM)) {
+      const bool valid = base + lane < items;
+      if (!split_item<FORM == kPairsEarly && !HASDIV>(
+              b, unit, valid ? walk.u : 0, valid ? walk.pm : 0, valid, t))
+        continue;
+      if (HASDIV) {
+        // sources of different directions: every source of every item
+        push_entries(ring, pq, t.valid ? b.S : 0, 0, b.S, t.aux, t.Gh, t.rq,
+                     t.Gl, t.rl,
+                     make_float4(t.n0[0], t.n0[1], t.n0[2], t.scal));
+        drain();
+        continue;
+      }
+      lattice_range(b, N2, t, L);
+      if (b.iv_ok && __all_sync(0xffffffffu, L.ncomb <= 8)) {
+        const int maxc =
+            (int)__reduce_max_sync(0xffffffffu, (unsigned)L.ncomb);
+        if (COUNT) nivals += __reduce_add_sync(0xffffffffu, (unsigned)L.ncomb);
+        for (int c = 0; c < maxc; ++c) {
+          lattice_interval(a, b, N2, t, L, c, k1, k2, dx, nt);
+          // no lane has an entry for this lattice point: nothing to push
+          if (!__any_sync(0xffffffffu, k2 > k1)) continue;
+          push_entries(ring, pq, k2 > k1 ? k2 - k1 : 0, k1, k2 - k1,
+                       t.aux | kIntervalEntry, t.Gh, dx, t.Gl, t.rl,
+                       entry_data<INTERP>(a, k2 > k1, nt, t.scal));
+          drain();
+        }
+      } else {
+        if (COUNT)
+          nblocks += __popc(__ballot_sync(0xffffffffu, t.valid)) * b.nblk;
+        for (int bb = 0; bb < b.nblk; ++bb) {
+          push_block(b, ring, pq, t, bb);
+          drain();
+        }
+      }
+    }
+    if (pq.ct > pq.ch)
+      nterms += sum_pairs<INTERP, HASDIV>(a, b, ring, pq, unit, cache, tags,
+                                          acc, npairs);
   }
-  if (pq.ct > pq.ch)
-    nterms += sum_pairs<INTERP, HASDIV>(a, b, ring, pq, unit, cache, tags, acc);
-  cnt.terms += nterms;
+  cnt.terms += nterms + __reduce_add_sync(0xffffffffu, nlines);
   if (COUNT) {
-    cnt.pairs += pq.ct;
+    cnt.pairs += __reduce_add_sync(0xffffffffu, npairs);
     cnt.ivals += nivals;
     cnt.blocks += nblocks;
   }

@@ -26,6 +26,12 @@
 //      survives the cut, its term (exp, F_cell from the cell's tricubic
 //      polynomial in a per-warp shared-memory cache, or from the table)
 //      into its own Kahan sum;
+//      In shots of many sources and steps (split_form) a lane takes a whole
+//      segment of an entry instead, on which F_cell is a polynomial of degree
+//      9 in delta and the exponent a parabola: ~15 instructions per step in
+//      place of ~8 per lane and step of the pair queue (sum_tasks).  Large
+//      shot: 164.5 -> 104.7 ms; the 512^2 pixels at its centre, where the
+//      batches of items without a lattice point in reach end early, 5.0 -> 2.6;
 //   4. the 32 lane sums are reduced with warp shuffles in float-float.
 // The order of every operation depends only on the pixel's own inputs, so
 // a pixel's value does not depend on what else is in the launch.
@@ -35,8 +41,8 @@
 namespace nbgb {
 
 // COUNT: also count the pairs, intervals and block tests (a.wstats)
-template <int INTERP, int HASDIV, int COUNT, bool FF>
-__global__ void __launch_bounds__(kSplitThreads, 5)
+template <int INTERP, int HASDIV, int COUNT, bool FF, int FORM>
+__global__ void __launch_bounds__(kSplitThreads, FORM == kLines ? kLineBlocks : 5)
     spots_split_kernel(SpotArgs a, unsigned long long *work) {
   extern __shared__ float sms[];
   SplitBlock b;
@@ -76,7 +82,7 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
     __syncwarp();
     double mine = 0.0;  // lane bi keeps the sum of pixel bi
     for (int bi = 0; bi < nb; ++bi) {
-      const double v = split_sum<INTERP, HASDIV, COUNT>(
+      const double v = split_sum<INTERP, HASDIV, FORM, COUNT>(
           a, b, unit + bi * U * kUnitFloats, cnt);
       if (lane == bi) mine = v;
     }
@@ -97,17 +103,27 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
   }
 }
 
+using SplitKernel = void (*)(SpotArgs, unsigned long long *);
+
+template <int INTERP, int COUNT, bool FF>
+static SplitKernel pick_split(const SpotArgs &a) {
+  if (a.has_div) return spots_split_kernel<INTERP, 1, COUNT, FF, kPairs>;
+  switch (split_form(a, a.PM, a.S)) {
+    case kLines: return spots_split_kernel<INTERP, 0, COUNT, FF, kLines>;
+    // (the early test changes no sum and no count: not built with counters)
+    case kPairsEarly:
+      if (!COUNT)
+        return spots_split_kernel<INTERP, 0, COUNT, FF,
+                                  COUNT ? kPairs : kPairsEarly>;
+  }
+  return spots_split_kernel<INTERP, 0, COUNT, FF, kPairs>;
+}
+
 template <bool FF>
-static void (*pick_split(const SpotArgs &a))(SpotArgs, unsigned long long *) {
+static SplitKernel pick_split(const SpotArgs &a) {
   if (a.wstats)
-    return a.interp ? (a.has_div ? spots_split_kernel<1, 1, 1, FF>
-                                 : spots_split_kernel<1, 0, 1, FF>)
-                    : (a.has_div ? spots_split_kernel<0, 1, 1, FF>
-                                 : spots_split_kernel<0, 0, 1, FF>);
-  return a.interp ? (a.has_div ? spots_split_kernel<1, 1, 0, FF>
-                               : spots_split_kernel<1, 0, 0, FF>)
-                  : (a.has_div ? spots_split_kernel<0, 1, 0, FF>
-                               : spots_split_kernel<0, 0, 0, FF>);
+    return a.interp ? pick_split<1, 1, FF>(a) : pick_split<0, 1, FF>(a);
+  return a.interp ? pick_split<1, 0, FF>(a) : pick_split<0, 0, FF>(a);
 }
 
 size_t split_smem_bytes(const SpotArgs &a) {
