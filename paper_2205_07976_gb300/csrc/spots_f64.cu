@@ -238,11 +238,15 @@ cudaError_t build_f64_table(const float *F, long long n, double *F64t,
   return cudaGetLastError();
 }
 
-// 2^lsplit neighbouring lanes share a pixel (f64_split): 2^lk of them take
-// every 2^lk-th source, each with the orientations of its residue
+// 2^(lu + lk + lm) neighbouring lanes share a pixel (f64_split): each takes
+// every 2^lu-th unit, of those every 2^lk-th source, and of those every 2^lm-th
+// orientation
+struct F64Split {
+  int lu, lk, lm;
+};
 template <int SHAPE, int INTERP>
 __global__ void __launch_bounds__(kTileThreads, 4)
-    spots_f64_kernel(SpotArgs a, int lsplit, int lk) {
+    spots_f64_kernel(SpotArgs a, F64Split sp) {
   extern __shared__ double sm[];
   double *s_ax = sm;
   double *s_src = sm + a.PM * 9;
@@ -251,11 +255,13 @@ __global__ void __launch_bounds__(kTileThreads, 4)
     s_src[i] = a.src64[i];
   __syncthreads();
 
+  const int lsplit = sp.lu + sp.lk + sp.lm;
   const long long slot =
       ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> lsplit;
   const int part = threadIdx.x & ((1 << lsplit) - 1);
-  const int k0 = part & ((1 << lk) - 1), dk = 1 << lk, m0 = part >> lk,
-            dm = 1 << (lsplit - lk);
+  const int du = 1 << sp.lu, dk = 1 << sp.lk, dm = 1 << sp.lm;
+  const int u0 = part & (du - 1), k0 = (part >> sp.lu) & (dk - 1),
+            m0 = part >> (sp.lu + sp.lk);
   long long gp = 0;
   int q = 0, s = 0, fp = 0;
   const bool ok =
@@ -266,49 +272,49 @@ __global__ void __launch_bounds__(kTileThreads, 4)
   const double px = P.px;
   const int os = a.os;
   double acc = 0.0;
-  for (int i = 0; i < (ok ? os : 0); ++i) {
-    for (int j = 0; j < os; ++j) {
-      for (int t = 0; t < a.T; ++t) {
-        double cf = (fp + (i + 0.5) / os) * px,
-               cs = (s + (j + 0.5) / os) * px, cn = t * a.dt;
-        double pos[3], d[3];
+  const int U = ok ? os * os * a.T : 0;
+  for (int u = u0; u < U; u += du) {
+    const int t = u % a.T, i = u / a.T / os, j = u / a.T % os;
+    // (x / 1 is x: a division is ten FP64 instructions)
+    const double fi = os == 1 ? i + 0.5 : (i + 0.5) / os,
+                 fj = os == 1 ? j + 0.5 : (j + 0.5) / os;
+    double cf = (fp + fi) * px, cs = (s + fj) * px, cn = t * a.dt;
+    double pos[3], d[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
-          pos[c] = P.origin[c] + cf * P.fdir[c] + cs * P.sdir[c] +
-                   cn * P.ndir[c];
-        double R = sqrt(dot3d(pos, pos));
+    for (int c = 0; c < 3; ++c)
+      pos[c] = P.origin[c] + cf * P.fdir[c] + cs * P.sdir[c] +
+               cn * P.ndir[c];
+    double R = sqrt(dot3d(pos, pos));
 #pragma unroll
-        for (int c = 0; c < 3; ++c) d[c] = pos[c] / R;
-        double omega = px * px * dot3d(P.ndir, pos) / (R * R * R);
-        double cap = 1.0;
-        if (a.thickness > 0.0) {
-          double L = a.atten * dot3d(d, P.ndir);
-          cap = exp(-t * a.dt / L) - exp(-(t + 1) * a.dt / L);
-        }
-        for (int k = k0; k < a.S; k += dk) {
-          const double *src = s_src + k * SRC64_STRIDE;
-          const double lam = src[SRC64_LAM];
-          const double *dir = src + SRC64_DIR;
-          double Sv[3];
+    for (int c = 0; c < 3; ++c) d[c] = pos[c] / R;
+    double omega = px * px * dot3d(P.ndir, pos) / (R * R * R);
+    double cap = 1.0;
+    if (a.thickness > 0.0) {
+      double L = a.atten * dot3d(d, P.ndir);
+      cap = exp(-t * a.dt / L) - exp(-(t + 1) * a.dt / L);
+    }
+    for (int k = k0; k < a.S; k += dk) {
+      const double *src = s_src + k * SRC64_STRIDE;
+      const double lam = src[SRC64_LAM];
+      const double *dir = src + SRC64_DIR;
+      double Sv[3];
 #pragma unroll
-          for (int c = 0; c < 3; ++c) Sv[c] = (d[c] - dir[c]) / lam;
-          // Kahn: cos 2psi sin^2 2theta = (d.E')^2 - (d.B')^2 for unit d
-          double c2 = dot3d(d, dir), x = dot3d(d, src + SRC64_E),
-                 y = dot3d(d, src + SRC64_B);
-          double pol = 0.5 * (1.0 + c2 * c2 - a.kahn64 * (x * x - y * y));
-          // the step's factors that do not depend on phi x mosaic
-          const double wcpo = src[SRC64_W] * cap * pol * omega;
-          for (int pm = m0; pm < a.PM; pm += dm) {
-            const double *A = s_ax + pm * 9;
-            double h[3] = {dot3d(A, Sv), dot3d(A + 3, Sv), dot3d(A + 6, Sv)};
-            long long n[3];
-            double f[3];
-            nearest_f64(h, n, f);
-            const double a_ =
-                fcell_f64<INTERP>(a, f, n) * flatt_f64<SHAPE>(a, f);
-            acc = fma(a_ * a_, wcpo, acc);
-          }
-        }
+      for (int c = 0; c < 3; ++c) Sv[c] = (d[c] - dir[c]) / lam;
+      // Kahn: cos 2psi sin^2 2theta = (d.E')^2 - (d.B')^2 for unit d
+      double c2 = dot3d(d, dir), x = dot3d(d, src + SRC64_E),
+             y = dot3d(d, src + SRC64_B);
+      double pol = 0.5 * (1.0 + c2 * c2 - a.kahn64 * (x * x - y * y));
+      // the step's factors that do not depend on phi x mosaic
+      const double wcpo = src[SRC64_W] * cap * pol * omega;
+      for (int pm = m0; pm < a.PM; pm += dm) {
+        const double *A = s_ax + pm * 9;
+        double h[3] = {dot3d(A, Sv), dot3d(A + 3, Sv), dot3d(A + 6, Sv)};
+        long long n[3];
+        double f[3];
+        nearest_f64(h, n, f);
+        const double a_ =
+            fcell_f64<INTERP>(a, f, n) * flatt_f64<SHAPE>(a, f);
+        acc = fma(a_ * a_, wcpo, acc);
       }
     }
   }
@@ -321,27 +327,36 @@ __global__ void __launch_bounds__(kTileThreads, 4)
 // How many lanes share a pixel (log2).  The FP64 unit is a scheduler's own, so
 // a launch takes as long as the scheduler with the most warps: 307 x 211
 // pixels one per lane are 3.6 warps for each of the 608 schedulers, so 4 for
-// most.  Parts of at least 128 steps keep the repeated geometry (~130 FP64
-// instructions against 110 per sinc step) below 1 %, and a rule on the shot
-// alone keeps a pixel's value the same in every launch.  That shot (sinc, 2000
-// steps): 33.3 -> 30.2 ms.
-static int f64_split(const SpotArgs &a) {
+// most, and a list of 9216 pixels leaves half of them without a warp.  Units
+// are split as far as a power of two divides them, which repeats nothing (that
+// list with 8 units of 12 steps: 870 -> 490 us, half of it the list and the image copy); sources and orientations while
+// parts keep at least 128 steps, so that the repeated geometry (~130 FP64
+// instructions against 110 per sinc step) stays below 1 % (307 x 211 pixels,
+// sinc, 2000 steps: 33.3 -> 30.2 ms).  A rule on the shot alone keeps a pixel's
+// value the same in every launch.
+static F64Split f64_split(const SpotArgs &a) {
+  F64Split s = {0, 0, 0};
+  const int U = a.os * a.os * a.T;
+  while (s.lu < 5 && U % (2 << s.lu) == 0) ++s.lu;
   int l = 0;
-  while (l < 5 && ((long long)a.S * a.PM) >> (l + 1) >= 128) ++l;
-  return l;
+  while (s.lu + l < 5 && ((long long)a.S * a.PM) >> (l + 1) >= 128) ++l;
+  while (s.lk < l && 2 << s.lk <= a.S) ++s.lk;  // sources first
+  s.lm = l - s.lk;
+  return s;
 }
 
 cudaError_t launch_spots_f64(const SpotArgs &a, cudaStream_t st) {
   size_t smem = (size_t)(a.PM * 9 + a.S * SRC64_STRIDE) * sizeof(double);
-  const int lsplit = f64_split(a);
-  int lk = 0;  // as many sources side by side as there are
-  while (lk < lsplit && 2 << lk <= a.S) ++lk;
+  F64Split split = f64_split(a);
+  const long long most = a.pixlist ? a.n_list : (long long)a.n_tiles * kTileThreads;
+  if (most > 1ll << 32) split = {0, 0, 0};  // keeps the grid below 2^31
+  const int lsplit = split.lu + split.lk + split.lm;
   const long long pixels =
       a.pixlist ? a.n_list : (long long)a.n_tiles * kTileThreads;
   const long long blocks =
       ((pixels << lsplit) + kTileThreads - 1) / kTileThreads;
   if (blocks <= 0) return cudaSuccess;
-  void (*kern)(SpotArgs, int, int) = nullptr;
+  void (*kern)(SpotArgs, F64Split) = nullptr;
   int key = a.shape * 2 + a.interp;
   switch (key) {
     case 0: kern = spots_f64_kernel<0, 0>; break;
@@ -352,7 +367,7 @@ cudaError_t launch_spots_f64(const SpotArgs &a, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)blocks, kTileThreads, smem, st>>>(a, lsplit, lk);
+  kern<<<(unsigned)blocks, kTileThreads, smem, st>>>(a, split);
   return cudaGetLastError();
 }
 

@@ -27,6 +27,16 @@ def test_lanes_per_pixel(S, M, N, interp):
                                   nbgb.simulate(s, "f64")[sub])
 
 
+@pytest.mark.parametrize("os,T", [(2, 2), (3, 1), (2, 3), (1, 2), (8, 1)])
+@pytest.mark.parametrize("shape", [W.SHAPE_SINC, W.SHAPE_GAUSS])
+def test_units_shared_by_lanes(os, T, shape):
+    s = W.precision_shot(10, n_src=3, n_mosaic=4)
+    s.shape, s.oversample, s.n_layers = shape, os, T
+    s.thickness_m, s.atten_m = 4e-4, 3e-4
+    s = W.shrink(s, 19, 11, 610, 630)
+    check_f64(nbgb.simulate(s, "f64"), oracle.image(s))
+
+
 def test_lattice_points_ties_and_far_from_the_table():
     # h, k, l = -+ multiples of 1/2 (ties), exact lattice points, and values
     # beyond 2^30: axes along the components of d - i0 of single pixels
