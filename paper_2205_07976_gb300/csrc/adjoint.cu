@@ -44,7 +44,7 @@ struct AdjointArgs {
   double *partials;      // [blocks][kGradN]
   float kcs;             // r_e^2 fluence scale / (os^2 M Phi)
   // term-ring kernel: rows of 32 pixels handed to warps by a counter;
-  // partials holds one row of the ten sums per pixel row
+  // partials holds one row of the sums per pixel row
   unsigned long long *rows_next;
   long long n_rows;
 };
@@ -427,7 +427,18 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
 // its pixel, whose unit geometry and weight dL/dI K cap pol omega sit in a
 // per-warp table.  Each lane adds what it evaluates into FP32 sums, which
 // the warp folds into FP64 every 16 passes with a fixed butterfly, so the
-// ten scalars stay deterministic.
+// thirteen scalars stay deterministic.
+//
+// Bound by latency: 12 warps per SM (168 registers; the columns below take
+// 51 KB a block) issue in 47 % of the cycles.  The lanes run through a row of
+// sources, or up to a full ring, in one short loop; taking one step per trip
+// through the outer states cost 64-panel shot (S = 8, 10 domains, 18 % of
+// the steps surviving) 0.3 ms of 2.64.  Flushes of columns were next: a lane
+// per float4 of the column and one pass over a group's lanes where a lane
+// per float took four, 0.27 ms.  Tried beside it and slower or no faster:
+// columns swizzled over the banks (the updates then conflict), records not
+// sorted or grouped without an order (more flushes), records given to lanes
+// that hold their column (fewer flushes, a longer sort).
 constexpr int kAdjRing = 64;  // pending < 32 after a pass, + 32 pushed
 constexpr int kAdjFold = 16;  // passes between folds into FP64
 
@@ -494,8 +505,8 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   int held_key = -1;
   // Flushes, cooperatively, the columns of the lanes with `need`: lanes
   // with the same key are summed entry by entry (in FP32, in lane order)
-  // and each touched node gets one FP64 atomic; the 100 entries of a group
-  // are split over the 32 lanes.  Called by all lanes.
+  // and each touched node gets one FP64 atomic; lane r < 25 takes row r of
+  // the columns.  Called by all lanes.
   auto flush_columns = [&](bool need) {
     unsigned todo = __ballot_sync(0xffffffffu, need && held_key >= 0);
     while (todo) {
@@ -505,22 +516,26 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
       todo &= ~grp;
       const int c0 = (key & 1023) - 1, c1 = ((key >> 10) & 1023) - 1,
                 c2 = ((key >> 20) & 1023) - 1;
-      for (int e = lane; e < 100; e += 32) {
-        const int r = e >> 2, kk = e & 3;
-        float v = 0.f;
+      if (lane < 25) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         for (unsigned m = grp; m; m &= m - 1) {
-          float *col = reinterpret_cast<float *>(
-              &s_col[r][warp * 32 + __ffs(m) - 1]);
-          v += col[kk];
-          col[kk] = 0.f;
+          float4 *col = &s_col[lane][warp * 32 + __ffs(m) - 1];
+          const float4 c = *col;
+          v.x += c.x;
+          v.y += c.y;
+          v.z += c.z;
+          v.w += c.w;
+          *col = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        if (v != 0.f)
-          atomicAdd(g.gradF + nb_idx(a.check, NB_SITE_GRADF,
-                                     ((long long)(c0 - 2 + r / 5) * a.hn[1] +
-                                      (c1 - 2 + r % 5)) * a.hn[2] +
-                                         (c2 - 1 + kk),
-                                     table_size(a)),
-                    (double)v);
+        const long long at = ((long long)(c0 - 2 + lane / 5) * a.hn[1] +
+                              (c1 - 2 + lane % 5)) * a.hn[2] + (c2 - 1);
+        const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          if (vv[kk] != 0.f)
+            atomicAdd(g.gradF + nb_idx(a.check, NB_SITE_GRADF, at + kk,
+                                       table_size(a)),
+                      (double)vv[kk]);
       }
     }
     if (need) held_key = -1;
@@ -714,7 +729,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   // 32 entries of the pixel list) from a counter, and per pixel its steps
   // (unit, phi x mosaic, source): one step per iteration, the same
   // sequence in every lane.  The ring is drained before a unit's row of
-  // the unit table is rewritten and at the end of a pixel row, whose ten
+  // the unit table is rewritten and at the end of a pixel row, whose
   // sums then go to the row's own partial row: the sums do not depend on
   // which warp took which row.
   const int U = a.os * a.os * a.T;
@@ -807,9 +822,10 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
       }
       new_pm = false;
     }
-    // step (u, pm, k): the cheap cut test, then the exact offset of a
-    // surviving step and its record
-    {
+    // steps (u, pm, k ..) until the row of sources ends or the ring holds a
+    // pass: the cheap cut test, then the exact offset of a surviving step
+    // and its record
+    do {
       const float *src = s_src + k * SRC32_STRIDE;
       const float dh = src[SRC32_DH], dl = src[SRC32_DL];
       float fr[3], nf[3];
@@ -824,26 +840,28 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
       rad2 = fmaf(N2[2] * fr[2], fr[2], rad2);
       const bool hit = ok && rad2 <= cutg;
       const unsigned hm = __ballot_sync(0xffffffffu, hit);
-      if (hit) {
-        int npk = 0;
+      if (hm) {
+        if (hit) {
+          int npk = 0;
 #pragma unroll
-        for (int x = 0; x < 3; ++x) {
-          const float sx = fmaf(Gh[x], dh, __fsub_rn(rq[x], nf[x]));
-          fr[x] = sx + fmaf(Gh[x], dl, fmaf(Gl[x], dh, rl[x]));
-          const int nx = __float2int_rn(n0[x] + nf[x]) - a.hmin[x];
-          npk |= (min(max(nx, -1), a.hn[x]) + 1) << (10 * x);
+          for (int x = 0; x < 3; ++x) {
+            const float sx = fmaf(Gh[x], dh, __fsub_rn(rq[x], nf[x]));
+            fr[x] = sx + fmaf(Gh[x], dl, fmaf(Gl[x], dh, rl[x]));
+            const int nx = __float2int_rn(n0[x] + nf[x]) - a.hmin[x];
+            npk |= (min(max(nx, -1), a.hn[x]) + 1) << (10 * x);
+          }
+          const int slot =
+              (tail + __popc(hm & ((1u << lane) - 1u))) & (kAdjRing - 1);
+          rec_a[slot] = make_float4(fr[0], fr[1], fr[2], __int_as_float(npk));
+          rec_b[slot] = pm | (k << 11) | (lane << 21);
         }
-        const int slot =
-            (tail + __popc(hm & ((1u << lane) - 1u))) & (kAdjRing - 1);
-        rec_a[slot] = make_float4(fr[0], fr[1], fr[2], __int_as_float(npk));
-        rec_b[slot] = pm | (k << 11) | (lane << 21);
+        tail += __popc(hm);
       }
-      tail += __popc(hm);
-      __syncwarp();
-    }
+    } while (++k < a.S && tail - head < 32);
+    __syncwarp();
     // advance (u, pm, k); after the last step of the row's pixels the row
     // is done once its records are evaluated
-    if (++k == a.S) {
+    if (k == a.S) {
       k = 0;
       new_pm = true;
       if (++pm == a.PM) {
