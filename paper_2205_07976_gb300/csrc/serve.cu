@@ -31,6 +31,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <deque>
 #include <map>
 #include <string>
@@ -164,12 +165,23 @@ __global__ void __launch_bounds__(kSplitThreads, FORM == kLines ? kLineBlocks
         split_unit<0, FF>(base, P, s, f, lane - bi * U, unit + lane * kUnitFloats);
       }
       __syncwarp();
-      for (int bi = 0; bi < nb; ++bi) {
-        const long long p = w.first + warp + (long long)(i0 + bi) * kSplitWarps;
-        const double v = split_sum<INTERP, 0, FORM>(
-            base, b, unit + bi * U * kUnitFloats, cnt);
-        if (lane == 0) pool[sp.img_off + p] = sp.prefactor * v;
-      }
+      auto sum = [&](auto form) {
+        constexpr int F = decltype(form)::value, W = kLanes<F>;
+        for (int bi = 0; bi < nb; bi += 32 / W) {
+          const int pi = bi + (W == 32 ? 0 : lane / W);  // the lane's pixel
+          const bool ok = W == 32 || pi < nb;
+          const long long p =
+              w.first + warp + (long long)(i0 + pi) * kSplitWarps;
+          const double v = split_sum<INTERP, 0, F>(
+              base, b, unit + (ok ? pi : bi) * U * kUnitFloats, cnt, ok);
+          if ((lane & (W - 1)) == 0 && ok)
+            pool[sp.img_off + p] = sp.prefactor * v;
+        }
+      };
+      if (FORM != kLines && split_form(base, b.PM, b.S) == kHalves)
+        sum(std::integral_constant<int, kHalves>());
+      else
+        sum(std::integral_constant<int, FORM>());
       __syncwarp();  // the next batch rewrites the units
     }
     __syncthreads();  // the tables may be restaged for the next item
@@ -183,7 +195,7 @@ using ServeKernel = void (*)(SpotArgs, const SlotParams *, const WorkList *,
 template <bool FF>
 static ServeKernel pick_serve_warp(const SpotArgs &a, bool lines) {
   if (lines) return serve_warp_kernel<1, FF, kLines>;
-  return split_form(a, 1, 1) == kPairsEarly
+  return lattice_share(a) < kRareShare
              ? serve_warp_kernel<1, FF, kPairsEarly>
              : serve_warp_kernel<1, FF, kPairs>;
 }

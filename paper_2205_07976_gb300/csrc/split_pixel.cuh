@@ -536,26 +536,48 @@ struct PairQueue {
   int e0 = 0, en = 0, ch = 0, ct = 0;
 };
 
+// A warp sums one pixel with all its lanes, or one with every W of them: a
+// lane's place among its pixel's lanes, the first of them, and their bits of
+// a ballot.
+template <int W>
+struct Lanes {
+  static constexpr unsigned mask = W == 32 ? 0xffffffffu : (1u << (W & 31)) - 1u;
+  int l, first;
+  __device__ __forceinline__ Lanes() {
+    const int lane = threadIdx.x & 31;
+    l = lane & (W - 1);
+    first = lane & ~(W - 1);
+  }
+  __device__ __forceinline__ unsigned own(unsigned ballot) const {
+    return (ballot >> first) & mask;
+  }
+};
+// entries of the ring of a pixel's lanes
+template <int W>
+constexpr int kRing = kEntries * W / 32;
+
 // Appends one entry per lane with len > 0 pairs (or tasks), in lane order: the
 // state of the lane's item (r and d4 as SplitEntry describes) and the words
 // of SplitEntry::m.  Called by all lanes.
+template <int W = 32>
 __device__ __forceinline__ void push_entries(
     SplitEntry *ring, PairQueue &pq, int len, int mx, int my, int mw,
     const float Gh[3], const float r[3], const float Gl[3], const float rl[3],
     float4 d4) {
-  const int lane = threadIdx.x & 31;
-  const unsigned hm = __ballot_sync(0xffffffffu, len > 0);
-  if (hm == 0u) return;
+  const Lanes<W> at;
+  const unsigned any = __ballot_sync(0xffffffffu, len > 0);
+  if (any == 0u) return;
+  const unsigned hm = at.own(any);
   int inc = len;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
+  for (int o = 1; o < W; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o, W);
+    if (at.l >= o) inc += t;
   }
-  const int tot = __shfl_sync(0xffffffffu, inc, 31);
+  const int tot = __shfl_sync(0xffffffffu, inc, W - 1, W);
   if (len > 0) {
     SplitEntry &E =
-        ring[(pq.en + __popc(hm & ((1u << lane) - 1u))) & (kEntries - 1)];
+        ring[(pq.en + __popc(hm & ((1u << at.l) - 1u))) & (kRing<W> - 1)];
     E.a = make_float4(Gh[0], Gh[1], r[0], r[1]);
     E.b = make_float4(Gl[0], Gl[1], rl[0], rl[1]);
     E.c = make_float4(Gh[2], r[2], Gl[2], rl[2]);
@@ -567,37 +589,41 @@ __device__ __forceinline__ void push_entries(
   __syncwarp();
 }
 
-// Sums the next min(32, ct - ch) pairs of the queue, one per lane: the exact
+// Sums the next min(W, ct - ch) pairs of the queue, one per lane: the exact
 // fractional offset of the step, the cut test, and for a surviving step its
 // term (F_cell from the cell cache, F_latt, weight) into the lane's Kahan
-// sum.  Called by all lanes; returns the number of surviving terms.
-template <int INTERP, int HASDIV>
+// sum; none where `go` (the same in all of a pixel's lanes) is false.  Called
+// by all lanes; returns the number of the warp's surviving terms.
+template <int INTERP, int HASDIV, int W = 32>
 __device__ __forceinline__ unsigned sum_pairs(
     const SpotArgs &a, const SplitBlock &b, const SplitEntry *ring,
     PairQueue &pq, const float *unit, float4 *cache, int *tags, Kahan &acc,
-    unsigned &npairs) {
-  const int lane = threadIdx.x & 31;
-  const int np = min(32, pq.ct - pq.ch);
-  // entries e0 .. e0 + 31 can overlap the window [ch, ch + 32)
+    unsigned &npairs, bool go = true) {
+  const Lanes<W> at;
+  const int lane = at.l;
+  const int np = go ? min(W, pq.ct - pq.ch) : 0;
+  // entries e0 .. e0 + W - 1 can overlap the window [ch, ch + W)
   int4 mm = make_int4(0, 0, 0x7fffffff, 0);
-  if (pq.e0 + lane < pq.en) mm = ring[(pq.e0 + lane) & (kEntries - 1)].m;
+  if (pq.e0 + lane < pq.en) mm = ring[(pq.e0 + lane) & (kRing<W> - 1)].m;
   const bool ov = pq.e0 + lane < pq.en && mm.z < pq.ch + np &&
                   mm.z + mm.y > pq.ch;
   // bit j of M: some entry starts at pair ch + j (entry e0 at bit 0)
-  const unsigned M = __reduce_or_sync(
-      0xffffffffu, ov ? 1u << max(mm.z - pq.ch, 0) : 0u);
-  const int j = __popc(M & (0xffffffffu >> (31 - lane))) - 1;
-  const int k1 = __shfl_sync(0xffffffffu, mm.x, j);
-  const int pos = __shfl_sync(0xffffffffu, mm.z, j);
-  const int aux = __shfl_sync(0xffffffffu, mm.w, j);
-  const unsigned done =
-      __ballot_sync(0xffffffffu, ov && mm.z + mm.y <= pq.ch + np);
+  const unsigned M = at.own(__reduce_or_sync(
+      0xffffffffu, ov ? 1u << (at.first + max(mm.z - pq.ch, 0)) : 0u));
+  // (W < 32: a pixel without pairs in this pass reads some entry, unused)
+  const int j0 = __popc(M & (at.mask >> (W - 1 - lane))) - 1,
+            j = W == 32 ? j0 : max(j0, 0);
+  const int k1 = __shfl_sync(0xffffffffu, mm.x, j, W);
+  const int pos = __shfl_sync(0xffffffffu, mm.z, j, W);
+  const int aux = __shfl_sync(0xffffffffu, mm.w, j, W);
+  const unsigned done = at.own(
+      __ballot_sync(0xffffffffu, ov && mm.z + mm.y <= pq.ch + np));
   const bool valid = lane < np;
   const int k =
       valid ? (int)nb_idx(a.check, NB_SITE_SOURCE, k1 + (pq.ch + lane - pos),
                           b.S)
             : 0;
-  const SplitEntry &E = ring[(pq.e0 + j) & (kEntries - 1)];
+  const SplitEntry &E = ring[(pq.e0 + j) & (kRing<W> - 1)];
   const float4 A = E.a, B = E.b, C = E.c, D = E.d;
   const float Gh[3] = {A.x, A.y, C.x}, r[3] = {A.z, A.w, C.y};
   const float Gl[3] = {B.x, B.y, C.z}, rl[3] = {B.z, B.w, C.w};
@@ -1186,6 +1212,7 @@ __device__ __forceinline__ float4 entry_data(const SpotArgs &a, bool any,
 // sources whose delta range keeps some axis farther than sqrt(cut)/N_x from
 // every integer holds no surviving term.  Pushes block bb of every lane's
 // item that may hold one.
+template <int W = 32>
 __device__ __forceinline__ void push_block(const SplitBlock &b,
                                            SplitEntry *ring, PairQueue &pq,
                                            const SplitItem &t, int bb) {
@@ -1204,13 +1231,26 @@ __device__ __forceinline__ void push_block(const SplitBlock &b,
   }
   const int st0 = bb * kSrcBlock;
   const int len = pass ? min(kSrcBlock, b.S - st0) : 0;
-  push_entries(ring, pq, len, st0, len, t.aux, t.Gh, t.rq, t.Gl, t.rl,
-               make_float4(t.n0[0], t.n0[1], t.n0[2], t.scal));
+  push_entries<W>(ring, pq, len, st0, len, t.aux, t.Gh, t.rq, t.Gl, t.rl,
+                  make_float4(t.n0[0], t.n0[1], t.n0[2], t.scal));
 }
 
 // How split_sum goes through the interval entries: pair by pair; the same
-// with split_item's early test; line by line, with that test (split_form)
-enum { kPairs = 0, kPairsEarly = 1, kLines = 2 };
+// with split_item's early test; line by line, with that test; pair by pair,
+// two pixels at a time with 16 lanes each (split_form)
+enum { kPairs = 0, kPairsEarly = 1, kLines = 2, kHalves = 3 };
+constexpr int kHalfItems = 16, kHalfSteps = 128;
+constexpr float kHalfPairs = 30.f;
+template <int FORM>
+constexpr int kLanes = FORM == kHalves ? 16 : 32;  // lanes per pixel
+
+// The share of h space within the cut of a lattice point; they are rare where
+// it is below kRareShare
+constexpr float kRareShare = 0.2f;
+__host__ __device__ inline float lattice_share(const SpotArgs &a) {
+  const float m = sqrtf(kGaussCut * 0.63f) * 2.f;
+  return m / a.N[0] * (m / a.N[1]) * (m / a.N[2]);
+}
 
 // The form for a shot of PM orientations and S sources.  Lines need enough
 // tasks per pixel to fill a pass, and enough steps per line to pay for its
@@ -1221,15 +1261,23 @@ enum { kPairs = 0, kPairsEarly = 1, kLines = 2 };
 // points are rare: N = 25 (0.07 of h space lies within the cut) 1.22 -> 1.05
 // ms on 1500^2 pixels with S = 11, M = 9, but at N = 15 (0.34) it finds one in
 // most batches, 1.86 -> 2.11 ms on the 64-panel shot.
+// Halves pay where a pixel's items leave half the lanes idle (64-panel shot, 10
+// items of 8 sources, tricubic 1.83 -> 1.29 ms, nearest 1.47 -> 0.96; N = 25, 9
+// items of 11 0.337 -> 0.286).  A pixel alone then takes its pairs 16 at a time
+// with the other half idle, so a list of few pixels waits for the longer chain:
+// 1000 pixels, 100 steps at N = 15 (34 pairs expected) 36.4 -> 39.0 us, 480 steps
+// 45.7 -> 54.1, but 37.3 -> 37.7 with 99 steps at N = 25 (7 pairs); hence the
+// limits on steps and on expected pairs.
 __host__ __device__ inline int split_form(const SpotArgs &a, int PM, int S) {
   if (a.has_div) return kPairs;
   if ((a.interp == 0 || a.C4) && S >= kLineSources &&
       (long long)a.os * a.os * a.T * PM * S >= kLineSteps)
     return kLines;
-  // the share of h space within the cut of a lattice point, per axis
-  const float m = sqrtf(kGaussCut * 0.63f) * 2.f;
-  return m / a.N[0] * (m / a.N[1]) * (m / a.N[2]) < 0.2f ? kPairsEarly
-                                                          : kPairs;
+  const long long items = (long long)a.os * a.os * a.T * PM;
+  if (items <= kHalfItems && items * S <= kHalfSteps &&
+      (float)(items * S) * lattice_share(a) <= kHalfPairs)
+    return kHalves;
+  return lattice_share(a) < kRareShare ? kPairsEarly : kPairs;
 }
 
 // The sum, without the prefactor, of the pixel whose U sub-pixel units are
@@ -1240,9 +1288,11 @@ template <int INTERP, int HASDIV, int FORM, int COUNT = 0>
 __device__ __forceinline__ double split_sum(const SpotArgs &a,
                                             const SplitBlock &b,
                                             const float *unit,
-                                            SplitCounts &cnt) {
+                                            SplitCounts &cnt, bool ok = true) {
+  constexpr int W = kLanes<FORM>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  SplitEntry *ring = b.ent_base + warp * kEntries;
+  SplitEntry *ring =
+      b.ent_base + warp * kEntries + (W == 32 ? 0 : lane / W * kRing<W>);
   float4 *cache = b.cell_cache + warp * kCellChunks * kCellSlots;
   int *tags = b.cell_tags + warp * kCellSlots;
   const int items = a.os * a.os * a.T * b.PM;
@@ -1330,6 +1380,50 @@ __device__ __forceinline__ double split_sum(const SpotArgs &a,
           nblocks += __popc(__ballot_sync(0xffffffffu, t.valid)) * b.nblk;
       }
     }
+  } else if (FORM == kHalves) {
+    // Each half of the warp goes through its own pixel: a pixel's items fit
+    // its lanes, its pairs are taken 16 at a time when 16 are there (or at
+    // the end), whatever the other half holds, so a pixel's sum does not
+    // depend on its neighbour.
+    const Lanes<W> at;
+    const bool valid = ok && at.l < items;
+    const int u = valid ? at.l / b.PM : 0;
+    auto drain = [&]() {
+      while (true) {
+        const bool go = pq.ct - pq.ch >= W;
+        if (!__any_sync(0xffffffffu, go)) break;
+        nterms += sum_pairs<INTERP, 0, W>(a, b, ring, pq, unit, cache, tags,
+                                          acc, npairs, go);
+      }
+    };
+    split_item<false>(b, unit, u, valid ? at.l - u * b.PM : 0, valid, t);
+    lattice_range(b, N2, t, L);
+    const bool lat =
+        b.iv_ok && at.own(__ballot_sync(0xffffffffu, L.ncomb > 8)) == 0u;
+    const int mine = lat ? L.ncomb : 0;
+    const int maxc = (int)__reduce_max_sync(0xffffffffu, (unsigned)mine);
+    if (COUNT) nivals += __reduce_add_sync(0xffffffffu, (unsigned)mine);
+    for (int c = 0; c < maxc; ++c) {
+      lattice_interval(a, b, N2, t, L, c, k1, k2, dx, nt);
+      if (c >= mine) k2 = k1;
+      if (!__any_sync(0xffffffffu, k2 > k1)) continue;
+      push_entries<W>(ring, pq, k2 > k1 ? k2 - k1 : 0, k1, k2 - k1,
+                      t.aux | kIntervalEntry, t.Gh, dx, t.Gl, t.rl,
+                      entry_data<INTERP>(a, k2 > k1, nt, t.scal));
+      drain();
+    }
+    t.valid = t.valid && !lat;
+    const unsigned scan = __ballot_sync(0xffffffffu, t.valid);
+    if (scan) {
+      if (COUNT) nblocks += __popc(scan) * b.nblk;
+      for (int bb = 0; bb < b.nblk; ++bb) {
+        push_block<W>(b, ring, pq, t, bb);
+        drain();
+      }
+    }
+    if (__any_sync(0xffffffffu, pq.ct > pq.ch))
+      nterms += sum_pairs<INTERP, 0, W>(a, b, ring, pq, unit, cache, tags, acc,
+                                        npairs);
   } else {
     auto drain = [&]() {
       while (pq.ct - pq.ch >= 32)
@@ -1396,7 +1490,7 @@ __device__ __forceinline__ double split_sum(const SpotArgs &a,
   float hi, lo;
   fast_two_sum(acc.s, -acc.c, hi, lo);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = W / 2; o > 0; o >>= 1) {
     const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
     const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
     float sh, se;

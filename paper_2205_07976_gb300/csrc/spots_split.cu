@@ -32,7 +32,10 @@
 //      place of ~8 per lane and step of the pair queue (sum_tasks).  Large
 //      shot: 164.5 -> 104.7 ms; the 512^2 pixels at its centre, where the
 //      batches of items without a lattice point in reach end early, 5.0 -> 2.6;
-//   4. the 32 lane sums are reduced with warp shuffles in float-float.
+//      In shots of few items and steps per pixel (split_form) each half of the
+//      warp takes a pixel of its own: with 10 items a pixel's pass over its
+//      items left 22 lanes idle;
+//   4. a pixel's lane sums are reduced with warp shuffles in float-float.
 // The order of every operation depends only on the pixel's own inputs, so
 // a pixel's value does not depend on what else is in the launch.
 // Pixels are handed to warps through an atomic counter in a scratch word.
@@ -62,7 +65,11 @@ __global__ void __launch_bounds__(kSplitThreads, FORM == kLines ? kLineBlocks : 
   const long long most =
       per_warp >= 256 ? kMaxUnits
       : (long long)U * a.PM * a.S <= 8192 ? per_warp / 16 : 1;
-  const int B = (int)max(1ll, min((long long)(kMaxUnits / U), most));
+  // (as many as the warp sums side by side where it gets so many)
+  constexpr int W = kLanes<FORM>;
+  const long long least = per_warp >= 32 / W ? 32 / W : 1;
+  const int B =
+      (int)max(1ll, min((long long)(kMaxUnits / U), max(most, least)));
   float *unit = b.unit_base + warp * kMaxUnits * kUnitFloats;
   while (true) {
     long long first = 0;
@@ -81,10 +88,18 @@ __global__ void __launch_bounds__(kSplitThreads, FORM == kLines ? kLineBlocks : 
     }
     __syncwarp();
     double mine = 0.0;  // lane bi keeps the sum of pixel bi
-    for (int bi = 0; bi < nb; ++bi) {
+    for (int bi = 0; bi < nb; bi += 32 / W) {
+      const int pi = bi + (W == 32 ? 0 : lane / W);  // this lane's pixel
+      const bool ok = W == 32 || pi < nb;
       const double v = split_sum<INTERP, HASDIV, FORM, COUNT>(
-          a, b, unit + bi * U * kUnitFloats, cnt);
-      if (lane == bi) mine = v;
+          a, b, unit + (ok ? pi : bi) * U * kUnitFloats, cnt, ok);
+      if (W == 32) {
+        if (lane == bi) mine = v;
+      } else {
+        const double got =
+            __shfl_sync(0xffffffffu, v, (lane - bi) * W & 31);
+        if (lane >= bi && lane < bi + 32 / W) mine = got;
+      }
     }
     // fused accumulate into the image: lanes 0 .. nb-1 add the batch's
     // pixels, consecutive in the image, in one coalesced access
@@ -110,6 +125,7 @@ static SplitKernel pick_split(const SpotArgs &a) {
   if (a.has_div) return spots_split_kernel<INTERP, 1, COUNT, FF, kPairs>;
   switch (split_form(a, a.PM, a.S)) {
     case kLines: return spots_split_kernel<INTERP, 0, COUNT, FF, kLines>;
+    case kHalves: return spots_split_kernel<INTERP, 0, COUNT, FF, kHalves>;
     // (the early test changes no sum and no count: not built with counters)
     case kPairsEarly:
       if (!COUNT)
