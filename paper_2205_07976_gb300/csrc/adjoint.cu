@@ -135,11 +135,12 @@ __device__ __forceinline__ void lagrange4_deriv(float x, float w[4]) {
 
 // One thread per pixel (nearest lookup, and tricubic lookup in tables too
 // long for the ring kernel below).  Bound by instruction issue: per (pixel,
-// orientation) about 150 for the double-float G and r, 20 per source for the
+// orientation) about 150 for the double-float G and r, 12 per source for the
 // cut test, and the evaluation of the surviving steps with 18 % of them
 // surviving.  64-panel shot (S = 8, 10 domains, nearest): 1316 -> 880 us with
 // the nine products Q in place of 18 per orientation, FP32 sums folded by
-// warp, and each lane taking its own surviving steps.
+// warp, and each lane taking its own surviving steps; -> 795 with the cut
+// tested two sources at a time (cut_sums).
 template <int HASF, int INTERP>
 __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
     spots_adjoint_kernel(AdjointArgs g) {
@@ -255,18 +256,15 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
             for (int k0 = 0; k0 < a.S; k0 += 32) {
             unsigned hits = 0;
             const int nk = min(32, a.S - k0);
-            for (int j = 0; j < nk; ++j) {
-              const float dh = s_src[(k0 + j) * SRC32_STRIDE + SRC32_DH];
-              float fr[3];
-#pragma unroll
-              for (int x = 0; x < 3; ++x) {
-                const float tq = fmaf(Gh[x], dh, rq[x]);
-                fr[x] = tq - rintf(tq);
-              }
-              float rad2 = N2[0] * fr[0] * fr[0];
-              rad2 = fmaf(N2[1] * fr[1], fr[1], rad2);
-              rad2 = fmaf(N2[2] * fr[2], fr[2], rad2);
-              if (!(rad2 > cutg)) hits |= 1u << j;
+            for (int j = 0; j < nk; j += 2) {
+              const float *src = s_src + (k0 + j) * SRC32_STRIDE;
+              const bool two = j + 1 < nk;
+              const float2 rad2 = cut_sums(
+                  Gh, rq, a.N,
+                  make_float2(src[SRC32_DH],
+                              src[two ? SRC32_STRIDE + SRC32_DH : SRC32_DH]));
+              if (!(rad2.x > cutg)) hits |= 1u << j;
+              if (two && !(rad2.y > cutg)) hits |= 2u << j;
             }
             while (hits) {
               const float *src =
@@ -832,7 +830,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
         const float tq = fmaf(Gh[x], dh, rq[x]);
-        nf[x] = rintf(tq);
+        nf[x] = __fsub_rn(__fadd_rn(tq, kRoundAdd), kRoundAdd);  // rint
         fr[x] = tq - nf[x];
       }
       float rad2 = N2[0] * fr[0] * fr[0];

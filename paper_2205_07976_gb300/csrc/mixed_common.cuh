@@ -343,4 +343,29 @@ __device__ __forceinline__ float fcell_f32(const SpotArgs &a, const int n[3],
   return a.defF;
 }
 
+constexpr float kRoundAdd = 12582912.f;  // 1.5 * 2^23: x + it - it = rint(x)
+
+// Exponent sums sum N_x^2 f_x^2 of the steps of two sources (delta_hi in dh),
+// f_x the offset of G_x delta + r_x from its nearest integer, for the cut test
+// (|G_x delta + r_x| < 2^22: the rounding is an addition, which leaves the unit
+// of conversions and reciprocals, 16 lanes wide, to the terms).  The nearest
+// adjoint on the 64-panel shot (S = 8, 10 domains): 880 -> 795 us; the forward
+// thread kernel gained nothing from it (1.76 ms per refinement step both ways).
+__device__ __forceinline__ float2 cut_sums(const float G[3], const float r[3],
+                                           const float N[3], float2 dh) {
+  const float2 up = make_float2(kRoundAdd, kRoundAdd),
+               down = make_float2(-kRoundAdd, -kRoundAdd),
+               minus = make_float2(-1.f, -1.f);
+  float2 rad = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    const float2 t =
+        ffma2(make_float2(G[x], G[x]), dh, make_float2(r[x], r[x]));
+    const float2 n = fadd2(fadd2(t, up), down);
+    const float2 f = fmul2(ffma2(n, minus, t), make_float2(N[x], N[x]));
+    rad = x ? ffma2(f, f, rad) : fmul2(f, f);
+  }
+  return rad;
+}
+
 }  // namespace nbgb
