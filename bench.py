@@ -53,12 +53,12 @@ MAX_SM_MHZ = 2070.0  # GB300's maximum SM clock
 # kernel, from one ncu capture (profiles/spots_split_large_shot_dram.txt:
 # the mean of two launches);
 # valid only while the kernel sources hash to the value they had then
-TRAFFIC_CAPTURE = {"bytes": (80408320 + 22961920 + 80121344 + 23371520) // 2,
+TRAFFIC_CAPTURE = {"bytes": (80293376 + 27656192 + 80080640 + 28163328) // 2,
                    "sources": ["paper_2205_07976_gb300/csrc/spots_split.cu",
                                "paper_2205_07976_gb300/csrc/split_pixel.cuh",
                                "paper_2205_07976_gb300/csrc/mixed_common.cuh",
                                "paper_2205_07976_gb300/csrc/nbgb_internal.cuh"],
-                   "sha256_16": "068389bc3a988e15"}
+                   "sha256_16": "a52943de1b33279a"}
 
 
 def captured_traffic():
@@ -75,13 +75,14 @@ def captured_traffic():
 # Pipe utilisation (% of active cycles) of the warp-per-pixel kernel from
 # one ncu --set full capture on a 512x512 window of the large shot
 # (profiles/spots_split_window512_full.txt), keyed like the traffic figure
-PIPES_CAPTURE = {"sm__pipe_fma_cycles_active_pct": 36.3,
-                 "sm__pipe_alu_cycles_active_pct": 40.1,
-                 "sm__inst_executed_pipe_lsu_pct": 41.3,
-                 "smsp__issue_active_pct": 74.1,
-                 "l1tex__data_pipe_lsu_wavefronts_pct": 54.5,
+PIPES_CAPTURE = {"sm__pipe_fma_cycles_active_pct": 27.6,
+                 "sm__pipe_alu_cycles_active_pct": 34.2,
+                 "sm__inst_executed_pipe_lsu_pct": 16.3,
+                 "sm__pipe_fp64_cycles_active_pct": 36.3,
+                 "smsp__issue_active_pct": 55.7,
+                 "l1tex__data_pipe_lsu_wavefronts_pct": 43.3,
                  "window": "512x512 centred on the large shot",
-                 "sha256_16": "068389bc3a988e15"}
+                 "sha256_16": "a52943de1b33279a"}
 
 
 def captured_pipes():
@@ -425,7 +426,10 @@ def run_e2e(args, sim, shot, world, pg, torch, np, nbgb):
 
 
 def run_f64(args, shot, local, stream, torch, nbgb, W):
-    """The plain FP64 form on every n-th row of the same shot."""
+    """The FP64 form on every n-th row of the same shot.  Its kernel leaves out
+    the steps that a bound shows to be below 2^-56 of the pixel's sum; the
+    counted rate credits every step of the definition, so it can exceed the
+    peak and is a rate of the method's work, not of the unit's activity."""
     rows = W.strided_rows(shot, args.f64_rows_every)
     sim64 = nbgb.Sim("f64", device=local, stream=stream).set_shot(shot)
     sim64.add_spots(rows)
@@ -450,7 +454,10 @@ def run_f64(args, shot, local, stream, torch, nbgb, W):
             "roofline": {"bound": "fp64", "achieved": achieved,
                          "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak if peak > 0 else None,
-                         "kernel": "spots_f64_kernel",
+                         "counts": "every step of the definition (those "
+                                   "below 2^-56 of a pixel's sum are left "
+                                   "out, so frac can exceed 1)",
+                         "kernel": "spots_f64_warp_kernel",
                          "peak_source": "measured: independent FP64 FMA "
                                         "chains on every SM "
                                         "(nb_fp64_peak_tflops)"}}

@@ -329,11 +329,11 @@ __global__ void __launch_bounds__(kTileThreads, 4)
 // pixels one per lane are 3.6 warps for each of the 608 schedulers, so 4 for
 // most, and a list of 9216 pixels leaves half of them without a warp.  Units
 // are split as far as a power of two divides them, which repeats nothing (that
-// list with 8 units of 12 steps: 870 -> 490 us, half of it the list and the image copy); sources and orientations while
-// parts keep at least 128 steps, so that the repeated geometry (~130 FP64
-// instructions against 110 per sinc step) stays below 1 % (307 x 211 pixels,
-// sinc, 2000 steps: 33.3 -> 30.2 ms).  A rule on the shot alone keeps a pixel's
-// value the same in every launch.
+// list with 8 units of 12 steps: 870 -> 490 us, half of it the list and the
+// image copy); sources and orientations while parts keep at least 128 steps, so
+// that the repeated geometry (~130 FP64 instructions against 110 per sinc step)
+// stays below 1 % (307 x 211 pixels, sinc, 2000 steps: 33.3 -> 30.2 ms).  A
+// rule on the shot alone keeps a pixel's value the same in every launch.
 static F64Split f64_split(const SpotArgs &a) {
   F64Split s = {0, 0, 0};
   const int U = a.os * a.os * a.T;
