@@ -892,18 +892,24 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
   const float Gh[3] = {Ea.x, Ea.y, Ec.x}, dx[3] = {Ea.z, Ea.w, Ec.y};
   const float Gl[3] = {Eb.x, Eb.y, Ec.z}, rl[3] = {Eb.z, Eb.w, Ec.w};
   const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
-  // the middle source is the origin of the line
-  const int mid = (p + e) >> 1;
-  const float4 sm =
-      *reinterpret_cast<const float4 *>(b.src + mid * SRC32_STRIDE);
-  const float half = fmaxf(b.dh[max(e - 1, 0)] - sm.z, sm.z - b.dh[p]);
+  // The origin of the line is the mean of the first and the last source: its
+  // offsets' signs name the segment's cell even where rounding put a source at
+  // a sign change on the other side of the cut (line_segments compares with
+  // an approximate quotient).  A source's own signs would then name the
+  // neighbouring cell, and the other sources be extrapolated from it.
+  const float4 sf = *reinterpret_cast<const float4 *>(
+                   b.src + p * SRC32_STRIDE),
+               sl = *reinterpret_cast<const float4 *>(
+                   b.src + max(e - 1, 0) * SRC32_STRIDE);
+  const float dm = 0.5f * (sf.z + sl.z), dml = 0.5f * (sf.x + sl.x);
+  const float half = 0.5f * (sl.z - sf.z);
   const float ih = half > 0.f ? __fdividef(1.f, half) : 0.f;
   float f0[3], fl0[3], g[3];
   float A = 0.f, Bq = 0.f;
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
-    const float sx = fmaf(Gh[x], sm.z, dx[x]);
-    const float c = fmaf(Gh[x], sm.x, fmaf(Gl[x], sm.z, rl[x]));
+    const float sx = fmaf(Gh[x], dm, dx[x]);
+    const float c = fmaf(Gh[x], dml, fmaf(Gl[x], dm, rl[x]));
     f0[x] = __fadd_rn(sx, c);
     fl0[x] = __fsub_rn(c, __fsub_rn(f0[x], sx));
     g[x] = Gh[x] * half;
@@ -945,8 +951,8 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
   if (__all_sync(0xffffffffu, line)) {
     const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
     const float *src = b.src + p * SRC32_STRIDE + SRC32_PAIR;
-    const f32x2 ih2 = splat2(ih), rl2 = splat2(-sm.x * ih),
-                rh2 = splat2(-sm.z), ts2 = splat2(-ts), cA2 = splat2(cA),
+    const f32x2 ih2 = splat2(ih), rl2 = splat2(-dml * ih),
+                rh2 = splat2(-dm), ts2 = splat2(-ts), cA2 = splat2(cA),
                 e02 = splat2(e0);
     f32x2 q2[10];
     if (INTERP == 1) {
