@@ -841,6 +841,20 @@ __device__ __forceinline__ void line_segments(const SplitBlock &b, int k1,
   mw = b1 | (b2 << 11);
 }
 
+// The table-relative lattice point of a line entry (entry_data)
+template <int INTERP>
+__device__ __forceinline__ void entry_index(const float4 &d, int nt[3]) {
+  if (INTERP == 1) {
+    const int npk = __float_as_int(d.y);
+#pragma unroll
+    for (int x = 0; x < 3; ++x) nt[x] = ((npk >> (10 * x)) & 1023) - 1;
+  } else {
+    nt[0] = __float_as_int(d.x);
+    nt[1] = __float_as_int(d.y);
+    nt[2] = __float_as_int(d.z);
+  }
+}
+
 // Sums the next min(32, ct - ch) tasks of a queue of line entries, one per
 // lane, into the lane's Kahan sum.  Called by all lanes; returns the lane's
 // number of steps under the cut and adds its steps to npairs.
@@ -928,12 +942,7 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
   const float e0 = -kLog2 * R, cA = -kLog2 * A;
   float q[10], Fn = 0.f;
   bool line = true;  // the segment's cell lies in the table
-  int nt[3];
   if (INTERP == 1) {
-    const int npk = __float_as_int(Ed.y);
-    nt[0] = (npk & 1023) - 1;
-    nt[1] = ((npk >> 10) & 1023) - 1;
-    nt[2] = ((npk >> 20) & 1023) - 1;
     CellRef c;
     cell_of_entry(a, n > 0, f0, __float_as_int(Ed.x), __float_as_int(Ed.z), c);
     line = c.tri || n == 0;
@@ -941,14 +950,22 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
       cell_line(a.C4 + (size_t)nb_idx(a.check, NB_SITE_CELL, c.ci,
                                       cell_count(a)) * kCellChunks,
                 c.x, g, q);
-  } else {
-    nt[0] = __float_as_int(Ed.x);
-    nt[1] = __float_as_int(Ed.y);
-    nt[2] = __float_as_int(Ed.z);
-    if (n) Fn = fcell_f32<0>(a, nt, f0);
+  } else if (n) {
+    int nt[3];
+    entry_index<INTERP>(Ed, nt);
+    Fn = fcell_f32<0>(a, nt, f0);
   }
   unsigned hits = 0;
-  if (__all_sync(0xffffffffu, line)) {
+  // chunks of 16 steps to be summed step by step, from the table: all of them
+  // where some lane's cell reaches out of the table; and those whose sum is
+  // not finite, as a line multiplies the steps beyond the cut (and beyond an
+  // odd end) by zero, which a table entry that is not finite, or whose square
+  // is not, does not survive
+  unsigned redo = 0;
+  const bool lines = __all_sync(0xffffffffu, line);
+  if (!lines) {
+    redo = ~0u;
+  } else {
     const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
     const float *src = b.src + p * SRC32_STRIDE + SRC32_PAIR;
     const f32x2 ih2 = splat2(ih), rl2 = splat2(-dml * ih),
@@ -994,11 +1011,24 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
         }
       }
       const float2 sum = upk2(sum2);
-      acc.add((sum.x + sum.y) * fac);
+      const float v = (sum.x + sum.y) * fac;
+      if (fabsf(v) <= 3.4e38f)
+        acc.add(v);
+      else
+        redo |= 1u << (i0 >> 4);
     }
-  } else {
-    // some lane's cell reaches out of the table: step by step from the table
+  }
+  if (__any_sync(0xffffffffu, redo != 0u)) {
+    // the entry read again: kept in registers it would cost the loop above
+    // (large shot 101.8 -> 105.9 ms)
+    asm volatile("" ::: "memory");
+    const float4 Ea = E4.a, Eb = E4.b, Ec = E4.c, Ed = E4.d;
+    const float Gh[3] = {Ea.x, Ea.y, Ec.x}, dx[3] = {Ea.z, Ea.w, Ec.y};
+    const float Gl[3] = {Eb.x, Eb.y, Ec.z}, rl[3] = {Eb.z, Eb.w, Ec.w};
+    int nt[3];
+    entry_index<INTERP>(Ed, nt);
     for (int i = 0; i < n; ++i) {
+      if (!(redo >> (i >> 4) & 1u)) continue;
       const float4 sw = *reinterpret_cast<const float4 *>(
           b.src + (p + i) * SRC32_STRIDE);
       float fr[3], rad2 = 0.f;
@@ -1012,7 +1042,7 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
         const float F = fcell_f32<INTERP>(a, nt, fr);
         acc.add(F * F * (a.N6 * __expf(-2.f * rad2 * (1.f / 0.63f))) *
                 (sw.y * Ed.w));
-        ++hits;
+        hits += !lines;  // (a line has counted its own)
       }
     }
   }

@@ -1,5 +1,7 @@
-"""The line form (test_split_lines_gpu) where a line's cell changes: sources
-right at an offset's sign change.  Tolerance: the mixed form's own, 1e-5."""
+"""The line form (test_split_lines_gpu) where a line's cell changes and where
+its table is special: sources right at an offset's sign change, and entries
+that are not finite.  Tolerances: the mixed form's own, 1e-5; which pixels are
+finite is exact."""
 import numpy as np
 import pytest
 
@@ -8,6 +10,8 @@ from paper_2205_07976_gb300 import nbgb
 from paper_2205_07976_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
+
+CUT = 44.0 * 0.63  # steps with sum N^2 f^2 above this have no FP32 term
 
 
 def _pixel_shot(u, N, axes, d, px=1e-4):
@@ -59,3 +63,55 @@ def test_sources_at_a_sign_change():
         assert ref[0] > 0
         worst = max(worst, abs(got[0] - ref[0]) / ref[0])
     assert worst <= 1e-5, worst
+
+
+def _reach(s, entry):
+    """Per pixel: whether a step under the cut uses the table entry, and
+    whether one might, up to the FP32 rounding of the cut and of a cell's
+    boundary."""
+    p = s.panels[0]
+    ij = np.stack(np.meshgrid(np.arange(p.nslow), np.arange(p.nfast),
+                              indexing="ij"), -1).reshape(-1, 2) + 0.5
+    pos = (p.origin + p.pixel_m * (ij[:, 1:] * p.fdir + ij[:, :1] * p.sdir))
+    v = pos / np.linalg.norm(pos, axis=1, keepdims=True) - s.dirs[0]
+    sure = np.zeros(len(pos), bool)
+    maybe = np.zeros(len(pos), bool)
+    for um in s.umats:
+        g = v @ (s.axes @ um.T).T
+        h = g[:, None, :] / s.lambdas[None, :, None]
+        n = np.rint(h)
+        f = h - n
+        r = np.sum((s.ncells * f) ** 2, -1)
+        if s.interp == W.INTERP_NEAREST:
+            use = near = np.all(n == entry, -1)
+        else:
+            lo = np.floor(h) - 1
+            use = np.all((entry >= lo) & (entry <= lo + 3), -1)
+            lo_d, lo_u = np.floor(h - 1e-6) - 1, np.floor(h + 1e-6) - 1
+            near = np.all((entry >= lo_d) & (entry <= lo_u + 3), -1)
+            use &= np.all(lo_d == lo_u, -1)
+        sure |= np.any(use & (r <= CUT * (1 - 1e-4)), 1)
+        maybe |= np.any(near & (r <= CUT * (1 + 1e-4)), 1)
+    return sure, maybe
+
+
+@pytest.mark.parametrize("interp", [W.INTERP_NEAREST, W.INTERP_TRICUBIC])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, 3e38])
+def test_table_entries_that_are_not_finite(interp, bad):
+    """A pixel is not finite exactly where a step under the cut uses the
+    entry (3e38: its square is not)."""
+    s = W.large_shot(n_src=100, n_mosaic=12)
+    s.oversample, s.n_layers, s.thickness_m, s.interp = 1, 1, 0.0, interp
+    s = W.shrink(s, 61, 47, 2433 - 30, 890 - 23)
+    p = s.panels[0]
+    pos = p.origin + p.pixel_m * (30.0 * p.fdir + 23.0 * p.sdir)
+    h = s.axes @ (pos / np.linalg.norm(pos) - s.dirs[0]) / s.lambdas[50]
+    entry = np.rint(h).astype(int)
+    s.F = s.F.copy()
+    s.F[tuple(entry - s.hkl_min)] = bad
+    sure, maybe = _reach(s, entry)
+    assert sure.any() and not maybe.all()
+    for variant in ("warp", "thread"):
+        ok = np.isfinite(nbgb.simulate(s, "mixed", variant=variant))
+        assert not ok[sure].any(), variant
+        assert ok[~maybe].all(), (variant, int((~ok[~maybe]).sum()))
