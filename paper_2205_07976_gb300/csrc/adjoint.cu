@@ -28,10 +28,10 @@
 // so the kernels sum the nine products Q_xc = e_x v'_c over all steps, and the
 // host contracts them once with the six derivatives of the lab axes.  (Forming
 // the 18 products dA_x · v of every orientation, and 18 FMAs per term, took
-// 54 shared loads and 54 FMAs per orientation.)  The thirteen sums go per
-// thread into FP32, per warp into a butterfly, from there into FP64 and
-// per block or pixel row into a partial row; the rows are added in a fixed
-// order.
+// 54 shared loads and 54 FMAs per orientation.)  The thirteen sums are FP32
+// over a limited number of steps (a unit's in the thread kernel, 16 passes of a
+// warp in the ring kernel) and FP64 from there on; per block or pixel row they
+// go into a partial row, and the rows are added in a fixed order.
 #include "mixed_common.cuh"
 
 namespace nbgb {
@@ -42,15 +42,16 @@ struct AdjointArgs {
   const double *dLdI;    // [npix]
   double *gradF;         // [nh*nk*nl], accumulated into
   double *partials;      // [blocks][kGradN]
-  float kcs;             // r_e^2 fluence scale / (os^2 M Phi)
+  double kc;             // r_e^2 fluence / (os^2 M Phi)
+  double scale;
   // term-ring kernel: rows of 32 pixels handed to warps by a counter;
   // partials holds one row of the sums per pixel row
   unsigned long long *rows_next;
   long long n_rows;
 };
 
-// the sums: Q_xc (3 x + c), the three dL/dN and dL/dscale, without the
-// prefactor
+// the sums, each step weighted with dL/dI kc: Q_xc (3 x + c), the three dL/dN
+// (both without the scale) and dL/dscale
 constexpr int kGradN = 13;
 static_assert(kGradN == kAdjointSums, "the host contracts these sums");
 
@@ -138,9 +139,12 @@ __device__ __forceinline__ void lagrange4_deriv(float x, float w[4]) {
 // orientation) about 150 for the double-float G and r, 12 per source for the
 // cut test, and the evaluation of the surviving steps with 18 % of them
 // surviving.  64-panel shot (S = 8, 10 domains, nearest): 1316 -> 880 us with
-// the nine products Q in place of 18 per orientation, FP32 sums folded by
-// warp, and each lane taking its own surviving steps; -> 795 with the cut
-// tested two sources at a time (cut_sums).
+// the nine products Q in place of 18 per orientation and each lane taking its
+// own surviving steps; -> 795 with the cut tested two sources at a time
+// (cut_sums).  A unit's sums are FP32 (dL/dscale compensated); over the units,
+// dL/dI and the pixels they are FP64 (refinement step 1.63 -> 1.66 ms).  All
+// of them FP32 over a pixel's 40 000 steps put dL/dN and dL/dscale off by 3e-6
+// to 1.3e-5 in place of 1e-8 to 8e-7.
 template <int HASF, int INTERP>
 __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
     spots_adjoint_kernel(AdjointArgs g) {
@@ -192,20 +196,19 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   if (INTERP && HASF)
     for (int e = 0; e < 125; ++e) s_facc[e][threadIdx.x] = 0.f;
 
-  float acc[kGradN];
-#pragma unroll
-  for (int r = 0; r < kGradN; ++r) acc[r] = 0.f;
-
   long long item = a.pixlist ? (long long)blockIdx.x * blockDim.x + threadIdx.x
                              : (long long)blockIdx.x;
-  long long gp;
-  int q, s, f;
-  if (map_pixel(a, item, threadIdx.x, gp, q, s, f)) {
-    const DevPanel &P = a.panels[q];
+  long long gp = 0;
+  int q = 0, s = 0, f = 0;
+  const int lane = threadIdx.x & 31;
+  double mine = 0.0;  // lanes 2 r and 2 r + 1: the warp's sum r
+  {
+    const bool ok = map_pixel(a, item, threadIdx.x, gp, q, s, f);
+    const DevPanel &P = a.panels[ok ? q : 0];
     const int os = a.os;
     const float kahn = a.kahn;
     const float cutg = kGaussCut * 0.63f;
-    const float wp = (float)g.dLdI[gp];
+    const double wk = ok ? g.dLdI[gp] * g.kc : 0.0;
     const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
     const float cn0[3] = {2.f / a.N[0], 2.f / a.N[1], 2.f / a.N[2]},
                 cn1[3] = {-4.f * a.N[0] * (1.f / 0.63f),
@@ -214,6 +217,12 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
     for (int i = 0; i < os; ++i)
       for (int j = 0; j < os; ++j)
         for (int t = 0; t < a.T; ++t) {
+          double ws = 0.0;
+          Kahan acc12;
+          float acc[12];
+#pragma unroll
+          for (int r = 0; r < 12; ++r) acc[r] = 0.f;
+          if (ok) {
           float vh[3], vl[3], df[3], omega;
           unit_geometry_ff(a, P, s, f, i, j, t, vh, vl, df, omega);
           float cap = 1.f;
@@ -229,7 +238,8 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
                 ye = df[0] * a.b0f[0] + df[1] * a.b0f[1] + df[2] * a.b0f[2];
           float scal = omega * cap * 0.5f *
                        (1.f + c2 * c2 - kahn * (xe * xe - ye * ye));
-          const float Wt = wp * scal;
+          ws = wk * (double)scal;
+          const float fscal = HASF ? (float)(ws * g.scale) : 0.f;
           for (int pm = 0; pm < a.PM; ++pm) {
             const float *Ah = s_axh + pm * 9, *Al = s_axl + pm * 9;
             float Gh[3], Gl[3], rq[3], rl[3], n0[3];
@@ -331,10 +341,10 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
               }
               if (!tri) fc = inside ? __ldg(a.F + nb_idx(a.check, NB_SITE_F, fidx, table_size(a))) : a.defF;
               const float w = src[SRC32_W];
-              const float tw = Wt * (fc * fc * fl2 * w);
+              const float tw = fc * fc * fl2 * w;
               // d term / d h_x = term dlog_x + 2 F dF/dh_x F_latt^2 w
               const float uk = a.u0h + dh, tu = tw * uk,
-                          fgu = Wt * (2.f * fc * fl2 * w) * uk;
+                          fgu = 2.f * fc * fl2 * w * uk;
 #pragma unroll
               for (int x = 0; x < 3; ++x) {
                 E[x] += fmaf(tu, -4.f * N2[x] * fr[x] * (1.f / 0.63f),
@@ -342,9 +352,9 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
                 acc[9 + x] = fmaf(tw, fmaf(cn1[x] * fr[x], fr[x], cn0[x]),
                                   acc[9 + x]);
               }
-              acc[12] += tw;
+              acc12.add(tw);
               if (HASF) {
-                const float gvf = Wt * g.kcs * (2.f * fc * fl2 * w);
+                const float gvf = fscal * (2.f * fc * fl2 * w);
                 if (tri) {
                   if (!holding || n[0] != held[0] || n[1] != held[1] ||
                       n[2] != held[2]) {
@@ -389,24 +399,40 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
               for (int c = 0; c < 3; ++c)
                 acc[3 * x + c] = fmaf(E[x], vr[c], acc[3 * x + c]);
           }
+          }
+          // the unit's sums, weighted, over the warp in FP64: of 16 a lane
+          // hands half to a lane 16 away, of the other 8 half to one 8 away,
+          // ...: 16 additions in place of 65, and nothing but one sum to keep
+          // from unit to unit
+          double v[16];
+#pragma unroll
+          for (int r = 0; r < 16; ++r)
+            v[r] = r < 12    ? ws * (double)acc[r]
+                   : r == 12 ? ws * acc12.value()
+                             : 0.0;
+#pragma unroll
+          for (int n = 8; n > 0; n >>= 1) {
+            const bool up = (lane & 2 * n) != 0;
+#pragma unroll
+            for (int r = 0; r < n; ++r) {
+              const double keep = up ? v[r + n] : v[r],
+                           give = up ? v[r] : v[r + n];
+              v[r] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * n);
+            }
+          }
+          mine += v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
         }
   }
   if (INTERP && HASF) flush_node();
   if (HASF && near_idx >= 0) atomicAdd(g.gradF + nb_idx(a.check, NB_SITE_GRADF, near_idx, table_size(a)), (double)near_sum);
-  // block reduction in a fixed order: a butterfly in FP32, the warps in FP64
-  __shared__ float red[kTileThreads / 32][kGradN];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int r = 0; r < kGradN; ++r) {
-    float v = acc[r];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[warp][r] = v;
-  }
+  // the block's sums in FP64, in a fixed order
+  __shared__ double red[kTileThreads / 32][kGradN];
+  if ((lane & 1) == 0 && lane / 2 < kGradN)
+    red[threadIdx.x >> 5][lane / 2] = mine;
   __syncthreads();
   if (threadIdx.x < kGradN) {
     double v = 0.0;
-    for (int w = 0; w < kTileThreads / 32; ++w) v += (double)red[w][threadIdx.x];
+    for (int w = 0; w < kTileThreads / 32; ++w) v += red[w][threadIdx.x];
     g.partials[(size_t)blockIdx.x * kGradN + threadIdx.x] = v;
   }
 }
@@ -550,6 +576,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
   const float cutg = kGaussCut * 0.63f;
   const float kahn = a.kahn;
+  const float scalef = (float)g.scale;
   float acc[kGradN];
 #pragma unroll
   for (int r = 0; r < kGradN; ++r) acc[r] = 0.f;
@@ -691,7 +718,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
       }
       acc[12] += tw;
       if (HASF) {
-        const float gvf = Wt * g.kcs * (2.f * fc * fl2 * w);
+        const float gvf = Wt * scalef * (2.f * fc * fl2 * w);
         if (tri) {
           // the column was flushed unless it holds this key
           held_key = (npk & 0xfffff) | ((fl[2] + 1) << 20);
@@ -780,7 +807,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
         f = 0;
       }
       P = a.panels + q;
-      W0 = ok ? (float)g.dLdI[gp] : 0.f;
+      W0 = ok ? (float)(g.dLdI[gp] * g.kc) : 0.f;
       new_pixel = false;
     }
     if (new_unit) {
@@ -1039,7 +1066,7 @@ size_t adjoint_scratch_bytes(const SpotArgs &a) {
          sizeof(double);
 }
 
-// writes the kGradN sums, without the prefactor kc, to sums_out
+// writes the kGradN sums, without the scale, to sums_out
 cudaError_t launch_adjoint(const SpotArgs &a, const float *rot,
                            const double *dLdI, double *gradF,
                            double *partials, double kc, double scale,
@@ -1050,7 +1077,8 @@ cudaError_t launch_adjoint(const SpotArgs &a, const float *rot,
   g.dLdI = dLdI;
   g.gradF = gradF;
   g.partials = partials;
-  g.kcs = (float)(kc * scale);
+  g.kc = kc;
+  g.scale = scale;
   g.rows_next = nullptr;
   g.n_rows = 0;
   size_t smem = adjoint_smem_bytes(a, a.interp && gradF);
@@ -1094,15 +1122,15 @@ cudaError_t launch_adjoint(const SpotArgs &a, const float *rot,
 }
 
 // grad (10) from the kGradN sums and the derivatives of the lab axes
-void adjoint_gradient(const double *sums, const double daxes[6][9], double kc,
+void adjoint_gradient(const double *sums, const double daxes[6][9],
                       double scale, double *grad) {
   for (int r = 0; r < 6; ++r) {
     double v = 0.0;
     for (int i = 0; i < 9; ++i) v += daxes[r][i] * sums[i];
-    grad[r] = kc * scale * v;
+    grad[r] = scale * v;
   }
-  for (int x = 0; x < 3; ++x) grad[6 + x] = kc * scale * sums[9 + x];
-  grad[9] = kc * sums[12];
+  for (int x = 0; x < 3; ++x) grad[6 + x] = scale * sums[9 + x];
+  grad[9] = sums[12];
 }
 
 int loss_blocks(long long n) {

@@ -1165,7 +1165,7 @@ int nb_adjoint(nb_sim *s, const double *dLdI, double grad[10],
                         cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "adjoint");
-  nbgb::adjoint_gradient(sums, s->daxes, kc, s->scale, grad);
+  nbgb::adjoint_gradient(sums, s->daxes, s->scale, grad);
   return read_check(s);
 }
 

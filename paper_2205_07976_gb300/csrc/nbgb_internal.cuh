@@ -384,7 +384,7 @@ cudaError_t launch_adjoint(const SpotArgs &a, const float *rot,
                            double *partials, double kc, double scale,
                            double *sums_out, int sm_count, cudaStream_t st);
 constexpr int kAdjointSums = 13;
-void adjoint_gradient(const double *sums, const double daxes[6][9], double kc,
+void adjoint_gradient(const double *sums, const double daxes[6][9],
                       double scale, double *grad);
 cudaError_t launch_poisson_loss(const double *img, const double *y,
                                 long long n, double bkg, double *dLdI,
