@@ -1335,8 +1335,10 @@ int nb_add_background(nb_sim *s) {
     void join(const Node &o) {  // o after this
       const double w = W + o.W, d = o.ubar - ubar;
       if (w > 0.0) {
-        V += o.V + d * d * (W * o.W / w);
-        ubar += d * (o.W / w);
+        // (the quotient first: W o.W may leave the range of FP64)
+        const double q = o.W / w;
+        V += o.V + d * d * (W * q);
+        ubar += d * q;
       } else {
         ubar = (ubar * n + o.ubar * o.n) / (n + o.n);
       }
