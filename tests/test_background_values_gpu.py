@@ -1,12 +1,36 @@
-"""The background with weights whose products leave the range of FP64, at
-the FP64 form's own 1e-12."""
+"""The background at scattering angles whose square is next to the least
+normal FP32 number, and with weights whose products leave the range of FP64:
+the two forms' own tolerances, 1e-12 and 1e-5."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_2205_07976_gb300 import workloads as W
 from tests.test_background_gpu import TOL, bg_image
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", ["f64", "mixed"])
+@pytest.mark.parametrize("e", [-46, -50, -54])
+def test_tiny_angles(precision, e):
+    """A pixel 2^e m off the beam at 1 m, and knots of that size."""
+    s = W.large_shot(n_src=1, n_mosaic=1)
+    s.oversample, s.n_layers, s.thickness_m = 1, 1, 0.0
+    s.lambdas = np.array([1.0])
+    px = 2.0 ** -30
+    s.panels = [W.Panel(origin=np.array([-0.5 * px + 2.0 ** e, -0.5 * px, 1.0]),
+                        fdir=np.array([1.0, 0.0, 0.0]),
+                        sdir=np.array([0.0, 1.0, 0.0]),
+                        ndir=np.array([0.0, 0.0, 1.0]), pixel_m=px, nfast=1,
+                        nslow=1)]
+    # stol = 2^(e - 1): a quarter of the way down from 1000 to 0
+    bg = W.Background(stol=np.array([0.0, 2.0 ** (e + 1)]),
+                      F=np.array([1000.0, 0.0]), n_molecules=1e10)
+    ref = oracle.background(s, bg)
+    got = bg_image(s, bg, precision)
+    assert ref[0] > 0
+    assert abs(got[0] - ref[0]) <= TOL[precision] * ref[0], (got, ref)
 
 
 @pytest.mark.parametrize("c", [1e-200, 1e-170, 1e160, 1e200])
