@@ -325,9 +325,10 @@ enum { NB_REQ_UNKNOWN = -1, NB_REQ_QUEUED = 0, NB_REQ_RUNNING = 1,
  *                fluence, polarization.
  * Every step is one replay of one of two CUDA graphs, used in turn: the
  * work-list upload from that graph's pinned buffer, a counter reset and
- * persistent kernels whose blocks pull work items of 128 pixels: the
- * thread-per-pixel kernel, and (for requests with tricubic lookup and >= 8
- * mosaic domains) the two forms of the warp-per-pixel kernel.
+ * persistent kernels whose blocks pull work items: the thread-per-pixel
+ * kernel (128 pixels), and (for requests with tricubic lookup and >= 8 mosaic
+ * domains) the two forms of the warp-per-pixel kernel (128 pixels, 64 for
+ * small requests).  A kernel without an item in the step is not launched.
  * Errors: NB_EINVAL (bad sizes), NB_ENOMEM, NB_ECUDA. */
 int nb_server_create(nb_server **out, int device, void *cuda_stream,
                      int max_slots, long long pool_bytes,

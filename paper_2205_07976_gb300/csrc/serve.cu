@@ -9,11 +9,13 @@
 //   submit  -> FIFO queue (inputs copied, tables built on the host)
 //   step    -> admit while a slot and room in the image pool exist (first
 //              fit; a blocked head request stops bypassing after 8 steps);
-//              cut the active requests into work items of 128 pixels up to a
-//              pixel-step budget: half shared equally by the running requests, the
+//              cut the active requests into work items (128 pixels,
+//              64 for small requests of the warp kernels) up to a pixel-step
+//              budget: half shared equally by the running requests, the
 //              rest to the oldest first; replay one of two CUDA graphs
 //              (work list upload from its own pinned buffer, counter reset,
-//              the persistent kernels); then wait for the step queued
+//              the persistent kernels; lists without an item are neither
+//              uploaded nor run); then wait for the step queued
 //              by the previous call, so the GPU runs one step while the host
 //              prepares the next; requests whose last item ran in a
 //              finished step are complete
@@ -30,6 +32,7 @@
 
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <type_traits>
 #include <deque>
@@ -46,9 +49,10 @@ namespace nbgb {
 constexpr int kServeMaxPM = 64;
 constexpr int kServeMaxSrc = 128;
 constexpr int kServeItemPixels = kTileThreads;  // one pixel per thread
-// the warp kernels: 32 pixels per warp (of 48 requests with up to 4e6 pixels:
-// 64 pixels 28.0 ms, 128 26.9, 256 27.2; as parallel branches of the graph
-// instead of one kernel after another, 28.9, 27.6 and 29.5)
+// the warp kernels: 32 pixels per warp, 16 for a request that could not give
+// every block an item of that many (item_pixels).  48 requests with up to 4e6
+// pixels: 27.5 ms with 32 for all, 29.0 with 16; single requests of up to 2500
+// pixels, nine of ten within 103 and 88 us.
 constexpr int kServeWarpItemPixels = 128;
 constexpr int kServeMaxItems = 16384;
 
@@ -235,6 +239,13 @@ struct Buf {
 
 constexpr int kKinds = 3;  // kinds of requests (Request::kind)
 
+// a kind's nodes in the graph of a step, and what they are set to
+struct StepNodes {
+  cudaGraphNode_t copy = nullptr, kernel = nullptr;
+  bool on = true;
+  size_t bytes = sizeof(WorkList);  // of its work list
+};
+
 struct Request {
   long long id;
   SlotParams params;  // host copy (img_off set at admission)
@@ -279,7 +290,9 @@ struct nb_server {
   int blocks_w[2] = {0, 0};  // of the warp kernels, pairs and lines
   size_t smem_w = 0;
   nbgb::SpotArgs base;
+  cudaGraph_t graph_of[2] = {nullptr, nullptr};
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  StepNodes nodes[2][kKinds];
   cudaEvent_t done_ev[2] = {nullptr, nullptr};
   bool in_flight[2] = {false, false};
   long long step_of[2] = {0, 0};
@@ -340,37 +353,79 @@ static cudaStream_t stream_of(const nb_server *s, int b) {
   return b == 0 ? s->stream : s->stream2;
 }
 
-// The graph of one step from host buffer b, on stream_of(b): its work
-// lists to its own device copies, its counters reset, the persistent
-// kernels.
+// The graph of one step from host buffer b: its work lists to its own device
+// copies, its counters reset, the persistent kernels.
 static int build_graph(nb_server *s, int b) {
-  cudaStream_t st = stream_of(s, b);
-  cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) return sfail(s, NB_ECUDA, "graph capture begin");
   WorkList *dw = (WorkList *)s->d_work.p + kKinds * b;
   unsigned *ctr = (unsigned *)s->d_counter.p + kKinds * b;
-  cudaMemcpyAsync(dw, s->h_work[b], kKinds * sizeof(WorkList),
-                  cudaMemcpyHostToDevice, st);
-  cudaMemsetAsync(ctr, 0, kKinds * sizeof(unsigned), st);
-  // the kernel with the longest items first: the last blocks of each leave
-  // SMs to the next one (in the order thread, pairs, lines the batch of 48
-  // requests above took 29.6 instead of 26.9 ms)
-  for (int k = s->interp == NB_INTERP_TRICUBIC ? kKinds - 1 : 0; k >= 0; --k) {
+  const SlotParams *slots = (const SlotParams *)s->d_slots.p;
+  double *pool = (double *)s->d_pool.p;
+  const int kinds = s->interp == NB_INTERP_TRICUBIC ? kKinds : 1;
+  cudaError_t e = cudaGraphCreate(&s->graph_of[b], 0);
+  cudaGraph_t g = s->graph_of[b];
+  cudaGraphNode_t last, copies[kKinds];
+  for (int k = 0; k < kinds && e == cudaSuccess; ++k) {
+    e = cudaGraphAddMemcpyNode1D(&copies[k], g, nullptr, 0, dw + k,
+                                 s->h_work[b] + k, sizeof(WorkList),
+                                 cudaMemcpyHostToDevice);
+    s->nodes[b][k].copy = copies[k];
+  }
+  cudaMemsetParams ms = {};
+  ms.dst = ctr;
+  ms.elementSize = sizeof(unsigned);
+  ms.width = kKinds;
+  ms.height = 1;
+  if (e == cudaSuccess) e = cudaGraphAddMemsetNode(&last, g, copies, kinds, &ms);
+  // the warp kernels, whose items are the longest, before the thread kernel:
+  // the last blocks of each leave SMs to the next one
+  for (int k = kinds - 1; k >= 0 && e == cudaSuccess; --k) {
     const nbgb::ServeKernel kern =
         k ? nbgb::serve_warp(s->base, k == 2)
           : s->interp ? nbgb::serve_kernel<1> : nbgb::serve_kernel<0>;
-    kern<<<k ? s->blocks_w[k - 1] : s->blocks,
-           k ? nbgb::kSplitThreads : nbgb::kTileThreads, k ? s->smem_w : 0,
-           st>>>(s->base, (const SlotParams *)s->d_slots.p, dw + k, ctr + k,
-                 (double *)s->d_pool.p);
+    const WorkList *list = dw + k;
+    unsigned *counter = ctr + k;
+    void *args[] = {&s->base, &slots, &list, &counter, &pool};
+    cudaKernelNodeParams kp = {};
+    kp.func = (void *)kern;
+    kp.gridDim = dim3(k ? s->blocks_w[k - 1] : s->blocks);
+    kp.blockDim = dim3(k ? nbgb::kSplitThreads : nbgb::kTileThreads);
+    kp.sharedMemBytes = k ? (unsigned)s->smem_w : 0u;
+    kp.kernelParams = args;
+    const cudaGraphNode_t prev = last;
+    e = cudaGraphAddKernelNode(&last, g, &prev, 1, &kp);
+    s->nodes[b][k].kernel = last;
   }
-  cudaGraph_t g = nullptr;
-  e = cudaStreamEndCapture(st, &g);
-  if (e != cudaSuccess) return sfail(s, NB_ECUDA, "graph capture end");
-  e = cudaGraphInstantiate(&s->graph[b], g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) return sfail(s, NB_ECUDA, "graph instantiate");
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&s->graph[b], g, 0);
+  if (e != cudaSuccess) return sfail(s, NB_ECUDA, "step graph");
   return NB_OK;
+}
+
+// Sets the graph of buffer b, which is not in flight, to its lists: a kind
+// without items has its nodes off, and of the others the items are uploaded and
+// not the whole list, in steps of 512 items, so that the size seldom changes
+// (request of a few hundred pixels: 68 -> 55 us).
+static cudaError_t set_graph(nb_server *s, int b) {
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < kKinds && e == cudaSuccess; ++k) {
+    StepNodes &nd = s->nodes[b][k];
+    const int n = s->h_work[b][k].n;
+    if (!nd.copy) continue;
+    if (nd.on != (n > 0)) {
+      e = cudaGraphNodeSetEnabled(s->graph[b], nd.copy, n > 0);
+      if (e == cudaSuccess)
+        e = cudaGraphNodeSetEnabled(s->graph[b], nd.kernel, n > 0);
+      if (e == cudaSuccess) nd.on = n > 0;
+    }
+    const size_t bytes = offsetof(WorkList, items) +
+                         (size_t)((n + 511) & ~511) * sizeof(WorkItem);
+    if (e == cudaSuccess && n > 0 && bytes != nd.bytes) {
+      e = cudaGraphExecMemcpyNodeSetParams1D(
+          s->graph[b], nd.copy, (WorkList *)s->d_work.p + kKinds * b + k,
+          s->h_work[b] + k, bytes, cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) nd.bytes = bytes;
+    }
+  }
+  return e;
 }
 
 extern "C" {
@@ -620,6 +675,7 @@ int nb_server_free(nb_server *s) {
   }
   for (int b = 0; b < 2; ++b) {
     if (s->graph[b]) cudaGraphExecDestroy(s->graph[b]);
+    if (s->graph_of[b]) cudaGraphDestroy(s->graph_of[b]);
     if (s->done_ev[b]) cudaEventDestroy(s->done_ev[b]);
     if (s->up_ev[b]) cudaEventDestroy(s->up_ev[b]);
     if (s->h_work[b]) cudaFreeHost(s->h_work[b]);
@@ -766,6 +822,13 @@ static int finish_oldest(nb_server *s, double timeout_s) {
   return NB_OK;
 }
 
+// pixels of a work item of r
+static long long item_pixels(const nb_server *s, const Request &r) {
+  if (!r.kind) return nbgb::kServeItemPixels;
+  const long long px = nbgb::kServeWarpItemPixels;
+  return r.npix < px * s->blocks_w[r.kind - 1] ? px / 2 : px;
+}
+
 static bool any_schedulable(const nb_server *s) {
   for (auto &kv : s->reqs)
     if (kv.second.state == NB_REQ_RUNNING && kv.second.next < kv.second.npix)
@@ -808,8 +871,7 @@ int nb_server_step(nb_server *s, double timeout_s, int *n_active) {
         Request &r = *act[j];
         WorkList *L = wl + r.kind;
         int &n = n_items[r.kind];
-        const long long cap = r.kind ? nbgb::kServeWarpItemPixels
-                                     : nbgb::kServeItemPixels;
+        const long long cap = item_pixels(s, r);
         long long mine = 0;  // pixel-steps given to r in this pass
         for (int k = 0; r.next < r.npix && used < s->budget &&
                         n < nbgb::kServeMaxItems &&
@@ -840,6 +902,7 @@ int nb_server_step(nb_server *s, double timeout_s, int *n_active) {
       // are on the other stream: wait for them (not for its kernels)
       cudaError_t e = cudaEventRecord(s->up_ev[b], st);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->up_ev[b ^ 1], 0);
+      if (e == cudaSuccess) e = set_graph(s, b);
       if (e == cudaSuccess) e = cudaGraphLaunch(s->graph[b], st);
       if (e == cudaSuccess) e = cudaEventRecord(s->done_ev[b], st);
       if (e != cudaSuccess) {
