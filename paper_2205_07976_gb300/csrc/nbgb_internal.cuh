@@ -38,7 +38,8 @@ enum {
   NB_SITE_IMAGE = 4,    // image pixel
   NB_SITE_SOURCE = 5,   // source row
   NB_SITE_GRADF = 6,    // structure-factor gradient entry
-  NB_SITE_KNOT = 7      // background knot
+  NB_SITE_KNOT = 7,     // background knot
+  NB_SITE_NODE = 8      // background node of a run of sources
 };
 
 __device__ __forceinline__ long long nb_idx(unsigned long long *word, int site,

@@ -901,6 +901,8 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
   }
   const int n = e - p;
   npairs += n;
+  const int pf = (int)nb_idx(a.check, NB_SITE_SOURCE, p, b.S),
+            pl = (int)nb_idx(a.check, NB_SITE_SOURCE, max(e - 1, 0), b.S);
   const SplitEntry &E4 = ring[(pq.e0 + j) & (kEntries - 1)];
   const float4 Ea = E4.a, Eb = E4.b, Ec = E4.c, Ed = E4.d;
   const float Gh[3] = {Ea.x, Ea.y, Ec.x}, dx[3] = {Ea.z, Ea.w, Ec.y};
@@ -912,9 +914,9 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
   // an approximate quotient).  A source's own signs would then name the
   // neighbouring cell, and the other sources be extrapolated from it.
   const float4 sf = *reinterpret_cast<const float4 *>(
-                   b.src + p * SRC32_STRIDE),
+                   b.src + pf * SRC32_STRIDE),
                sl = *reinterpret_cast<const float4 *>(
-                   b.src + max(e - 1, 0) * SRC32_STRIDE);
+                   b.src + pl * SRC32_STRIDE);
   const float dm = 0.5f * (sf.z + sl.z), dml = 0.5f * (sf.x + sl.x);
   const float half = 0.5f * (sl.z - sf.z);
   const float ih = half > 0.f ? __fdividef(1.f, half) : 0.f;
@@ -967,7 +969,7 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
     redo = ~0u;
   } else {
     const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
-    const float *src = b.src + p * SRC32_STRIDE + SRC32_PAIR;
+    const float *src = b.src + pf * SRC32_STRIDE + SRC32_PAIR;
     const f32x2 ih2 = splat2(ih), rl2 = splat2(-dml * ih),
                 rh2 = splat2(-dm), ts2 = splat2(-ts), cA2 = splat2(cA),
                 e02 = splat2(e0);
@@ -1030,7 +1032,7 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
     for (int i = 0; i < n; ++i) {
       if (!(redo >> (i >> 4) & 1u)) continue;
       const float4 sw = *reinterpret_cast<const float4 *>(
-          b.src + (p + i) * SRC32_STRIDE);
+          b.src + (pf + i) * SRC32_STRIDE);
       float fr[3], rad2 = 0.f;
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
