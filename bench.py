@@ -53,12 +53,13 @@ MAX_SM_MHZ = 2070.0  # GB300's maximum SM clock
 # kernel, from one ncu capture (profiles/spots_split_large_shot_dram.txt:
 # the mean of two launches);
 # valid only while the kernel sources hash to the value they had then
-TRAFFIC_CAPTURE = {"bytes": (80293376 + 27656192 + 80080640 + 28163328) // 2,
+TRAFFIC_CAPTURE = {"bytes": (79876864 + 21332992 + 80176640 + 21391616) // 2,
                    "sources": ["paper_2205_07976_gb300/csrc/spots_split.cu",
+                               "paper_2205_07976_gb300/csrc/split_kernel.cuh",
                                "paper_2205_07976_gb300/csrc/split_pixel.cuh",
                                "paper_2205_07976_gb300/csrc/mixed_common.cuh",
                                "paper_2205_07976_gb300/csrc/nbgb_internal.cuh"],
-                   "sha256_16": "a52943de1b33279a"}
+                   "sha256_16": "acd951c08ae206ab"}
 
 
 def captured_traffic():
@@ -75,14 +76,14 @@ def captured_traffic():
 # Pipe utilisation (% of active cycles) of the warp-per-pixel kernel from
 # one ncu --set full capture on a 512x512 window of the large shot
 # (profiles/spots_split_window512_full.txt), keyed like the traffic figure
-PIPES_CAPTURE = {"sm__pipe_fma_cycles_active_pct": 27.6,
-                 "sm__pipe_alu_cycles_active_pct": 34.2,
-                 "sm__inst_executed_pipe_lsu_pct": 16.3,
-                 "sm__pipe_fp64_cycles_active_pct": 36.3,
-                 "smsp__issue_active_pct": 55.7,
-                 "l1tex__data_pipe_lsu_wavefronts_pct": 43.3,
+PIPES_CAPTURE = {"sm__pipe_fma_cycles_active_pct": 28.7,
+                 "sm__pipe_alu_cycles_active_pct": 33.1,
+                 "sm__inst_executed_pipe_lsu_pct": 12.1,
+                 "sm__pipe_fp64_cycles_active_pct": 37.1,
+                 "smsp__issue_active_pct": 52.7,
+                 "l1tex__data_pipe_lsu_wavefronts_pct": 39.0,
                  "window": "512x512 centred on the large shot",
-                 "sha256_16": "a52943de1b33279a"}
+                 "sha256_16": "acd951c08ae206ab"}
 
 
 def captured_pipes():

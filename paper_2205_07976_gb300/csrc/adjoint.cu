@@ -142,9 +142,9 @@ __device__ __forceinline__ void lagrange4_deriv(float x, float w[4]) {
 // the nine products Q in place of 18 per orientation and each lane taking its
 // own surviving steps; -> 795 with the cut tested two sources at a time
 // (cut_sums).  A unit's sums are FP32 (dL/dscale compensated); over the units,
-// dL/dI and the pixels they are FP64 (refinement step 1.63 -> 1.66 ms).  All
-// of them FP32 over a pixel's 40 000 steps put dL/dN and dL/dscale off by 3e-6
-// to 1.3e-5 in place of 1e-8 to 8e-7.
+// dL/dI and the pixels they are FP64, which costs 35 us: all of them FP32 over a
+// pixel's 40 000 steps put dL/dN and dL/dscale off by 3e-6 to 1.3e-5 in place
+// of 1e-8 to 8e-7.
 template <int HASF, int INTERP>
 __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
     spots_adjoint_kernel(AdjointArgs g) {
@@ -947,7 +947,7 @@ static cudaError_t reduce_partials(const double *part, long long n,
 // Poisson loss L = sum_p (I_p + bkg - y_p log(I_p + bkg)) and dL/dI_p.
 // Bound by the FP64 pipe (1/64 of the FP32 rate), so the logarithm and the
 // quotient share what they can.  m = 2^e z, z in [1, 2); a table of 64
-// intervals gives c ~ 1/z, and r = z c - 1 (|r| < 2^-7, exact in one FMA) is
+// intervals gives c ~ 1/z, and r = z c - 1 (|r| < 2^-7, rounded once) is
 // both the argument of log1p, summed as its series to r^9 (remainder below
 // 2^-72; after Tang, "Table-driven implementation of the logarithm function",
 // 1990), and the first correction of the reciprocal.  About 30 FP64

@@ -1146,8 +1146,8 @@ int nb_adjoint(nb_sim *s, const double *dLdI, double grad[10],
   ensure_cell_polynomials(s);  // tricubic value and gradient per cell
   SpotArgs a;
   fill_args(s, a);
-  // (the limit leaves room for 45 floats per orientation that the kernels no
-  // longer stage: sizes that were refused stay refused)
+  // (the limit counts 72 floats per orientation, as it did when the
+  // kernels staged so many, not 27: sizes that were refused stay refused)
   if (nbgb::adjoint_smem_bytes(a, a.interp == NB_INTERP_TRICUBIC && gradF) +
           (size_t)180 * a.PM > 200 * 1024)
     return fail(s, NB_EINVAL, "tables exceed 200 KB of shared memory");
@@ -1250,7 +1250,8 @@ int nb_get_work(nb_sim *s, long long *counts, int n_counts) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "statistics read");
     if (s->precision == NB_F64) {
-      // every step is tested and evaluated
+      // every step is accounted for: evaluated, or (spots_f64_warp_kernel)
+      // shown to be below a rounding of the pixel's sum
       v[NB_WORK_PAIRS] = v[NB_WORK_TERMS] = s->last_pixel_steps;
     } else {
       v[NB_WORK_TERMS] = (long long)c[0];

@@ -724,8 +724,8 @@ __device__ __forceinline__ unsigned sum_pairs(
 // and, as long as no offset changes its sign, F_cell is one cell's tricubic
 // polynomial on a line: a polynomial of degree 9 in t.  A lane that takes such
 // a segment makes its ten coefficients once (cell_line: ~180 FMAs, packed where
-// two powers of x go side by side) and then spends ~25 instructions on a step,
-// one of them a shared load, where the pair queue spends ~250 per 32 steps on
+// two powers of x go side by side) and then spends ~15 instructions on a step,
+// two of them shared loads for a pair of steps, where the pair queue spends ~250 per 32 steps on
 // finding entry, source and cell and on 63 FMAs and 16 shared loads per step.
 
 // Coefficients q of F(x0 + g tau), a cell's polynomial (SpotArgs::C4 at cp) on

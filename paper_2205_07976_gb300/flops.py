@@ -66,8 +66,11 @@ ITEM_RANGE = 18
 
 
 def performed_flops(shot, work: dict) -> float:
-    """FP32 flops a launch performed, from the nb_get_work counts of that
-    launch (keys of nbgb.WORK_NAMES).  For the thread-per-pixel kernels
+    """FP32 flops of the work a launch went through, from the nb_get_work
+    counts of that launch (keys of nbgb.WORK_NAMES), at the costs above.  The
+    warp kernel's line form sums its pairs and terms along a line for fewer
+    flops than these, the costs of evaluating each by itself, so for it the
+    figure is an upper bound.  For the thread-per-pixel kernels
     (every step tested, no intervals) this equals algorithmic_flops."""
     per_term = TERM_ACCUM + (TERM_GAUSS if shot.shape == 1 else 0) + (
         TERM_TRICUBIC if shot.interp == 1 else 0)
