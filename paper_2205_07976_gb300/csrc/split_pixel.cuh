@@ -720,7 +720,7 @@ __device__ __forceinline__ unsigned sum_pairs(
 //
 // The steps of an interval entry lie on a line: with t = delta - delta_0 their
 // offset from the lattice point is f = f0 + G t.  So
-//   sum N^2 f^2 = Rmin + A (t - t*)^2,  A = sum N^2 G^2,
+//   sum N^2 f^2 = R* + 2 B* (t - t*) + A (t - t*)^2,  A = sum N^2 G^2,
 // and, as long as no offset changes its sign, F_cell is one cell's tricubic
 // polynomial on a line: a polynomial of degree 9 in t.  A lane that takes such
 // a segment makes its ten coefficients once (cell_line: ~180 FMAs, packed where
@@ -864,8 +864,9 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
                                               const SplitEntry *ring,
                                               PairQueue &pq, Kahan &acc,
                                               unsigned &npairs) {
-  constexpr float kLog2 = 2.f / 0.63f * 1.44269504f;  // exponent per R
-  const float ecut = -kGaussCut * 0.63f * kLog2;
+  // a term's base-2 exponent is -kExp R, R = sum N^2 f^2
+  constexpr double kExp = 2.0 / 0.63 * 1.4426950408889634;
+  constexpr float kExpH = (float)kExp, kExpL = (float)(kExp - (double)kExpH);
   const int lane = threadIdx.x & 31;
   const int np = min(32, pq.ct - pq.ch);
   // the entry of each task, as in sum_pairs
@@ -905,9 +906,6 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
             pl = (int)nb_idx(a.check, NB_SITE_SOURCE, max(e - 1, 0), b.S);
   const SplitEntry &E4 = ring[(pq.e0 + j) & (kEntries - 1)];
   const float4 Ea = E4.a, Eb = E4.b, Ec = E4.c, Ed = E4.d;
-  const float Gh[3] = {Ea.x, Ea.y, Ec.x}, dx[3] = {Ea.z, Ea.w, Ec.y};
-  const float Gl[3] = {Eb.x, Eb.y, Ec.z}, rl[3] = {Eb.z, Eb.w, Ec.w};
-  const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
   // The origin of the line is the mean of the first and the last source: its
   // offsets' signs name the segment's cell even where rounding put a source at
   // a sign change on the other side of the cut (line_segments compares with
@@ -920,28 +918,70 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
   const float dm = 0.5f * (sf.z + sl.z), dml = 0.5f * (sf.x + sl.x);
   const float half = 0.5f * (sl.z - sf.z);
   const float ih = half > 0.f ? __fdividef(1.f, half) : 0.f;
-  float f0[3], fl0[3], g[3];
-  float A = 0.f, Bq = 0.f;
-#pragma unroll
-  for (int x = 0; x < 3; ++x) {
-    const float sx = fmaf(Gh[x], dm, dx[x]);
-    const float c = fmaf(Gh[x], dml, fmaf(Gl[x], dm, rl[x]));
-    f0[x] = __fadd_rn(sx, c);
-    fl0[x] = __fsub_rn(c, __fsub_rn(f0[x], sx));
-    g[x] = Gh[x] * half;
-    A = fmaf(N2[x] * g[x], g[x], A);
-    Bq = fmaf(N2[x] * g[x], f0[x], Bq);
-  }
-  // tau = (delta - delta_0) / half; R = Rmin + A (tau - ts)^2
-  const float ts = A > 0.f ? -__fdividef(Bq, A) : 0.f;
-  float R = 0.f;
+  // axes h and k side by side in packed operations, l in scalar ones; x - y as
+  // ffma2(y, -1, x), one rounding
+  const f32x2 m1 = splat2(-1.f);
+  const f32x2 Gp = pk2(make_float2(Ea.x, Ea.y)),
+              Glp = pk2(make_float2(Eb.x, Eb.y)), half2 = splat2(half),
+              N2p = pk2(make_float2(a.N[0] * a.N[0], a.N[1] * a.N[1]));
+  const float N2l = a.N[2] * a.N[2];
+  const f32x2 sp = ffma2(Gp, splat2(dm), pk2(make_float2(Ea.z, Ea.w))),
+              cp = ffma2(Gp, splat2(dml),
+                         ffma2(Glp, splat2(dm), pk2(make_float2(Eb.z, Eb.w)))),
+              f0p = fadd2(sp, cp), flp = ffma2(ffma2(sp, m1, f0p), m1, cp),
+              gp = fmul2(Gp, half2), ngp = fmul2(N2p, gp);
+  const float sl_ = fmaf(Ec.x, dm, Ec.y),
+              cl = fmaf(Ec.x, dml, fmaf(Ec.z, dm, Ec.w)),
+              f0l = __fadd_rn(sl_, cl), fll = __fsub_rn(cl, __fsub_rn(f0l, sl_)),
+              gl = Ec.x * half, ngl = N2l * gl;
+  const float2 A2 = upk2(fmul2(ngp, gp)), B2 = upk2(fmul2(ngp, f0p)),
+               f0h = upk2(f0p), g2 = upk2(gp);
+  const float A = fmaf(ngl, gl, A2.x + A2.y),
+              B = fmaf(ngl, f0l, B2.x + B2.y);
+  const float f0[3] = {f0h.x, f0h.y, f0l}, g[3] = {g2.x, g2.y, gl};
+  // The exponents about the task's point nearest to the lattice point, tau* in
+  // [-1, 1]: with u = tau - tau*
+  //   -kExp R = -ei + ef - kExp (2 B* u + A u^2),
+  // R and its slope B* formed at tau* from double-float offsets, ei whole.
+  // The largest terms, at u near 0, then carry the rounding of a small number
+  // even where all of a pixel's terms lie far from their lattice points (R 15
+  // to 26, against 64 bits, rms of a task's sum: 5.3e-6 about the vertex of the
+  // whole line in FP32, 2.5e-6; pair by pair 3.5e-6).
+  const float ts =
+      A > 0.f ? fminf(fmaxf(-__fdividef(B, A), -1.f), 1.f) : 0.f;
   const float th = ts * half;
-#pragma unroll
-  for (int x = 0; x < 3; ++x) {
-    const float fs = fmaf(Gh[x], th, f0[x]) + fmaf(Gl[x], th, fl0[x]);
-    R = fmaf(N2[x] * fs, fs, R);
+  float R, Rl, Bs;
+  {
+    const f32x2 th2 = splat2(th);
+    // G th, its rounding (negative), and its sum with f0
+    const f32x2 p1 = fmul2(Gp, th2), e1 = ffma2(Gp, ffma2(th2, m1, 0ull), p1),
+                s1 = fadd2(f0p, p1), bb = ffma2(f0p, m1, s1),
+                e2 = fadd2(ffma2(ffma2(bb, m1, s1), m1, f0p),
+                           ffma2(bb, m1, p1)),
+                lo = fadd2(ffma2(e1, m1, e2), ffma2(Glp, th2, flp)),
+                fs = fadd2(s1, lo), fl = ffma2(ffma2(s1, m1, fs), m1, lo),
+                t = fmul2(N2p, fs), te = ffma2(fmul2(N2p, m1), fs, t),
+                p2 = fmul2(t, fs), e3 = ffma2(fmul2(t, m1), fs, p2);
+    // the rests: 2 t fl - te fs - e3 (te and e3 are negative)
+    const float2 q = upk2(p2),
+                 rest = upk2(ffma2(fadd2(t, t), fl,
+                                   ffma2(ffma2(te, fs, e3), m1, 0ull))),
+                 b2 = upk2(fmul2(ngp, fs));
+    float p1l, e1l, s1l, e2l, fsl, fl_, tl, tel, p2l, e3l, s2, e4, e5;
+    two_prod(Ec.x, th, p1l, e1l);
+    two_sum(f0l, p1l, s1l, e2l);
+    fast_two_sum(s1l, (e1l + e2l) + fmaf(Ec.z, th, fll), fsl, fl_);
+    two_prod(N2l, fsl, tl, tel);
+    two_prod(tl, fsl, p2l, e3l);
+    two_sum(q.x, q.y, s2, e4);
+    two_sum(s2, p2l, R, e5);
+    Rl = (rest.x + rest.y) + (e3l + (e4 + e5)) + fmaf(tel, fsl, 2.f * tl * fl_);
+    Bs = fmaf(ngl, fsl, b2.x + b2.y);
   }
-  const float e0 = -kLog2 * R, cA = -kLog2 * A;
+  const float ei = rintf(kExpH * R);
+  const float ef = fmaf(-kExpH, R, ei) - fmaf(kExpL, R, kExpH * Rl);
+  const float eB = -2.f * kExpH * Bs, eA = -kExpH * A;
+  const float ecut = ei - kGaussCut * 0.63f * kExpH;
   float q[10], Fn = 0.f;
   bool line = true;  // the segment's cell lies in the table
   if (INTERP == 1) {
@@ -971,15 +1011,18 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
     const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
     const float *src = b.src + pf * SRC32_STRIDE + SRC32_PAIR;
     const f32x2 ih2 = splat2(ih), rl2 = splat2(-dml * ih),
-                rh2 = splat2(-dm), ts2 = splat2(-ts), cA2 = splat2(cA),
-                e02 = splat2(e0);
+                rh2 = splat2(-dm), ts2 = splat2(-ts), eA2 = splat2(eA),
+                eB2 = splat2(eB), ef2 = splat2(ef);
     f32x2 q2[10];
     if (INTERP == 1) {
 #pragma unroll
       for (int d = 0; d < 10; ++d) q2[d] = splat2(q[d]);
     }
-    // (nearest lookup: the entry's one structure factor)
-    const float fac = INTERP == 1 ? a.N6 * Ed.w : Fn * Fn * (a.N6 * Ed.w);
+    // (nearest lookup: the entry's one structure factor), and 2^-ei in two
+    // factors, as ei reaches 130
+    const float fac = (INTERP == 1 ? a.N6 * Ed.w : Fn * Fn * (a.N6 * Ed.w)) *
+                      5.4210109e-20f;
+    const float scale = __int_as_float((127 + 64 - (int)ei) << 23);
     for (int i0 = 0; i0 < nmax; i0 += 16) {
       f32x2 sum2 = splat2(0.f);  // at most 8 terms per lane half
       const int iend = min(i0 + 16, nmax);
@@ -991,8 +1034,8 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
               *reinterpret_cast<const f32x2 *>(src + i * SRC32_STRIDE + 4);
           const f32x2 tau =
               ffma2(fadd2(sd.x, rh2), ih2, ffma2(sd.y, ih2, rl2));
-          const f32x2 tt = fadd2(tau, ts2);
-          const float2 xe = upk2(ffma2(fmul2(cA2, tt), tt, e02));
+          const f32x2 u = fadd2(tau, ts2);
+          const float2 xe = upk2(ffma2(ffma2(eA2, u, eB2), u, ef2));
           float2 Ex;
           asm("ex2.approx.f32 %0, %1;" : "=f"(Ex.x) : "f"(xe.x));
           asm("ex2.approx.f32 %0, %1;" : "=f"(Ex.y) : "f"(xe.y));
@@ -1013,7 +1056,7 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
         }
       }
       const float2 sum = upk2(sum2);
-      const float v = (sum.x + sum.y) * fac;
+      const float v = (sum.x + sum.y) * scale * fac;
       if (fabsf(v) <= 3.4e38f)
         acc.add(v);
       else
@@ -1027,6 +1070,7 @@ __device__ __forceinline__ unsigned sum_tasks(const SpotArgs &a,
     const float4 Ea = E4.a, Eb = E4.b, Ec = E4.c, Ed = E4.d;
     const float Gh[3] = {Ea.x, Ea.y, Ec.x}, dx[3] = {Ea.z, Ea.w, Ec.y};
     const float Gl[3] = {Eb.x, Eb.y, Ec.z}, rl[3] = {Eb.z, Eb.w, Ec.w};
+    const float N2[3] = {a.N[0] * a.N[0], a.N[1] * a.N[1], a.N[2] * a.N[2]};
     int nt[3];
     entry_index<INTERP>(Ed, nt);
     for (int i = 0; i < n; ++i) {

@@ -115,3 +115,34 @@ def test_table_entries_that_are_not_finite(interp, bad):
         ok = np.isfinite(nbgb.simulate(s, "mixed", variant=variant))
         assert not ok[sure].any(), variant
         assert ok[~maybe].all(), (variant, int((~ok[~maybe]).sum()))
+
+
+def test_pixels_far_from_every_lattice_point():
+    """Windows whose terms all lie far out in a reflection's tail (their
+    brightest pixel 1e-12 to 1e-30 of a peak), where a term's error is its
+    exponent's: against the FP64 form, window by window, in the geometric mean
+    no more than half above the thread kernel's error, which forms every
+    exponent from its own offset."""
+    err = {"warp": [], "thread": []}
+    for S, M, N, interp, f0, s0 in (
+            (100, 30, 18.0, 1, 580, 371), (64, 50, 18.0, 1, 940, 2100),
+            (64, 50, 25.0, 0, 1855, 2236), (40, 50, 18.0, 1, 942, 2860),
+            (100, 30, 25.0, 0, 1859, 1472), (40, 50, 18.0, 0, 1027, 1129),
+            (64, 50, 18.0, 1, 2250, 2447), (40, 50, 18.0, 0, 2945, 1956),
+            (100, 30, 18.0, 1, 483, 834), (40, 30, 25.0, 1, 2667, 1731),
+            (64, 50, 25.0, 1, 2200, 2952), (64, 50, 60.0, 0, 847, 2959)):
+        s = W.large_shot(n_src=S, n_mosaic=M)
+        s.oversample, s.n_layers, s.thickness_m = 1, 1, 0.0
+        s.interp, s.ncells = interp, np.array([N, N, N])
+        s = W.shrink(s, 16, 16, f0, s0)
+        ref = nbgb.simulate(s, "f64")
+        if not 1e-30 < ref.max() / (8e-8 * N ** 6) < 1e-12:
+            continue
+        m = ref > 1e-2 * ref.max()
+        for v in err:
+            got = nbgb.simulate(s, "mixed", variant=v)
+            e = (got - ref)[m] / ref[m]
+            err[v].append(np.mean(e ** 2))
+    assert len(err["warp"]) >= 6
+    rms = {v: np.exp(0.5 * np.mean(np.log(e))) for v, e in err.items()}
+    assert rms["warp"] <= 1.5 * rms["thread"], rms
