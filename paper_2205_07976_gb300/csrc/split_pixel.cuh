@@ -308,6 +308,18 @@ __host__ __device__ inline size_t split_smem_layout(int PM, int S) {
   return off;
 }
 
+// Whether the ellipsoids of neighbouring lattice points at the (widened) cut
+// are disjoint, so that a source has one of them at most
+__host__ __device__ inline float cut_wide() {
+  return kGaussCut * 0.63f * 1.02f + 1e-4f;
+}
+constexpr float kDisjoint = 0.49f;
+__host__ __device__ inline bool lattice_disjoint(const SpotArgs &a) {
+  const float m = sqrtf(cut_wide());
+  return m / a.N[0] < kDisjoint && m / a.N[1] < kDisjoint &&
+         m / a.N[2] < kDisjoint;
+}
+
 // Stages a shot's tables (double-float axes [PM][9], interleaved into
 // (hi, lo) pairs, and source rows [S][12]) into the dynamic shared memory
 // `sms` and derives the pruning constants.  Called by every thread of the
@@ -388,13 +400,12 @@ __device__ __forceinline__ void split_stage(SplitBlock &b, float *sms,
   b.u0l = u0l;
   // a widened cut for the conservative tests: every surviving term has
   // sum N^2 f^2 <= cutg < cwide, so |f_x| <= sqrt(cwide) / N_x
-  const float cutg = kGaussCut * 0.63f;
-  b.cwide = cutg * 1.02f + 1e-4f;
+  b.cwide = cut_wide();
   for (int x = 0; x < 3; ++x) b.cmarg[x] = sqrtf(b.cwide) / a.N[x];
   // exact delta-intervals per lattice point need the ellipsoids of
   // neighbouring lattice points to be disjoint: sqrt(cwide)/N < 1/2
-  b.iv_ok = dh_sorted && b.cmarg[0] < 0.49f && b.cmarg[1] < 0.49f &&
-            b.cmarg[2] < 0.49f;
+  b.iv_ok = dh_sorted && b.cmarg[0] < kDisjoint && b.cmarg[1] < kDisjoint &&
+            b.cmarg[2] < kDisjoint;
   b.dmin = S > 0 ? s_dh[0] : 0.f;
   b.dmax = S > 0 ? s_dh[S - 1] : 0.f;
   b.dmarg = 1e-3f * (b.dmax - b.dmin) / (float)(S > 1 ? S - 1 : 1);
@@ -1339,8 +1350,12 @@ __host__ __device__ inline float lattice_share(const SpotArgs &a) {
 // coefficients (pairs with the early test -> lines, 700^2 pixels: 1 unit, S =
 // 100, M = 12 0.605 -> 0.541 ms; S = 60, M = 30 0.750 -> 0.621; S = 30, M = 50
 // 0.820 -> 0.816; S = 20, M = 50 0.696 -> 0.777; S = 60, M = 12, 1000^2 0.787 ->
-// 0.873; large shot, 1024^2: 18.2 -> 10.2).  The early test pays where lattice
-// points are rare: N = 25 (0.07 of h space lies within the cut) 1.22 -> 1.05
+// 0.873; large shot, 1024^2: 18.2 -> 10.2).  Where the ellipsoids of lattice points
+// overlap (N < 15.4) there are no interval entries, and the blocks of sources
+// are better summed by the pair kernels and their 20 warps per SM (300^2
+// pixels, N = 8, 10 items of 180 sources: 2.07 -> 1.68 ms).  The early test pays
+// where lattice points are rare: N = 25 (0.07 of h space lies within the cut)
+// 1.22 -> 1.05
 // ms on 1500^2 pixels with S = 11, M = 9, but at N = 15 (0.34) it finds one in
 // most batches, 1.86 -> 2.11 ms on the 64-panel shot.
 // Halves pay where a pixel's items leave half the lanes idle (64-panel shot, 10
@@ -1352,10 +1367,10 @@ __host__ __device__ inline float lattice_share(const SpotArgs &a) {
 // limits on steps and on expected pairs.
 __host__ __device__ inline int split_form(const SpotArgs &a, int PM, int S) {
   if (a.has_div) return kPairs;
-  if ((a.interp == 0 || a.C4) && S >= kLineSources &&
-      (long long)a.os * a.os * a.T * PM * S >= kLineSteps)
-    return kLines;
   const long long items = (long long)a.os * a.os * a.T * PM;
+  if ((a.interp == 0 || a.C4) && S >= kLineSources &&
+      items * S >= kLineSteps && lattice_disjoint(a))
+    return kLines;
   if (items <= kHalfItems && items * S <= kHalfSteps &&
       (float)(items * S) * lattice_share(a) <= kHalfPairs)
     return kHalves;
