@@ -1348,6 +1348,8 @@ int nb_add_background(nb_sim *s) {
     }
   };
   std::vector<double> nodes;
+  int cnt_max = 0;               // of the groups with nodes: the most sources,
+  double span_per_source = 0.0;  // the largest relative range of u per source
   for (int g = 0; g < G; ++g) {
     const int first = rng[4 * g], cnt = rng[4 * g + 1];
     bool ok = true;
@@ -1363,6 +1365,10 @@ int nb_add_background(nb_sim *s) {
     grp[12 * g + 3] = span > 0.0 ? (cnt - 1) / span : 0.0;
     if (!ok) continue;
     rng[4 * g + 2] = (int)nodes.size() / 4;
+    cnt_max = std::max(cnt_max, cnt);
+    span_per_source = std::max(
+        span_per_source,
+        2.0 * span / ((leaf[0].ubar + leaf[cnt - 1].ubar) * cnt));
     std::vector<Node> t(4 * (size_t)cnt);
     t[cnt - 1] = leaf[cnt - 1];
     for (int i = cnt - 2; i >= 0; --i) {  // suffixes
@@ -1399,12 +1405,15 @@ int nb_add_background(nb_sim *s) {
                 "background tables exceed 200 KB of shared memory");
   // with many sources and knots the nodes may not fit as well: every source
   // is then visited
+  // (nor are they of use where every group is one source)
   b.n_nodes = (int)nodes.size() / 4;
-  if (nbgb::background_smem_bytes(b, f64) > 200 * 1024) {
+  if (cnt_max < 2 || nbgb::background_smem_bytes(b, f64) > 200 * 1024) {
     b.n_nodes = 0;
+    cnt_max = 0;
     nodes.clear();
     for (int g = 0; g < G; ++g) rng[4 * g + 2] = -1;
   }
+  b.form = nbgb::bg_form(f64, cnt_max, span_per_source, n);
   // one double blob: groups, then (F64) knots and sources; one float blob
   std::vector<double> b64(grp);
   std::vector<float> b32;

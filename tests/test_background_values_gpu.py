@@ -1,12 +1,13 @@
 """The background at scattering angles whose square is next to the least
-normal FP32 number, and with weights whose products leave the range of FP64:
-the two forms' own tolerances, 1e-12 and 1e-5."""
+normal FP32 number, with weights whose products leave the range of FP64, and
+in every form of the kernels (nodes, nodes or single sources where knots are
+dense, single sources): the two forms' own tolerances, 1e-12 and 1e-5."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_2205_07976_gb300 import workloads as W
-from tests.test_background_gpu import TOL, bg_image
+from tests.test_background_gpu import TOL, bg_image, check
 
 pytestmark = pytest.mark.gpu
 
@@ -44,3 +45,30 @@ def test_fp64_weights_over_the_range(c):
     s.weights = w * c
     got = bg_image(s, bg, "f64") / c
     assert np.all(np.abs(got - ref) <= TOL["f64"] * ref)
+
+
+def _beam(s, S, width, tilt=0.0):
+    s.dirs, s.lambdas, s.weights = W.gaussian_spectrum(
+        S, 9.5, width, (tilt, 0.0, 1.0))
+
+
+@pytest.mark.parametrize("precision", ["f64", "mixed"])
+@pytest.mark.parametrize("S,knots,dirs,neg", [
+    (9, 4096, 1, False), (8, 4096, 1, False), (33, 4096, 1, False),
+    (100, 4096, 1, False), (64, 40, 64, False), (65, 40, 1, True),
+    (31, 700, 3, True), (2, 4096, 1, False)])
+def test_dense_knots_single_sources_and_negative_weights(precision, S, knots,
+                                                         dirs, neg):
+    s = W.shrink(W.large_shot(n_src=1, n_mosaic=1), 35, 19, 1400, 900)
+    _beam(s, S, 0.005)
+    rng = np.random.default_rng(2)
+    d = np.concatenate([1e-3 * rng.standard_normal((dirs, 2)),
+                        np.ones((dirs, 1))], 1)
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    if dirs > 1:
+        s.dirs = d[np.arange(S) % dirs]
+    if neg:
+        s.weights = s.weights.copy()
+        s.weights[S // 3] *= -0.5
+    bg = W.amorphous_background(knots, stol_max=0.5)
+    check(bg_image(s, bg, precision), oracle.background(s, bg), precision)
