@@ -129,6 +129,10 @@ struct nb_sim {
   // amorphous background: knots, scattering factors, molecules in the beam
   bool have_bg = false;
   std::vector<double> bg_stol, bg_F;
+  // the background's tables (background_tables): whether they are out of date,
+  // and what a launch needs of them
+  bool bg_dirty = true;
+  int bg_groups = 0, bg_nodes = 0, bg_form = 0;
   double bg_nmol = 0;
   DevBuf d_bg64, d_bg32, d_bgrng;
 };
@@ -806,6 +810,7 @@ int nb_set_beam(nb_sim *s, const double *dirs, const double *lambda_A,
   std::memcpy(s->evec, e, sizeof e);
   s->have_beam = true;
   s->tables_dirty = true;
+  s->bg_dirty = true;
   return NB_OK;
 }
 
@@ -1288,19 +1293,19 @@ int nb_set_background(nb_sim *s, const double *stol, const double *F,
     return fail(s, NB_EINVAL, "n_molecules");
   s->bg_stol.assign(stol, stol + n_knots);
   s->bg_F.assign(F, F + n_knots);
+  s->bg_dirty = true;
   s->bg_nmol = n_molecules;
   s->have_bg = true;
   return NB_OK;
 }
 
-int nb_add_background(nb_sim *s) {
-  nbgb::NvtxRange nvtx_("nb_add_background");
-  if (!s) return NB_EINVAL;
-  if (!s->have_beam || !s->have_det || !s->have_bg)
-    return fail(s, NB_ESTATE,
-                "beam, detector and background table must be set first");
-  DeviceGuard g(s->device);
+// The tables of the background kernels: the sources grouped by direction, the
+// knots, and the nodes of the groups.  They depend on the beam and the
+// scattering curve, and are made again when one of these was set (400 sources of
+// one direction: 33 us of host work).
+static int background_tables(nb_sim *s) {
   const int S = s->n_src, n = (int)s->bg_stol.size();
+  const bool f64 = s->precision == NB_F64;
   // group the sources (already in ascending 1/lambda) by direction; the
   // order inside a group stays ascending
   std::vector<int> order, rng;
@@ -1327,7 +1332,6 @@ int nb_add_background(nb_sim *s) {
     rng.push_back(0);
   }
   const int G = (int)rng.size() / 4;
-  const bool f64 = s->precision == NB_F64;
   // the nodes of each group without negative weights, in the layout of
   // bg_group_sum; two runs are joined by their means and variance sums
   struct Node {
@@ -1455,6 +1459,34 @@ int nb_add_background(nb_sim *s) {
                     cudaMemcpyHostToDevice, s->stream);
   cudaMemcpyAsync(s->d_bgrng.p, rng.data(), rng.size() * sizeof(int),
                   cudaMemcpyHostToDevice, s->stream);
+  if ((e = cudaGetLastError()) != cudaSuccess)
+    return cuda_fail(s, e, "background tables");
+  s->bg_groups = G;
+  s->bg_nodes = b.n_nodes;
+  s->bg_form = b.form;
+  s->bg_dirty = false;
+  return NB_OK;
+}
+
+int nb_add_background(nb_sim *s) {
+  nbgb::NvtxRange nvtx_("nb_add_background");
+  if (!s) return NB_EINVAL;
+  if (!s->have_beam || !s->have_det || !s->have_bg)
+    return fail(s, NB_ESTATE,
+                "beam, detector and background table must be set first");
+  DeviceGuard g(s->device);
+  if (s->bg_dirty) {
+    const int rc = background_tables(s);
+    if (rc != NB_OK) return rc;
+  }
+  const int S = s->n_src, n = (int)s->bg_stol.size(), G = s->bg_groups;
+  const bool f64 = s->precision == NB_F64;
+  nbgb::BgArgs b;
+  std::memset(&b, 0, sizeof b);
+  b.n_knots = n;
+  b.n_groups = G;
+  b.n_nodes = s->bg_nodes;
+  b.form = s->bg_form;
   SpotArgs &a = b.geo;
   a.check = (unsigned long long *)s->d_check.p;  // NB_CHECK builds only
   a.panels = (const DevPanel *)s->d_panels.p;
@@ -1480,9 +1512,8 @@ int nb_add_background(nb_sim *s) {
   b.grp_range = (const int *)s->d_bgrng.p;
   b.prefactor = nbgb::kElectronRadius * nbgb::kElectronRadius * s->fluence *
                 s->bg_nmol / ((double)s->os * s->os);
-  e = nbgb::launch_background(b, f64, s->sm_count, s->stream);
+  const cudaError_t e = nbgb::launch_background(b, f64, s->sm_count, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "background launch");
-  // the pageable copies above are staged before the launch returns
   return read_check(s);
 }
 

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_2205_07976_gb300 import nbgb
 from paper_2205_07976_gb300 import workloads as W
 from tests.test_background_gpu import TOL, bg_image, check
 
@@ -50,6 +51,47 @@ def test_fp64_weights_over_the_range(c):
 def _beam(s, S, width, tilt=0.0):
     s.dirs, s.lambdas, s.weights = W.gaussian_spectrum(
         S, 9.5, width, (tilt, 0.0, 1.0))
+
+
+@pytest.mark.parametrize("precision", ["f64", "mixed"])
+def test_tables_follow_the_beam_and_the_curve(precision):
+    """One handle through beams and curves of every form of the kernel gives
+    bitwise what a fresh handle gives, and the same call twice the same."""
+    s = W.shrink(W.large_shot(n_src=1, n_mosaic=1), 35, 19, 1400, 900)
+    sim = None
+    for S, width, tilt, knots, neg in ((100, 0.005, 0.0, 64, False),
+                                       (9, 0.005, 0.0, 4096, False),
+                                       (9, 0.005, 0.002, 4096, False),
+                                       (50, 0.02, 0.0, 40, True),
+                                       (1, 0.005, 0.0, 40, False),
+                                       (100, 0.005, 0.0, 512, False)):
+        _beam(s, S, width, tilt)
+        if neg:
+            s.weights = s.weights.copy()
+            s.weights[3] *= -1.0
+        bg = W.amorphous_background(knots, stol_max=0.5)
+        ref = bg_image(s, bg, precision)
+        if sim is None:
+            sim = nbgb.Sim(precision).set_shot(s)
+        sim.set_beam(s)
+        sim.set_background(bg)
+        for _ in range(2):
+            sim.zero()
+            sim.add_background()
+            np.testing.assert_array_equal(sim.image(), ref)
+    # the curve alone, then the beam alone
+    sim.set_background(W.amorphous_background(33))
+    sim.zero()
+    sim.add_background()
+    np.testing.assert_array_equal(
+        sim.image(), bg_image(s, W.amorphous_background(33), precision))
+    _beam(s, 7, 0.01)
+    sim.set_beam(s)
+    sim.zero()
+    sim.add_background()
+    np.testing.assert_array_equal(
+        sim.image(), bg_image(s, W.amorphous_background(33), precision))
+    sim.close()
 
 
 @pytest.mark.parametrize("precision", ["f64", "mixed"])
