@@ -65,6 +65,16 @@ constexpr double kRoundBias = 6755399441055744.0;
 
 // The lattice point n nearest to h (ties down: ceil(h - 1/2)) and the offset
 // f = h - n (exact)
+__device__ __forceinline__ void nearest_ceil(const double h[3], long long n[3],
+                                             double f[3]) {
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    const double c = ceil(h[x] - 0.5);
+    n[x] = (long long)c;
+    f[x] = h[x] - c;
+  }
+}
+// the same by an addition where |h| allows it
 __device__ __forceinline__ void nearest_f64(const double h[3], long long n[3],
                                             double f[3]) {
   // |h| < 2^30 on all axes (integer compares of the high words; a double
@@ -80,12 +90,7 @@ __device__ __forceinline__ void nearest_f64(const double h[3], long long n[3],
       f[x] = h[x] - (s - kRoundBias);
     }
   } else {
-#pragma unroll
-    for (int x = 0; x < 3; ++x) {
-      const double c = ceil(h[x] - 0.5);
-      n[x] = (long long)c;
-      f[x] = h[x] - c;
-    }
+    nearest_ceil(h, n, f);
   }
 }
 
@@ -305,9 +310,15 @@ __global__ void __launch_bounds__(kTileThreads, 4)
         double h[3] = {dot3d(A, Sv), dot3d(A + 3, Sv), dot3d(A + 6, Sv)};
         long long n[3];
         double f[3];
-        nearest_f64(h, n, f);
-        const double a_ =
-            fcell_f64<INTERP>(a, f, n) * flatt_f64<SHAPE>(a, f);
+        // (Gaussian steps: a ceil measured faster than the biased addition, and
+        // F_latt before the lookup, whose results are else held across it:
+        // 64^2 pixels of 99 steps 695 -> 654 us; the sinc sweep 30.8 -> 30.3 ms)
+        if (SHAPE == 1)
+          nearest_ceil(h, n, f);
+        else
+          nearest_f64(h, n, f);
+        const double fl = flatt_f64<SHAPE>(a, f);
+        const double a_ = fcell_f64<INTERP>(a, f, n) * fl;
         acc = fma(a_ * a_, wcpo, acc);
       }
     }
