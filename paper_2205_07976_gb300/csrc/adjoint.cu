@@ -134,6 +134,23 @@ __device__ __forceinline__ void lagrange4_deriv(float x, float w[4]) {
   w[3] = (3.f * x2 - 1.f) * (1.f / 6.f);
 }
 
+// The sums v[0 .. kGradN) over the warp in FP64, sum r in lanes 2 r and 2 r + 1:
+// of 16 a lane hands half to a lane 16 away, of the other 8 half to one 8 away,
+// ...: 16 additions in place of 65
+__device__ __forceinline__ double warp_sums(double v[16]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = 8; n > 0; n >>= 1) {
+    const bool up = (lane & 2 * n) != 0;
+#pragma unroll
+    for (int r = 0; r < n; ++r) {
+      const double keep = up ? v[r + n] : v[r], give = up ? v[r] : v[r + n];
+      v[r] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * n);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
 // One thread per pixel (nearest lookup, and tricubic lookup in tables too
 // long for the ring kernel below).  Bound by instruction issue: per (pixel,
 // orientation) about 150 for the double-float G and r, 12 per source for the
@@ -141,10 +158,11 @@ __device__ __forceinline__ void lagrange4_deriv(float x, float w[4]) {
 // surviving.  64-panel shot (S = 8, 10 domains, nearest): 1316 -> 880 us with
 // the nine products Q in place of 18 per orientation and each lane taking its
 // own surviving steps; -> 795 with the cut tested two sources at a time
-// (cut_sums).  A unit's sums are FP32 (dL/dscale compensated); over the units,
-// dL/dI and the pixels they are FP64, which costs 35 us: all of them FP32 over a
-// pixel's 40 000 steps put dL/dN and dL/dscale off by 3e-6 to 1.3e-5 in place
-// of 1e-8 to 8e-7.
+// (cut_sums).  A unit's sums are FP32 (dL/dscale compensated), over the units
+// double-float in a column of shared memory, with dL/dI and over the pixels
+// FP64, which costs 35 us: all of them FP32 over a pixel's 40 000 steps put
+// dL/dN and dL/dscale off by 3e-6 to 1.3e-5 in place of 1e-8 to 8e-7.  (Folding
+// every unit into FP64: 4 x 128^2 pixels of 9 units of one step 100 us, not 63.)
 template <int HASF, int INTERP>
 __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
     spots_adjoint_kernel(AdjointArgs g) {
@@ -202,6 +220,12 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
   int q = 0, s = 0, f = 0;
   const int lane = threadIdx.x & 31;
   double mine = 0.0;  // lanes 2 r and 2 r + 1: the warp's sum r
+  // nearest lookup with several units: a pixel's sums over its units, as
+  // double-floats in shared memory (behind the tables)
+  constexpr bool kColumns = INTERP == 0;
+  const int n_units = a.os * a.os * a.T;
+  float2 (*s_tot)[kTileThreads] = reinterpret_cast<float2 (*)[kTileThreads]>(
+      s_rot + ((a.PM * 27 & 1) ? a.PM * 9 + 1 : a.PM * 9));
   {
     const bool ok = map_pixel(a, item, threadIdx.x, gp, q, s, f);
     const DevPanel &P = a.panels[ok ? q : 0];
@@ -217,7 +241,7 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
     for (int i = 0; i < os; ++i)
       for (int j = 0; j < os; ++j)
         for (int t = 0; t < a.T; ++t) {
-          double ws = 0.0;
+          float scal = 0.f;
           Kahan acc12;
           float acc[12];
 #pragma unroll
@@ -236,10 +260,9 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
                      df[2] * a.i0ff[2][0],
                 xe = df[0] * a.e0f[0] + df[1] * a.e0f[1] + df[2] * a.e0f[2],
                 ye = df[0] * a.b0f[0] + df[1] * a.b0f[1] + df[2] * a.b0f[2];
-          float scal = omega * cap * 0.5f *
-                       (1.f + c2 * c2 - kahn * (xe * xe - ye * ye));
-          ws = wk * (double)scal;
-          const float fscal = HASF ? (float)(ws * g.scale) : 0.f;
+          scal = omega * cap * 0.5f *
+                 (1.f + c2 * c2 - kahn * (xe * xe - ye * ye));
+          const float fscal = HASF ? (float)(wk * (double)scal * g.scale) : 0.f;
           for (int pm = 0; pm < a.PM; ++pm) {
             const float *Ah = s_axh + pm * 9, *Al = s_axl + pm * 9;
             float Gh[3], Gl[3], rq[3], rl[3], n0[3];
@@ -400,28 +423,44 @@ __global__ void __launch_bounds__(kTileThreads, INTERP ? 3 : 4)
                 acc[3 * x + c] = fmaf(E[x], vr[c], acc[3 * x + c]);
           }
           }
-          // the unit's sums, weighted, over the warp in FP64: of 16 a lane
-          // hands half to a lane 16 away, of the other 8 half to one 8 away,
-          // ...: 16 additions in place of 65, and nothing but one sum to keep
-          // from unit to unit
+          if (kColumns && n_units > 1) {
+            // into the thread's column of double-floats
+            const bool first = (i | j | t) == 0;
+#pragma unroll
+            for (int r = 0; r < kGradN; ++r) {
+              float p, e, lo, hi;
+              two_prod(scal, r < 12 ? acc[r] : acc12.s, p, e);
+              if (r == 12) e = fmaf(scal, -acc12.c, e);
+              float2 &col = s_tot[r][threadIdx.x];
+              const float2 old = first ? make_float2(0.f, 0.f) : col;
+              float s1, e1;
+              two_sum(old.x, p, s1, e1);
+              lo = old.y + (e1 + e);
+              fast_two_sum(s1, lo, hi, lo);
+              col = make_float2(hi, lo);
+            }
+            continue;
+          }
           double v[16];
 #pragma unroll
           for (int r = 0; r < 16; ++r)
-            v[r] = r < 12    ? ws * (double)acc[r]
-                   : r == 12 ? ws * acc12.value()
+            v[r] = r < 12    ? wk * (double)scal * (double)acc[r]
+                   : r == 12 ? wk * (double)scal * acc12.value()
                              : 0.0;
-#pragma unroll
-          for (int n = 8; n > 0; n >>= 1) {
-            const bool up = (lane & 2 * n) != 0;
-#pragma unroll
-            for (int r = 0; r < n; ++r) {
-              const double keep = up ? v[r + n] : v[r],
-                           give = up ? v[r] : v[r + n];
-              v[r] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * n);
-            }
-          }
-          mine += v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+          mine += warp_sums(v);
         }
+    if (kColumns && n_units > 1) {
+      double v[16];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        v[r] = 0.0;
+        if (r < kGradN && ok) {
+          const float2 c = s_tot[r][threadIdx.x];
+          v[r] = wk * ((double)c.x + (double)c.y);
+        }
+      }
+      mine = warp_sums(v);
+    }
   }
   if (INTERP && HASF) flush_node();
   if (HASF && near_idx >= 0) atomicAdd(g.gradF + nb_idx(a.check, NB_SITE_GRADF, near_idx, table_size(a)), (double)near_sum);
@@ -1082,6 +1121,10 @@ cudaError_t launch_adjoint(const SpotArgs &a, const float *rot,
   g.rows_next = nullptr;
   g.n_rows = 0;
   size_t smem = adjoint_smem_bytes(a, a.interp && gradF);
+  // the columns of the pixels' sums, and a float to align them (beside tables
+  // of at most 200 KB that are counted with 180 bytes per orientation too many)
+  if (a.interp == 0 && a.os * a.os * a.T > 1)
+    smem += sizeof(float) + kGradN * kTileThreads * sizeof(float2);
   long long blocks = adjoint_blocks(a);
   if (blocks <= 0) return cudaSuccess;
   void (*kern)(AdjointArgs);
