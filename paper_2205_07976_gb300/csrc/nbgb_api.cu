@@ -531,6 +531,7 @@ static void fill_args(const nb_sim *s, SpotArgs &a) {
   a.src64 = (const double *)s->tab(s->o_src64);
   a.src32 = (const float *)s->tab(s->o_src32);
   a.u0 = s->u0;
+  a.span = nbgb::source_span(s->lam.data(), s->n_src, s->u0);
   split_ff(s->u0, a.u0h, a.u0l);
   pol_basis(s->dirs.data(), s->evec, a.e0, a.b0);
   a.kahn = (float)s->kahn;

@@ -176,6 +176,8 @@ struct SpotArgs {
   // log2((Na Nb Nc)^2 U PM sum|w| 2^56), U = os^2 T
   const float *fmax;
   float screen_kb;
+  // (largest - smallest 1/lambda) / u0, for the choice of the warp kernel's form
+  float span;
   // NB_CHECK builds: the word a failed bounds check writes (null: none)
   unsigned long long *check;
 };
@@ -355,6 +357,10 @@ __device__ __forceinline__ void lagrange4(T x, T w[4]) {
 void sort_sources(std::vector<double> &dirs, std::vector<double> &lam,
                   std::vector<double> &w);
 double source_u0(const double *lam, int S);
+// (largest - smallest 1/lambda) / u0 of sorted sources
+inline float source_span(const double *lam, int S, double u0) {
+  return (float)((1.0 / lam[S - 1] - 1.0 / lam[0]) / u0);
+}
 void shot_tables_f32(const std::vector<double> &ax, const double *lam,
                      const double *w, const double *dirs, int S,
                      const double *evec, double u0, bool plain_f32,

@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kSplitThreads, FORM == kLines ? kLineBlocks
             pool[sp.img_off + p] = sp.prefactor * v;
         }
       };
-      if (FORM != kLines && split_form(base, b.PM, b.S) == kHalves)
+      if (FORM != kLines && half_form(base, b.PM, b.S))
         sum(std::integral_constant<int, kHalves>());
       else
         sum(std::integral_constant<int, FORM>());
@@ -756,7 +756,11 @@ int nb_server_submit(nb_server *s, const double axes[9], const double *umats,
       (long long)s->os * s->os * s->T * n_mosaic >= 8 &&
       s->os * s->os * s->T <= 32)
     r.kind =
-        nbgb::split_form(s->base, n_mosaic, n_src) == nbgb::kLines ? 2 : 1;
+        nbgb::split_form(s->base, n_mosaic, n_src,
+                         nbgb::source_span(lam.data(), n_src, u0)) ==
+                nbgb::kLines
+            ? 2
+            : 1;
   s->queue.push_back(r.id);
   *request_id = r.id;
   s->reqs.emplace(r.id, std::move(r));

@@ -87,7 +87,7 @@ using SplitKernel = void (*)(SpotArgs, unsigned long long *);
 template <int INTERP, int COUNT, bool FF>
 static SplitKernel pick_split(const SpotArgs &a) {
   if (a.has_div) return spots_split_kernel<INTERP, 1, COUNT, FF, kPairs>;
-  switch (split_form(a, a.PM, a.S)) {
+  switch (split_form(a, a.PM, a.S, a.span)) {
     case kLines: return spots_split_kernel<INTERP, 0, COUNT, FF, kLines>;
     case kHalves: return spots_split_kernel<INTERP, 0, COUNT, FF, kHalves>;
     // (the early test changes no sum and no count: not built with counters)

@@ -50,6 +50,7 @@ constexpr int kIntervalEntry = 1 << 31;
 // 11.8 ms on 1024^2 pixels of the large shot when it was chosen.
 constexpr int kLineSources = 32;
 constexpr int kLineSteps = 1200;
+constexpr float kLineMean = 15.f;
 constexpr int kTaskLen = 32;
 constexpr int kLineBlocks = 4;
 constexpr int SRC32_PAIR = 4;
@@ -1340,9 +1341,25 @@ constexpr int kLanes = FORM == kHalves ? 16 : 32;  // lanes per pixel
 // The share of h space within the cut of a lattice point; they are rare where
 // it is below kRareShare
 constexpr float kRareShare = 0.2f;
+constexpr float kEarlyLine = 0.2f;  // least share of the sources on a line
 __host__ __device__ inline float lattice_share(const SpotArgs &a) {
   const float m = sqrtf(kGaussCut * 0.63f) * 2.f;
   return m / a.N[0] * (m / a.N[1]) * (m / a.N[2]);
+}
+
+// The sources on a line through a lattice point, for S of them over a relative
+// range span of 1/lambda: the width of the cut over the movement of h, at the
+// outermost h of the table
+inline float line_sources(const SpotArgs &a, int S, float span) {
+  float nh = 0.f;
+  for (int x = 0; x < 3; ++x) {
+    const int lo = a.hmin[x], hi = a.hmin[x] + a.hn[x] - 1;
+    const float h = (float)(-lo > hi ? -lo : hi);
+    nh = fmaxf(nh, a.N[x] * h);
+  }
+  const float move = nh * span;
+  return move > 0.f ? fminf((float)S, 2.f * sqrtf(kGaussCut * 0.63f) / move * S)
+                    : (float)S;
 }
 
 // The form for a shot of PM orientations and S sources.  Lines need enough
@@ -1353,11 +1370,19 @@ __host__ __device__ inline float lattice_share(const SpotArgs &a) {
 // 0.873; large shot, 1024^2: 18.2 -> 10.2).  Where the ellipsoids of lattice points
 // overlap (N < 15.4) there are no interval entries, and the blocks of sources
 // are better summed by the pair kernels and their 20 warps per SM (300^2
-// pixels, N = 8, 10 items of 180 sources: 2.07 -> 1.68 ms).  The early test pays
+// pixels, N = 8, 10 items of 180 sources: 2.07 -> 1.68 ms).  A line of few
+// sources does not pay for its coefficients either: 400^2 pixels, pairs -> lines,
+// 40 sources, 30 domains, 9 units, spectrum FWHM 2 %, N = 60 (2.3 sources on a
+// line, line_sources) 0.80 -> 1.07 ms, N = 18 (7.6) 2.85 -> 3.63; 100, 25, 4, N =
+// 25 (13.8) 1.25 -> 1.35, but 24^2 pixels 77 -> 53 us; 180, 25, 1, N = 40 (15.5)
+// 325 -> 314 us, N = 25 (24.8) 594 -> 504.  The early test pays
 // where lattice points are rare: N = 25 (0.07 of h space lies within the cut)
 // 1.22 -> 1.05
 // ms on 1500^2 pixels with S = 11, M = 9, but at N = 15 (0.34) it finds one in
-// most batches, 1.86 -> 2.11 ms on the 64-panel shot.
+// most batches, 1.86 -> 2.11 ms on the 64-panel shot, and so it does where a
+// sweep passes several: 400^2 pixels, 100 sources, 25 domains, 4 units, FWHM 2 %
+// (0.11 of the sources on a line) 1.17 -> 1.25 ms; 0.5 %, N = 60 (0.23) 784 -> 747
+// us.
 // Halves pay where a pixel's items leave half the lanes idle (64-panel shot, 10
 // items of 8 sources, tricubic 1.83 -> 1.29 ms, nearest 1.47 -> 0.96; N = 25, 9
 // items of 11 0.337 -> 0.286).  A pixel alone then takes its pairs 16 at a time
@@ -1365,16 +1390,22 @@ __host__ __device__ inline float lattice_share(const SpotArgs &a) {
 // 1000 pixels, 100 steps at N = 15 (34 pairs expected) 36.4 -> 39.0 us, 480 steps
 // 45.7 -> 54.1, but 37.3 -> 37.7 with 99 steps at N = 25 (7 pairs); hence the
 // limits on steps and on expected pairs.
-__host__ __device__ inline int split_form(const SpotArgs &a, int PM, int S) {
-  if (a.has_div) return kPairs;
+__host__ __device__ inline bool half_form(const SpotArgs &a, int PM, int S) {
   const long long items = (long long)a.os * a.os * a.T * PM;
+  return !a.has_div && items <= kHalfItems && items * S <= kHalfSteps &&
+         (float)(items * S) * lattice_share(a) <= kHalfPairs;
+}
+inline int split_form(const SpotArgs &a, int PM, int S, float span) {
+  if (a.has_div) return kPairs;
   if ((a.interp == 0 || a.C4) && S >= kLineSources &&
-      items * S >= kLineSteps && lattice_disjoint(a))
+      (long long)a.os * a.os * a.T * PM * S >= kLineSteps &&
+      lattice_disjoint(a) && line_sources(a, S, span) >= kLineMean)
     return kLines;
-  if (items <= kHalfItems && items * S <= kHalfSteps &&
-      (float)(items * S) * lattice_share(a) <= kHalfPairs)
-    return kHalves;
-  return lattice_share(a) < kRareShare ? kPairsEarly : kPairs;
+  if (half_form(a, PM, S)) return kHalves;
+  return lattice_share(a) < kRareShare &&
+                 line_sources(a, S, span) >= kEarlyLine * S
+             ? kPairsEarly
+             : kPairs;
 }
 
 // The sum, without the prefactor, of the pixel whose U sub-pixel units are

@@ -54,7 +54,7 @@ struct TableArgs {
   float *axh, *axl, *src32;
   DevPanel *panel_out;
   unsigned long long *counters;
-  double *u0_out;  // u0 written here for the spots launch
+  double *u0_out;  // u0 and the range of 1/lambda, for the spots launch
 };
 
 // One block: u0 = centre of the 1/lambda range, then the double-float
@@ -101,7 +101,8 @@ __global__ void noalloc_tables_kernel(TableArgs t) {
     *t.panel_out = t.panel;
     t.counters[0] = 0;
     t.counters[1] = 0;
-    *t.u0_out = u0;
+    t.u0_out[0] = u0;
+    t.u0_out[1] = s_max[0] - s_min[0];
   }
 }
 
@@ -267,10 +268,12 @@ extern "C" int nb_add_spots_noalloc(
   if (e != cudaSuccess) return NB_ECUDA;
   // u0 (double-float) is a kernel argument of the spots kernel: read it
   // back into host stack memory (the table kernel computed it on device)
-  double u0 = 0.0;
-  e = cudaMemcpyAsync(&u0, u0_dev, sizeof u0, cudaMemcpyDeviceToHost, st);
+  double ur[2] = {0.0, 0.0};
+  e = cudaMemcpyAsync(ur, u0_dev, sizeof ur, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return NB_ECUDA;
+  const double u0 = ur[0];
+  a.span = (float)(ur[1] / u0);
   a.u0 = u0;
   a.u0h = (float)u0;
   a.u0l = (float)(u0 - (double)a.u0h);
