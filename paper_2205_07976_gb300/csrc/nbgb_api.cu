@@ -132,7 +132,7 @@ struct nb_sim {
   // the background's tables (background_tables): whether they are out of date,
   // and what a launch needs of them
   bool bg_dirty = true;
-  int bg_groups = 0, bg_nodes = 0, bg_form = 0;
+  int bg_groups = 0, bg_nodes = 0;
   double bg_nmol = 0;
   DevBuf d_bg64, d_bg32, d_bgrng;
 };
@@ -1353,8 +1353,8 @@ static int background_tables(nb_sim *s) {
     }
   };
   std::vector<double> nodes;
-  int cnt_max = 0;               // of the groups with nodes: the most sources,
-  double span_per_source = 0.0;  // the largest relative range of u per source
+  int cnt_max = 0;     // of the groups with nodes: the most sources,
+  double range = 0.0;  // the largest relative range of u per source
   for (int g = 0; g < G; ++g) {
     const int first = rng[4 * g], cnt = rng[4 * g + 1];
     bool ok = true;
@@ -1371,9 +1371,8 @@ static int background_tables(nb_sim *s) {
     if (!ok) continue;
     rng[4 * g + 2] = (int)nodes.size() / 4;
     cnt_max = std::max(cnt_max, cnt);
-    span_per_source = std::max(
-        span_per_source,
-        2.0 * span / ((leaf[0].ubar + leaf[cnt - 1].ubar) * cnt));
+    range = std::max(
+        range, 2.0 * span / ((leaf[0].ubar + leaf[cnt - 1].ubar) * cnt));
     std::vector<Node> t(4 * (size_t)cnt);
     t[cnt - 1] = leaf[cnt - 1];
     for (int i = cnt - 2; i >= 0; --i) {  // suffixes
@@ -1410,15 +1409,14 @@ static int background_tables(nb_sim *s) {
                 "background tables exceed 200 KB of shared memory");
   // with many sources and knots the nodes may not fit as well: every source
   // is then visited
-  // (nor are they of use where every group is one source)
+  // (nor are they of use where every group is one source, or knots are dense)
   b.n_nodes = (int)nodes.size() / 4;
-  if (cnt_max < 2 || nbgb::background_smem_bytes(b, f64) > 200 * 1024) {
+  if (cnt_max < 2 || !nbgb::bg_use_nodes(f64, range, n) ||
+      nbgb::background_smem_bytes(b, f64) > 200 * 1024) {
     b.n_nodes = 0;
-    cnt_max = 0;
     nodes.clear();
     for (int g = 0; g < G; ++g) rng[4 * g + 2] = -1;
   }
-  b.form = nbgb::bg_form(f64, cnt_max, span_per_source, n);
   // one double blob: groups, then (F64) knots and sources; one float blob
   std::vector<double> b64(grp);
   std::vector<float> b32;
@@ -1464,7 +1462,6 @@ static int background_tables(nb_sim *s) {
     return cuda_fail(s, e, "background tables");
   s->bg_groups = G;
   s->bg_nodes = b.n_nodes;
-  s->bg_form = b.form;
   s->bg_dirty = false;
   return NB_OK;
 }
@@ -1487,7 +1484,6 @@ int nb_add_background(nb_sim *s) {
   b.n_knots = n;
   b.n_groups = G;
   b.n_nodes = s->bg_nodes;
-  b.form = s->bg_form;
   SpotArgs &a = b.geo;
   a.check = (unsigned long long *)s->d_check.p;  // NB_CHECK builds only
   a.panels = (const DevPanel *)s->d_panels.p;

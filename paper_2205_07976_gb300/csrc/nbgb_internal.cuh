@@ -424,10 +424,9 @@ struct BgArgs {
   const double *src64;    // [S][2] 1/lambda, w (grouped order)
   const float *src32;     // [S][2]
   double prefactor;       // r_e^2 fluence n_mol / os^2
-  int form;               // bg_form
 };
 constexpr int kMaxKnots = 4096;
-int bg_form(bool f64, int cnt, double span_per_source, int n);
+bool bg_use_nodes(bool f64, double range, int n);
 size_t background_smem_bytes(const BgArgs &b, bool f64);
 cudaError_t launch_background(const BgArgs &b, bool f64, int sm_count,
                               cudaStream_t st);
