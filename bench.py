@@ -53,13 +53,13 @@ MAX_SM_MHZ = 2070.0  # GB300's maximum SM clock
 # kernel, from one ncu capture (profiles/spots_split_large_shot_dram.txt:
 # the mean of two launches);
 # valid only while the kernel sources hash to the value they had then
-TRAFFIC_CAPTURE = {"bytes": (79876864 + 21332992 + 80176640 + 21391616) // 2,
+TRAFFIC_CAPTURE = {"bytes": (80124672 + 20957696 + 79852800 + 21054720) // 2,
                    "sources": ["paper_2205_07976_gb300/csrc/spots_split.cu",
                                "paper_2205_07976_gb300/csrc/split_kernel.cuh",
                                "paper_2205_07976_gb300/csrc/split_pixel.cuh",
                                "paper_2205_07976_gb300/csrc/mixed_common.cuh",
                                "paper_2205_07976_gb300/csrc/nbgb_internal.cuh"],
-                   "sha256_16": "acd951c08ae206ab"}
+                   "sha256_16": "67008d56c11af7b2"}
 
 
 def captured_traffic():
@@ -76,14 +76,14 @@ def captured_traffic():
 # Pipe utilisation (% of active cycles) of the warp-per-pixel kernel from
 # one ncu --set full capture on a 512x512 window of the large shot
 # (profiles/spots_split_window512_full.txt), keyed like the traffic figure
-PIPES_CAPTURE = {"sm__pipe_fma_cycles_active_pct": 28.7,
-                 "sm__pipe_alu_cycles_active_pct": 33.1,
-                 "sm__inst_executed_pipe_lsu_pct": 12.1,
-                 "sm__pipe_fp64_cycles_active_pct": 37.1,
-                 "smsp__issue_active_pct": 52.7,
-                 "l1tex__data_pipe_lsu_wavefronts_pct": 39.0,
+PIPES_CAPTURE = {"sm__pipe_fma_cycles_active_pct": 28.6,
+                 "sm__pipe_alu_cycles_active_pct": 32.6,
+                 "sm__inst_executed_pipe_lsu_pct": 11.6,
+                 "sm__pipe_fp64_cycles_active_pct": 35.5,
+                 "smsp__issue_active_pct": 51.6,
+                 "l1tex__data_pipe_lsu_wavefronts_pct": 37.2,
                  "window": "512x512 centred on the large shot",
-                 "sha256_16": "acd951c08ae206ab"}
+                 "sha256_16": "67008d56c11af7b2"}
 
 
 def captured_pipes():

@@ -737,8 +737,9 @@ __device__ __forceinline__ unsigned sum_pairs(
 // polynomial on a line: a polynomial of degree 9 in t.  A lane that takes such
 // a segment makes its ten coefficients once (cell_line: ~180 FMAs, packed where
 // two powers of x go side by side) and then spends ~15 instructions on a step,
-// two of them shared loads for a pair of steps, where the pair queue spends ~250 per 32 steps on
-// finding entry, source and cell and on 63 FMAs and 16 shared loads per step.
+// two of them shared loads for a pair of steps, where the pair queue spends ~250
+// per 32 steps on finding entry, source and cell and on 63 FMAs and 16 shared
+// loads per step.
 
 // Coefficients q of F(x0 + g tau), a cell's polynomial (SpotArgs::C4 at cp) on
 // a line: shifted and scaled per power of z, then Horner in y and x with
@@ -1362,34 +1363,33 @@ inline float line_sources(const SpotArgs &a, int S, float span) {
                     : (float)S;
 }
 
-// The form for a shot of PM orientations and S sources.  Lines need enough
-// tasks per pixel to fill a pass, and enough steps per line to pay for its
+// The form for a shot of PM orientations and S sources. Lines need enough tasks
+// per pixel to fill a pass, and enough steps per line to pay for its
 // coefficients (pairs with the early test -> lines, 700^2 pixels: 1 unit, S =
 // 100, M = 12 0.605 -> 0.541 ms; S = 60, M = 30 0.750 -> 0.621; S = 30, M = 50
-// 0.820 -> 0.816; S = 20, M = 50 0.696 -> 0.777; S = 60, M = 12, 1000^2 0.787 ->
-// 0.873; large shot, 1024^2: 18.2 -> 10.2).  Where the ellipsoids of lattice points
-// overlap (N < 15.4) there are no interval entries, and the blocks of sources
-// are better summed by the pair kernels and their 20 warps per SM (300^2
-// pixels, N = 8, 10 items of 180 sources: 2.07 -> 1.68 ms).  A line of few
-// sources does not pay for its coefficients either: 400^2 pixels, pairs -> lines,
-// 40 sources, 30 domains, 9 units, spectrum FWHM 2 %, N = 60 (2.3 sources on a
-// line, line_sources) 0.80 -> 1.07 ms, N = 18 (7.6) 2.85 -> 3.63; 100, 25, 4, N =
-// 25 (13.8) 1.25 -> 1.35, but 24^2 pixels 77 -> 53 us; 180, 25, 1, N = 40 (15.5)
-// 325 -> 314 us, N = 25 (24.8) 594 -> 504.  The early test pays
-// where lattice points are rare: N = 25 (0.07 of h space lies within the cut)
-// 1.22 -> 1.05
-// ms on 1500^2 pixels with S = 11, M = 9, but at N = 15 (0.34) it finds one in
-// most batches, 1.86 -> 2.11 ms on the 64-panel shot, and so it does where a
-// sweep passes several: 400^2 pixels, 100 sources, 25 domains, 4 units, FWHM 2 %
-// (0.11 of the sources on a line) 1.17 -> 1.25 ms; 0.5 %, N = 60 (0.23) 784 -> 747
-// us.
+// 0.820 -> 0.816; S = 20, M = 50 0.696 -> 0.777; S = 60, M = 12, 1000^2 0.787
+// -> 0.873; large shot, 1024^2: 18.2 -> 10.2). Where the ellipsoids of lattice
+// points overlap (N < 15.4) there are no interval entries, and the blocks of
+// sources are better summed by the pair kernels and their 20 warps per SM
+// (300^2 pixels, N = 8, 10 items of 180 sources: 2.07 -> 1.68 ms). A line of
+// few sources does not pay for its coefficients either: 400^2 pixels, pairs ->
+// lines, 40 sources, 30 domains, 9 units, spectrum FWHM 2 %, N = 60 (2.3
+// sources on a line, line_sources) 0.80 -> 1.07 ms, N = 18 (7.6) 2.85 -> 3.63;
+// 100, 25, 4, N = 25 (13.8) 1.25 -> 1.35, but 24^2 pixels 77 -> 53 us; 180, 25,
+// 1, N = 40 (15.5) 325 -> 314 us, N = 25 (24.8) 594 -> 504.
+// The early test pays where lattice points are rare: N = 25 (0.07 of h space
+// lies within the cut) 1.22 -> 1.05 ms on 1500^2 pixels with S = 11, M = 9, but
+// at N = 15 (0.34) it finds one in most batches, 1.86 -> 2.11 ms on the
+// 64-panel shot, and so it does where a sweep passes several: 400^2 pixels, 100
+// sources, 25 domains, 4 units, FWHM 2 % (0.11 of the sources on a line) 1.17
+// -> 1.25 ms; 0.5 %, N = 60 (0.23) 784 -> 747 us.
 // Halves pay where a pixel's items leave half the lanes idle (64-panel shot, 10
 // items of 8 sources, tricubic 1.83 -> 1.29 ms, nearest 1.47 -> 0.96; N = 25, 9
-// items of 11 0.337 -> 0.286).  A pixel alone then takes its pairs 16 at a time
+// items of 11 0.337 -> 0.286). A pixel alone then takes its pairs 16 at a time
 // with the other half idle, so a list of few pixels waits for the longer chain:
-// 1000 pixels, 100 steps at N = 15 (34 pairs expected) 36.4 -> 39.0 us, 480 steps
-// 45.7 -> 54.1, but 37.3 -> 37.7 with 99 steps at N = 25 (7 pairs); hence the
-// limits on steps and on expected pairs.
+// 1000 pixels, 100 steps at N = 15 (34 pairs expected) 36.4 -> 39.0 us, 480
+// steps 45.7 -> 54.1, but 37.3 -> 37.7 with 99 steps at N = 25 (7 pairs); hence
+// the limits on steps and on expected pairs.
 __host__ __device__ inline bool half_form(const SpotArgs &a, int PM, int S) {
   const long long items = (long long)a.os * a.os * a.T * PM;
   return !a.has_div && items <= kHalfItems && items * S <= kHalfSteps &&

@@ -11,7 +11,8 @@
 //      than 256 pixels in all); its lanes set up the
 //      U = os^2 x layers sub-pixel units of all B pixels (position,
 //      direction, solid angle, capture, polarization; in FP64, for one or two
-//      units per pixel in double-float) into shared memory, then the warp sums the pixels one after another;
+//      units per pixel in double-float) into shared memory, then the warp
+//      sums the pixels one after another;
 //   2. lanes take (unit, phi x mosaic) items 32 at a time and form G and r
 //      in double-float.  h_x = G_x delta + r_x is linear in a source's
 //      delta = 1/lambda - u0, so for each lattice point near the item's
@@ -30,8 +31,8 @@
 //      segment of an entry instead, on which F_cell is a polynomial of degree
 //      9 in delta and the exponent a parabola: ~15 instructions per step in
 //      place of ~8 per lane and step of the pair queue (sum_tasks).  Large
-//      shot: 164.5 -> 101.8 ms; the 512^2 pixels at its centre, where the
-//      batches of items without a lattice point in reach end early, 5.0 -> 2.6;
+//      shot: 164.5 -> 107.1 ms; the 512^2 pixels at its centre, where the
+//      batches of items without a lattice point in reach end early, 5.0 -> 2.7;
 //      In shots of few items and steps per pixel (split_form) each half of the
 //      warp takes a pixel of its own: with 10 items a pixel's pass over its
 //      items left 22 lanes idle;
